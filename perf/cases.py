@@ -196,10 +196,22 @@ def _solver(flows, case):
     return Solver(cavs, **opts)
 
 
-def _fill(s, flows, seed):
+def _fill(s, flows, seed, precision):
     for k, f in enumerate(flows):
         g, lam = _state(f, seed, k)
         s.set_state(k, (g + _vec(W, g)).cpu().numpy(), lam.cpu().numpy())
+    # a checkpoint holds the rows' padding too: start from one that has zeros there
+    buf, at = _state_tensor(s, precision), 9 * _planes(flows)
+    torch.cuda.synchronize()
+    capi.ifdlbm_save_state_dev(s.h, buf)
+    torch.cuda.synchronize()
+    for f in flows:
+        pitch = (f["nx"] + 31) // 32 * 32
+        buf[at:at + f["ny"] * pitch].view(f["ny"], pitch)[:, f["nx"]:] = 0.0
+        at += f["ny"] * pitch
+    torch.cuda.synchronize()
+    capi.ifdlbm_load_state_dev(s.h, buf)
+    torch.cuda.synchronize()
 
 
 def _state_tensor(s, precision):
@@ -226,7 +238,7 @@ def prepare(case, seed):
     if kind == "adjoint":
         flows[0]["grid_dt"] = True
     s = _solver(flows, case)
-    _fill(s, flows, seed)
+    _fill(s, flows, seed, case["precision"])
     st = {"kind": kind, "solver": s, "planes": _planes(flows)}
     if kind == "step":
         st["steps"], st["precision"] = case["steps"], case["precision"]
