@@ -896,7 +896,8 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
     }
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->b.lam[1], 0, off * tsize, s);
+  for (int p = 0; p < 2; ++p)
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->b.lam[p], 0, off * tsize, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->b.resid, 0, size_t(ncav) * 4 * sizeof(double), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->b.status, 0, sizeof(unsigned), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->b.pref, 0, size_t(ncav) * sizeof(double), s);
