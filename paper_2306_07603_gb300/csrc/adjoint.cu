@@ -521,7 +521,7 @@ __global__ void k_adj_reduce(const CavDev *cavs, const double *ppart, double *dp
   const CavDev &cv = cavs[blockIdx.x];
   __shared__ double sh[128][3];
   double acc[3] = {0, 0, 0};
-  for (int t = threadIdx.x; t < cv.nparts; t += blockDim.x)
+  for (int t = threadIdx.x; t < cv.tiles_x * cv.tiles_y; t += blockDim.x)
     for (int s = 0; s < 4; ++s)
 #pragma unroll
       for (int k = 0; k < 3; ++k) acc[k] += ppart[int64_t(cv.tile0 + t) * 12 + s * 3 + k];

@@ -47,6 +47,8 @@ struct ifdlbm_ctx {
   std::vector<double> courant;
   ifd::Bufs b{};
   int ntiles = 0;
+  int nblk64 = 0;      // FP64 staged kernels: blocks per launch
+  int nt64 = 128;      // ... and threads per block
   int ntasks = 0;      // fused kernel tasks
   int fused_nt = 128;  // fused kernel threads per CTA
   int fused_rows = 0;  // rows per task (0: automatic)
@@ -216,6 +218,7 @@ void enqueue_step(ifdlbm_ctx *h, int parity, bool want_residual) {
   a.cav = h->b.cav;
   a.geo = h->b.geo;
   a.tile_cav = h->b.tile_cav;
+  a.blk_cav = h->b.blk_cav;
   a.g_in = h->b.g[parity];
   a.g_out = h->b.g[parity ^ 1];
   a.lam_in = h->b.lam[parity];
@@ -230,9 +233,15 @@ void enqueue_step(ifdlbm_ctx *h, int parity, bool want_residual) {
   a.powt = h->b.powt;
   a.pref = h->b.pref;
   a.want_residual = want_residual ? 1 : 0;
-  timed(h, IFDLBM_KPROF_COLLIDE, [&] { ifd::launch_collide<T>(a, h->ntiles, h->stream); });
-  timed(h, IFDLBM_KPROF_HALF, [&] { ifd::launch_half<T>(a, h->ntiles, h->stream); });
-  timed(h, IFDLBM_KPROF_FULL, [&] { ifd::launch_full<T>(a, h->ntiles, h->stream); });
+  if constexpr (sizeof(T) == 8) {
+    timed(h, IFDLBM_KPROF_COLLIDE, [&] { ifd::launch_collide64(a, h->nblk64, h->nt64, h->stream); });
+    timed(h, IFDLBM_KPROF_HALF, [&] { ifd::launch_half64(a, h->nblk64, h->nt64, h->stream); });
+    timed(h, IFDLBM_KPROF_FULL, [&] { ifd::launch_full64(a, h->nblk64, h->nt64, h->stream); });
+  } else {
+    timed(h, IFDLBM_KPROF_COLLIDE, [&] { ifd::launch_collide(a, h->ntiles, h->stream); });
+    timed(h, IFDLBM_KPROF_HALF, [&] { ifd::launch_half(a, h->ntiles, h->stream); });
+    timed(h, IFDLBM_KPROF_FULL, [&] { ifd::launch_full(a, h->ntiles, h->stream); });
+  }
   if (want_residual)
     timed(h, IFDLBM_KPROF_REDUCE, [&] {
       ifd::launch_residual_reduce(h->b.cav, h->b.part, h->b.resid, h->ncav, h->stream);
@@ -475,6 +484,10 @@ int ifdlbm_default_options(ifdlbm_options *opt) {
 
 namespace {
 
+// Batches of up to this many nodes run the FP64 staged kernels in blocks of one
+// warp, which spread over all SMs, larger ones in blocks of four.
+constexpr int64_t SMALL_NODES64 = 100000;
+
 int validate_quad(ifdlbm_ctx *h, int idx, const ifdlbm_quad_cavity &q) {
   char buf[256];
   auto bad = [&](const char *what) {
@@ -669,6 +682,19 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
     cv.deta = 1.0 / (s.ny - 1);
     cv.inv2dxi = 1.0 / (2.0 * cv.dxi);
     cv.inv2deta = 1.0 / (2.0 * cv.deta);
+    {  // constants of the FP64 staged kernels
+      const double e = opt.eta_b, o = 1.0 - opt.eta_b;
+      cv.mix = ifd::Mix64{e, -(e + 4.0 * o), 3.0 * o, o, -(e + 2.0 * o), 2.0 * o};
+      for (int st = 0; st < 2; ++st) {
+        const double scale = st == 0 ? 0.5 * cv.dt : cv.dt;
+        cv.sxi[st] = scale * opt.c * cv.inv2dxi;
+        cv.seta[st] = scale * opt.c * cv.inv2deta;
+        const double E = -cv.seta[st] / H;
+        cv.mixe[st] = ifd::Mix64{E * cv.mix.ka, E * cv.mix.kb, E * cv.mix.k0,
+                                 E * cv.mix.kf, E * cv.mix.wb, E * cv.mix.w0};
+      }
+      cv.strain2 = 2.0 * std::pow(opt.c, 4) / (cv.cs2 * cv.cs2);
+    }
     cv.U = s.U_lid;
     cv.H = H;
     cv.rho0 = opt.rho0;
@@ -735,6 +761,26 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
   h->ntiles = tile0;
   h->total_plane = off;
   h->geo_len = goff;
+  const bool staged64 = !fused && opt.precision == IFDLBM_FP64;
+  std::vector<int> blk_cav;
+  if (staged64) {
+    // Blocks of the FP64 staged kernels (node_of, step64.cuh): interior nodes,
+    // then wall nodes of every cavity.
+    int64_t nodes = 0;
+    for (const CavDev &cv : h->cav) nodes += int64_t(cv.nx) * cv.ny;
+    h->nt64 = nodes <= SMALL_NODES64 ? 32 : 128;
+    for (int k = 0; k < ncav; ++k) {
+      CavDev &cv = h->cav[k];
+      auto blocks = [&](int64_t n) { return int((n + h->nt64 - 1) / h->nt64); };
+      cv.blk0 = int(blk_cav.size());
+      cv.nblk_in = blocks(int64_t(cv.nx - 2) * (cv.ny - 2));
+      cv.nblk = cv.nblk_in + blocks(2 * int64_t(cv.nx) + 2 * (cv.ny - 2));
+      blk_cav.resize(blk_cav.size() + cv.nblk, k);
+      cv.part0 = cv.blk0;
+      cv.nparts = cv.nblk;
+    }
+    h->nblk64 = int(blk_cav.size());
+  }
   if (fused) {  // task capacity: the finest layout the autotuner tries (64 threads, 16 rows)
     int cap = 0;
     const int rmin = opt.fused_rows ? std::min(opt.fused_rows, 16) : 16;
@@ -761,13 +807,14 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
     ok &= (h->counter = (int *)A(sizeof(int))) != nullptr;
     ok &= (h->tmaps = (unsigned char *)A(size_t(2) * ncav * ifd::TMAP_BYTES)) != nullptr;
   }
-  const int nslots = fused ? h->task_cap : h->ntiles;
+  const int nslots = fused ? h->task_cap : (staged64 ? h->nblk64 : h->ntiles);
+  if (staged64) ok &= (h->b.blk_cav = (int *)A(blk_cav.size() * sizeof(int))) != nullptr;
   ok &= (h->b.part = (double *)A(size_t(nslots) * ifd::NPART * sizeof(double))) != nullptr;
   ok &= (h->b.resid = (double *)A(size_t(ncav) * 4 * sizeof(double))) != nullptr;
   ok &= (h->b.tile_cav = (int *)A(size_t(h->ntiles) * sizeof(int))) != nullptr;
   ok &= (h->b.status = (unsigned *)A(sizeof(unsigned))) != nullptr;
   ok &= (h->b.cav = (CavDev *)A(size_t(ncav) * sizeof(CavDev))) != nullptr;
-  double *geo = (double *)A(size_t(4 * goff) * sizeof(double));
+  double *geo = (double *)A(size_t(6 * goff) * sizeof(double));
   ok &= geo != nullptr;
   float *geof = (float *)A(size_t(2 * goff) * sizeof(float));
   ok &= geof != nullptr;
@@ -792,6 +839,8 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
   h->b.geo.xeH = geo + goff;
   h->b.geo.xxi = geo + 2 * goff;
   h->b.geo.xeta = geo + 3 * goff;
+  h->b.geo.ax[0] = geo + 4 * goff;
+  h->b.geo.ax[1] = geo + 5 * goff;
   h->b.geo.cxix_f = geof;
   h->b.geo.jac_f = geof + goff;
   h->b.geo.gmet = gmet;
@@ -808,20 +857,27 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
   std::vector<int> tile_cav(h->ntiles);
   for (int k = 0; k < ncav; ++k)
     for (int t = 0; t < h->cav[k].tiles_x * h->cav[k].tiles_y; ++t) tile_cav[h->cav[k].tile0 + t] = k;
-  std::vector<double> geo_h(4 * goff);
+  std::vector<double> geo_h(6 * goff);
   std::copy(xix.begin(), xix.end(), geo_h.begin());
   std::copy(xeH.begin(), xeH.end(), geo_h.begin() + goff);
   std::copy(xxi.begin(), xxi.end(), geo_h.begin() + 2 * goff);
   std::copy(xeta.begin(), xeta.end(), geo_h.begin() + 3 * goff);
+  for (int st = 0; st < 2; ++st)
+    for (const CavDev &cv : h->cav)
+      for (int j = 0; j < cv.ny; ++j)
+        geo_h[(4 + st) * goff + cv.goff + j] = cv.sxi[st] * xix[cv.goff + j];
 
   cudaStream_t s = h->stream;
-  h->h2d_bytes = int64_t(tile_cav.size() * sizeof(int) + h->cav.size() * sizeof(CavDev) +
+  h->h2d_bytes = int64_t((tile_cav.size() + blk_cav.size()) * sizeof(int) + h->cav.size() * sizeof(CavDev) +
                          geo_h.size() * sizeof(double) + geof_h.size() * sizeof(float) +
                          ifd::POW_TABLE_SIZE * sizeof(double) +
                          size_t(ncav) * ifd::POWT_SIZE * sizeof(double) +
                          (quads ? size_t(8 * ncav) * sizeof(double) : 0));
   e = cudaMemcpyAsync(h->b.tile_cav, tile_cav.data(), tile_cav.size() * sizeof(int),
                       cudaMemcpyHostToDevice, s);
+  if (staged64 && e == cudaSuccess)
+    e = cudaMemcpyAsync(h->b.blk_cav, blk_cav.data(), blk_cav.size() * sizeof(int),
+                        cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->b.cav, h->cav.data(), h->cav.size() * sizeof(CavDev),
                         cudaMemcpyHostToDevice, s);
@@ -1368,6 +1424,7 @@ int ifdlbm_adjoint_step(ifdlbm_handle h, const void *state_n, void *adj, double 
   f.cav = h->b.cav;
   f.geo = h->b.geo;
   f.tile_cav = h->b.tile_cav;
+  f.blk_cav = h->b.blk_cav;
   f.g_in = state_n;
   f.lam_in = (const double *)state_n + 9 * h->total_plane;
   f.g_out = h->adj_g1;
@@ -1379,11 +1436,12 @@ int ifdlbm_adjoint_step(ifdlbm_handle h, const void *state_n, void *adj, double 
   f.part = h->b.part;
   f.status = h->b.status;
   f.powtab = h->b.powtab;
+  f.powt = h->b.powt;
   f.pref = h->b.pref;
   f.want_residual = 0;
-  ifd::launch_collide<double>(f, h->ntiles, h->stream);
-  ifd::launch_half<double>(f, h->ntiles, h->stream);
-  ifd::launch_full<double>(f, h->ntiles, h->stream);
+  ifd::launch_collide64(f, h->nblk64, h->nt64, h->stream);
+  ifd::launch_half64(f, h->nblk64, h->nt64, h->stream);
+  ifd::launch_full64(f, h->nblk64, h->nt64, h->stream);
   ifd::launch_adjoint_step(adj_args(h, state_n, adj), h->ntiles, h->ncav, dparams, h->stream);
   g_launches += 3 + 9;
   cudaError_t e = cudaGetLastError();

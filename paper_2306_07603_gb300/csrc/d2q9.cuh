@@ -170,43 +170,34 @@ static __device__ __noinline__ float lambda_implicit_f32(float a, float lam_star
   return lam;
 }
 
-// Relaxation time of Step (2): strain rate from f^ne (Eqs. 2.12-2.13, with
-// f = f(f-hat, lam_prev) of Eq. 2.18), q = |gamma-dot|^2 = 2 D:D, the
-// clamped power law mu = K max(|gamma-dot|, gamma_min)^(n-1) evaluated as
-// K max(q, gamma_min^2)^((n-1)/2) (Eq. 1.4), and lam = mu / c_s^2 (Eq. 2.14).
-// Pxx, Pxy, Pyy are sum_i c_ia c_ib (g_i - geq_i). The strain rate is formed
-// in T (the storage precision); the power law of Eq. (1.4) and the implicit
-// form's solve are FP64, as the FP32-deviation form specifies: pow_fast for
-// an FP64 strain rate, pow_tab (FP64 result, error within 6e-16) for the FP32
-// one, clamped at cv.gmin2_f. With cv.pow32 (FP32 storage only, an opt-in)
-// they are FP32 instead (pow_f32, lambda_implicit_f32; the clamp at the
-// largest float not above gamma_min^2). powt: the cavity's pow_tab table.
-template <class T>
-__device__ __forceinline__ double relaxation_time(T Pxx, T Pxy, T Pyy, double lam_prev,
-                                                  const CavDev &cv, const double *powtab,
-                                                  const double *powt) {
+// Relaxation time of Step (2) of the FP32 staged kernels: strain rate from f^ne
+// (Eqs. 2.12-2.13, with f = f(f-hat, lam_prev) of Eq. 2.18), q = |gamma-dot|^2 =
+// 2 D:D, the clamped power law mu = K max(|gamma-dot|, gamma_min)^(n-1)
+// evaluated as K max(q, gamma_min^2)^((n-1)/2) (Eq. 1.4), and lam = mu / c_s^2
+// (Eq. 2.14). Pxx, Pxy, Pyy are sum_i c_ia c_ib (g_i - geq_i). The strain rate
+// is formed in FP32, clamped at cv.gmin2_f; the power law of Eq. (1.4)
+// (pow_tab, FP64 result, error within 6e-16) and the implicit form's solve are
+// FP64, as the FP32-deviation form specifies. With cv.pow32 (an opt-in) they
+// are FP32 instead (pow_f32, lambda_implicit_f32; the clamp at the largest
+// float not above gamma_min^2). powt: the cavity's pow_tab table.
+__device__ __forceinline__ double relaxation_time(float Pxx, float Pxy, float Pyy,
+                                                  float lam_prev, const CavDev &cv,
+                                                  const double *powtab, const double *powt) {
   if (cv.implicit) {
-    const T G2 = T(0.5) * (Pxx * Pxx + T(2) * Pxy * Pxy + Pyy * Pyy);
-    if constexpr (sizeof(T) == 4)
-      if (cv.pow32)
-        return double(lambda_implicit_f32(2.0f * sqrtf(G2) * float(cv.inv_cs2), float(lam_prev), cv));
-    return lambda_implicit(2.0 * sqrt(double(G2)) * cv.inv_cs2, lam_prev, cv, powtab);
+    const float G2 = 0.5f * (Pxx * Pxx + 2.0f * Pxy * Pxy + Pyy * Pyy);
+    if (cv.pow32)
+      return double(lambda_implicit_f32(2.0f * sqrtf(G2) * float(cv.inv_cs2), lam_prev, cv));
+    return lambda_implicit(2.0 * sqrt(double(G2)) * cv.inv_cs2, double(lam_prev), cv, powtab);
   }
   // f^ne = 2 lam_prev/(2 lam_prev + dt) (f-hat - f^eq);  S = -sum c c f^ne / (lam_prev c_s^2)
-  const T k = T(-2) / ((T(2) * T(lam_prev) + T(cv.dt)) * T(cv.cs2));
-  const T Sxx = k * Pxx, Sxy = k * Pxy, Syy = k * Pyy;
-  if constexpr (sizeof(T) == 4) {
-    if (cv.pow32) {
-      const float q = fmaxf(0.5f * (Sxx * Sxx + 2.0f * Sxy * Sxy + Syy * Syy),
-                            __double2float_rd(cv.gmin2));
-      return double(float(cv.Kics2) * pow_f32(q, float(cv.half_nm1)));
-    }
-    const float q = fmaxf(0.5f * (Sxx * Sxx + 2.0f * Sxy * Sxy + Syy * Syy), cv.gmin2_f);
-    return pow_tab(q, powt, cv.half_nm1, cv.pb2, cv.pb3, cv.pb4, cv.pb5);
+  const float k = -2.0f / ((2.0f * lam_prev + float(cv.dt)) * float(cv.cs2));
+  const float Sxx = k * Pxx, Sxy = k * Pxy, Syy = k * Pyy;
+  const float q2 = 0.5f * (Sxx * Sxx + 2.0f * Sxy * Sxy + Syy * Syy);
+  if (cv.pow32) {
+    const float q = fmaxf(q2, __double2float_rd(cv.gmin2));
+    return double(float(cv.Kics2) * pow_f32(q, float(cv.half_nm1)));
   }
-  double q = double(T(0.5) * (Sxx * Sxx + T(2) * Sxy * Sxy + Syy * Syy));
-  q = q > cv.gmin2 ? q : cv.gmin2;
-  return cv.Kics2 * pow_fast(q, cv.half_nm1, powtab);
+  return pow_tab(fmaxf(q2, cv.gmin2_f), powt, cv.half_nm1, cv.pb2, cv.pb3, cv.pb4, cv.pb5);
 }
 
 // Second moments of the non-equilibrium deviation d_i = g_i - geq_i.

@@ -7,6 +7,15 @@
 
 namespace ifd {
 
+// Mixed difference of Eqs. (2.5)-(2.7) along one axis, times 2 d and signed so
+// that |c| times it is c D F: with a, b, f the neighbours downwind, upwind and
+// twice upwind of the node, ka a + kb b + k0 F[node] + kf f, the coefficients
+// that eta_b and 1 - eta_b combine to; next to the wall on the upwind side the
+// first-order form ka a + wb b + w0 F[node]. FP64 staged kernels.
+struct Mix64 {
+  double ka, kb, k0, kf, wb, w0;
+};
+
 // Per-cavity constants, resident in device global memory (one entry per
 // cavity of a handle). Offsets are in elements of the arena they index.
 struct CavDev {
@@ -40,6 +49,14 @@ struct CavDev {
   // the clamp of the FP32 strain rate, max(largest float <= gamma_min^2, FLT_MIN)
   double pb2;
   float pb3, pb4, pb5, gmin2_f;
+  // FP64 staged kernels (staged64.cu): thread blocks of this cavity and, for the
+  // half step [0] and the full step [1] (scale dt/2 and dt), the coefficients
+  // of the mixed difference (xi, unscaled; eta of the trapezoid, times -scale
+  // c / (2 deta H)) and scale c / (2 dxi), scale c / (2 deta)
+  int blk0, nblk_in, nblk;
+  Mix64 mix, mixe[2];
+  double sxi[2], seta[2];
+  double strain2;           // 2 c^4 / c_s^4: |gamma-dot|^2 = strain2 pp / (2 lam_prev + dt)^2
 };
 
 // 1-D metric arrays of the trapezoid map (Eq. 3.8.2), per cavity at goff:
@@ -51,6 +68,7 @@ struct CavDev {
 //   copies used only where the arithmetic is FP32 (fused FP32 kernel)
 struct Geo {
   const double *xix, *xeH, *xxi, *xeta;
+  const double *ax[2];  // scale c xi_x(eta_j) / (2 dxi), scale = dt/2 and dt (FP64 staged kernels)
   const float *cxix_f, *jac_f;
   // general quadrilaterals (staged kernels): per node, at 7 * off + k * plane,
   // k = 0..6: xi_x, xi_y, eta_x, eta_y, x_eta, y_eta, J (Eqs. 3.2-3.3)
@@ -73,6 +91,7 @@ struct Bufs {
   double *part;      // residual partials [nparts_total][8]
   double *resid;     // [ncav][4] residual outputs
   int *tile_cav;     // staged tile -> cavity
+  int *blk_cav;      // block of the FP64 staged kernels -> cavity
   unsigned *status;  // bit 0: non-finite velocity seen
   CavDev *cav;       // [ncav]
   Geo geo;
@@ -87,6 +106,7 @@ struct StepArgs {
   const CavDev *cav;
   Geo geo;
   const int *tile_cav;
+  const int *blk_cav;
   const void *g_in;
   void *g_out;
   const void *lam_in;  // relaxation-time planes in the storage type T
@@ -144,10 +164,14 @@ template <class T> bool launch_fused(const FusedArgs &a, int nt, int ntasks, cud
 template <class T> int fused_smem_bytes(int nt);
 template <class T> int fused_blocks_per_sm(int nt);
 
-// Staged kernels (staged.cu)
-template <class T> void launch_collide(const StepArgs &a, int ntiles, cudaStream_t s);
-template <class T> void launch_half(const StepArgs &a, int ntiles, cudaStream_t s);
-template <class T> void launch_full(const StepArgs &a, int ntiles, cudaStream_t s);
+// Staged kernels of the FP32 storage (staged.cu)
+void launch_collide(const StepArgs &a, int ntiles, cudaStream_t s);
+void launch_half(const StepArgs &a, int ntiles, cudaStream_t s);
+void launch_full(const StepArgs &a, int ntiles, cudaStream_t s);
+// ... and of the FP64 storage (staged64.cu), on nblk blocks of nt threads
+void launch_collide64(const StepArgs &a, int nblk, int nt, cudaStream_t s);
+void launch_half64(const StepArgs &a, int nblk, int nt, cudaStream_t s);
+void launch_full64(const StepArgs &a, int nblk, int nt, cudaStream_t s);
 void launch_residual_reduce(const CavDev *cav, const double *part, double *resid, int ncav,
                             cudaStream_t s);
 

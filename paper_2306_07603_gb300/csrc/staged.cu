@@ -1,4 +1,5 @@
-// Staged IFDLBM step: three launches per time step, no recomputation.
+// Staged IFDLBM step of the FP32 storage (staged64.cu has the FP64 one): three
+// launches per time step, no recomputation; and the helper kernels of both.
 //
 //   k_collide  every node: Step (2) (moments, f^eq, lagged power-law lam),
 //              Step (3) f-hat^+ (Eq. 2.15) and f-bar^+ (Eq. 2.16)
@@ -8,12 +9,6 @@
 //   k_full     every node: Step (5) f-hat(t+dt) (Eq. 3.6); wall nodes by
 //              non-equilibrium extrapolation (Step 6); residual partials of
 //              Eq. (2.19) and Eq. (5.1)
-//
-// On GB300 the FP64 pipe runs at a small fraction of the FP32 rate, so the
-// FP64 step is bound by FP64 instructions, not bytes: this organisation
-// keeps every node's arithmetic to exactly one evaluation and pays with
-// intermediate planes (f-bar^+, f-hat^+, f(t+dt/2)) that stay in L2 for
-// the grid sizes of a cavity sweep.
 //
 // A wall node (i, j) takes its neighbour (clamp(i, 1, nx-2), clamp(j, 1,
 // ny-2)): the adjacent node along the grid normal on a side, the diagonal
@@ -68,7 +63,7 @@ __global__ void __launch_bounds__(TILE_X *TILE_Y) k_collide(StepArgs a) {
   const int64_t b9 = 9 * cv.off;
   T g[9];
   load9((const T *)a.g_in + b9, cv.plane, node, g);
-  const double lam_prev = double(((const T *)a.lam_in)[cv.off + node]);
+  const T lam_prev = ((const T *)a.lam_in)[cv.off + node];
 
   const T c = T(cv.c), cs2 = T(cv.cs2), ics2 = T(cv.inv_cs2);
   T ux, uy, P;
@@ -606,20 +601,20 @@ void launch_pow_f32_selftest(int n, const double *x, double m, double *out, cuda
 // ---------------------------------------------------------------------------
 static const dim3 kTile(TILE_X, TILE_Y);
 
-template <class T> void launch_collide(const StepArgs &a, int ntiles, cudaStream_t s) {
-  k_collide<T><<<ntiles, kTile, 0, s>>>(a);
+void launch_collide(const StepArgs &a, int ntiles, cudaStream_t s) {
+  k_collide<float><<<ntiles, kTile, 0, s>>>(a);
 }
-template <class T> void launch_half(const StepArgs &a, int ntiles, cudaStream_t s) {
+void launch_half(const StepArgs &a, int ntiles, cudaStream_t s) {
   if (a.geo.gmet)
-    k_half<T, true><<<ntiles, kTile, 0, s>>>(a);
+    k_half<float, true><<<ntiles, kTile, 0, s>>>(a);
   else
-    k_half<T, false><<<ntiles, kTile, 0, s>>>(a);
+    k_half<float, false><<<ntiles, kTile, 0, s>>>(a);
 }
-template <class T> void launch_full(const StepArgs &a, int ntiles, cudaStream_t s) {
+void launch_full(const StepArgs &a, int ntiles, cudaStream_t s) {
   if (a.geo.gmet)
-    k_full<T, true><<<ntiles, kTile, 0, s>>>(a);
+    k_full<float, true><<<ntiles, kTile, 0, s>>>(a);
   else
-    k_full<T, false><<<ntiles, kTile, 0, s>>>(a);
+    k_full<float, false><<<ntiles, kTile, 0, s>>>(a);
 }
 void launch_residual_reduce(const CavDev *cav, const double *part, double *resid, int ncav,
                             cudaStream_t s) {
@@ -661,9 +656,6 @@ template <class T> void launch_rebase(const CavDev *cav, const int *tile_cav, vo
 }
 
 #define IFD_INSTANTIATE(T)                                                                     \
-  template void launch_collide<T>(const StepArgs &, int, cudaStream_t);                       \
-  template void launch_half<T>(const StepArgs &, int, cudaStream_t);                          \
-  template void launch_full<T>(const StepArgs &, int, cudaStream_t);                          \
   template void launch_init<T>(const CavDev *, const int *, void *, void *, int,              \
                                cudaStream_t);                                                  \
   template void launch_macros<T>(const CavDev *, Geo, int, const double *, const void *,      \
