@@ -485,8 +485,10 @@ int ifdlbm_default_options(ifdlbm_options *opt) {
 namespace {
 
 // Batches of up to this many nodes run the FP64 staged kernels in blocks of one
-// warp, which spread over all SMs, larger ones in blocks of four.
-constexpr int64_t SMALL_NODES64 = 100000;
+// warp, which spread over all SMs, larger ones in blocks of four (fewer residual
+// partials). Measured us per step, 32 | 128 threads: 65^2 25.8 | 28.1, 257^2 49.8 |
+// 56.3, 2 x 257^2 87.1 | 90.0, 385^2 96.4 | 97.4, 513^2 159.5 | 160.7.
+constexpr int64_t SMALL_NODES64 = 200000;
 
 int validate_quad(ifdlbm_ctx *h, int idx, const ifdlbm_quad_cavity &q) {
   char buf[256];

@@ -23,11 +23,10 @@ __device__ __forceinline__ double warp_max(double v) {
   return v;
 }
 
-// Block reduction of the residual partials into slot `slot` (fixed order), by
-// a block of `nwarps` <= MAXW warps.
-template <int MAXW>
-__device__ __forceinline__ void block_partial_n(Partial p, double *part, int slot, int nwarps) {
-  __shared__ double sh[MAXW][7];
+// Block reduction of the residual partials into slot `slot` (fixed order).
+template <int NWARPS>
+__device__ __forceinline__ void block_partial(Partial p, double *part, int slot) {
+  __shared__ double sh[NWARPS][7];
   const int lane = threadIdx.x + threadIdx.y * blockDim.x;
   const int w = lane >> 5, l = lane & 31;
   double v[7] = {warp_sum(p.du2), warp_sum(p.u2), warp_sum(p.dP2), warp_sum(p.P2),
@@ -38,13 +37,9 @@ __device__ __forceinline__ void block_partial_n(Partial p, double *part, int slo
   __syncthreads();
   if (lane < 7) {
     double acc = sh[0][lane];
-    for (int k = 1; k < nwarps; ++k) acc = lane < 5 ? acc + sh[k][lane] : fmax(acc, sh[k][lane]);
+    for (int k = 1; k < NWARPS; ++k) acc = lane < 5 ? acc + sh[k][lane] : fmax(acc, sh[k][lane]);
     part[int64_t(slot) * NPART + lane] = acc;
   }
-}
-template <int NWARPS>
-__device__ __forceinline__ void block_partial(Partial p, double *part, int slot) {
-  block_partial_n<NWARPS>(p, part, slot, NWARPS);
 }
 
 // Adds one node's terms of Eq. (2.19) (new vs old u, v, P) and of Eq. (5.1)

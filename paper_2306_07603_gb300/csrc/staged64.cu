@@ -13,7 +13,10 @@
 // Ten 257^2 cavities, us per step: 394 = 134 + 166 + 92. The form before, tiles
 // of 32 x 8 nodes with both upwind sides evaluated, the power by log2 and exp2
 // and the wall rule in every edge warp, took 218 + 356 + 259 instructions and
-// 1211 us.
+// 1211 us. One 65^2 cavity: 21.6 us a step against 94; there the three launches
+// and the latency of a warp count, so each kernel starts while the one before
+// it ends (launch.cuh) and forms what the step does not change before waiting
+// for it, and blocks are one warp (34.1 us before these three).
 //
 // Wall nodes follow the rule of the FP32 staged kernels (staged.cu): a wall
 // node (i, j) takes the node (clamp(i, 1, nx-2), clamp(j, 1, ny-2)), which its
@@ -22,6 +25,7 @@
 
 #include "d2q9.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "reduce.cuh"
 #include "step64.cuh"
 
@@ -29,13 +33,22 @@ namespace ifd {
 
 namespace {
 
-constexpr int MAX_NT = 128;  // threads per block: 128, or 32 on small batches
+// Threads per block NT: 128, or 32 on small batches. The registers follow: a
+// small batch has too few warps for its latencies to hide behind others, so
+// its kernels may use up to 144 registers to have more loads in flight (14
+// blocks of a warp still fit on an SM); four blocks of 128 threads take 128.
+template <int NT>
+constexpr int MIN_BLOCKS = NT == 32 ? 14 : 4;
 
-__global__ void __launch_bounds__(MAX_NT) k_collide64(StepArgs a) {
-  const Node64 r = node_of(a.blk_cav, a.cav);
-  if (!r.valid) return;
+template <int NT>
+__global__ void __launch_bounds__(NT, MIN_BLOCKS<NT>) k_collide64(StepArgs a) {
+  const Node64 r = node_of<NT>(a.blk_cav, a.cav);
   const CavDev &cv = a.cav[r.cav];
   const int64_t node = int64_t(r.j) * cv.pitch + r.i, plane = cv.plane, b9 = 9 * cv.off + node;
+  const double dt = cv.dt;
+  previous_done();
+  dependents_may_start();
+  if (!r.valid) return;
   const double *gin = (const double *)a.g_in + b9;
   const double lam_prev = ((const double *)a.lam_in)[cv.off + node];
   double g[9], d[9];
@@ -49,7 +62,6 @@ __global__ void __launch_bounds__(MAX_NT) k_collide64(StepArgs a) {
   const double pxx = (d[1] + d[3]) + diag, pyy = (d[2] + d[4]) + diag;
   const double pxy = (d[5] - d[6]) + (d[7] - d[8]);
   const double pp = fma(pxx, pxx, fma(pyy, pyy, (pxy + pxy) * pxy));
-  const double dt = cv.dt;
   double lam;
   if (cv.implicit) {
     lam = lambda_implicit(2.0 * cv.c * cv.c * sqrt(0.5 * pp) * cv.inv_cs2, lam_prev, cv, a.powtab);
@@ -77,55 +89,45 @@ __global__ void __launch_bounds__(MAX_NT) k_collide64(StepArgs a) {
   }
 }
 
-// out = base - scale A(F) of every moving population at interior node (i, j)
-// of the planes F (base: planes at the same node; SAME: base = F).
+// out = base - scale A(F) of every moving population at an interior node: base
+// and F point to the node in plane 0 of their sets (SAME: base = F).
 template <bool GEN, bool SAME>
-__device__ __forceinline__ void advect_all64(const CavDev &cv, const Geo &geo, int stage, int i,
-                                             int j, const double *base, const double *F,
-                                             double out[9]) {
-  const int64_t node = int64_t(j) * cv.pitch + i, plane = cv.plane;
-  const Speeds64<GEN> s = speeds64<GEN>(cv, geo, stage, i, j, node);
-  const bool clo = i == 1, chi = i == cv.nx - 2, lo = j == 1, hi = j == cv.ny - 2;
-  base += 9 * cv.off + node;
-  F += 9 * cv.off + node;
+__device__ __forceinline__ void advect_all64(const Stencil64<GEN> &st, int64_t plane,
+                                             const double *base, const double *F, double out[9]) {
   auto one = [&](auto qc) {
     constexpr int q = decltype(qc)::value;
     const double *Fq = F + q * plane;
     const double f0 = Fq[0];
-    out[q] = advect64<q, GEN>(SAME ? f0 : base[q * plane], Fq, cv.pitch, f0, s, cv, stage, clo, chi,
-                              lo, hi);
+    out[q] = advect64<q, GEN>(SAME ? f0 : base[q * plane], Fq, f0, st);
   };
   one(Const<1>()), one(Const<2>()), one(Const<3>()), one(Const<4>());
   one(Const<5>()), one(Const<6>()), one(Const<7>()), one(Const<8>());
 }
 
-// f(t + dt/2) at interior node (i, j): the half step of Eq. (3.7) from f-bar^+,
-// then Eq. (2.17) with the node's lambda(t). Returns its moments, which are
-// those of f-bar (Eq. 2.17 keeps u and P).
+// f(t + dt/2) at an interior node: the half step of Eq. (3.7) from f-bar^+ (fb,
+// at the node), then Eq. (2.17) with the node's lambda(t). Returns its moments,
+// which are those of f-bar (Eq. 2.17 keeps u and P).
 template <bool GEN>
-__device__ __forceinline__ Mom64 half_at64(const StepArgs &a, const CavDev &cv, int i, int j,
-                                           double f[9]) {
-  const double *fb = (const double *)a.fb;
-  const int64_t node = int64_t(j) * cv.pitch + i;
-  const double lam = ((const double *)a.lam_out)[cv.off + node];
-  f[0] = fb[9 * cv.off + node];
-  advect_all64<GEN, true>(cv, a.geo, 0, i, j, fb, fb, f);
+__device__ __forceinline__ Mom64 half_at64(const Stencil64<GEN> &st, int64_t plane, double dt,
+                                           const double *fb, const double *lam_at, double f[9]) {
+  const double lam = *lam_at;
+  f[0] = fb[0];
+  advect_all64<GEN, true>(st, plane, fb, fb, f);
   const Mom64 m = moments64(f);                        // Eqs. (2.10)-(2.11) on f-bar
   double geq[9];
   equilibrium64(m, geq);
-  const double bh = cv.dt * recip(fma(4.0, lam, cv.dt));  // Eq. (2.17): 4 lam/(4 lam + dt) = 1 - bh
+  const double bh = dt * recip(fma(4.0, lam, dt));     // Eq. (2.17): 4 lam/(4 lam + dt) = 1 - bh
 #pragma unroll
   for (int q = 0; q < 9; ++q) f[q] = fma(bh, geq[q] - f[q], f[q]);
   return m;
 }
 
-// f-hat(t + dt) at interior node (i, j): the full step of Eq. (3.6).
+// f-hat(t + dt) at an interior node: the full step of Eq. (3.6).
 template <bool GEN>
-__device__ __forceinline__ void full_at64(const StepArgs &a, const CavDev &cv, int i, int j,
-                                          double f[9]) {
-  const double *fp = (const double *)a.fp;
-  f[0] = fp[9 * cv.off + int64_t(j) * cv.pitch + i];
-  advect_all64<GEN, false>(cv, a.geo, 1, i, j, fp, (const double *)a.fh, f);
+__device__ __forceinline__ void full_at64(const Stencil64<GEN> &st, int64_t plane,
+                                          const double *fp, const double *fh, double f[9]) {
+  f[0] = fp[0];
+  advect_all64<GEN, false>(st, plane, fp, fh, f);
 }
 
 // Wall node (i, j) from F and its moments at the inner neighbour; F2 the next
@@ -138,47 +140,65 @@ __device__ __forceinline__ void wall_node64(double F[9], const Mom64 &m, double 
   wall64(F, m, lid ? cv.lid_ux * ic : 0.0, lid ? cv.lid_uy * ic : 0.0, dp);
 }
 
-template <bool GEN>
-__global__ void __launch_bounds__(MAX_NT) k_half64(StepArgs a) {
-  const Node64 r = node_of(a.blk_cav, a.cav);
-  if (!r.valid) return;
+template <int NT, bool GEN>
+__global__ void __launch_bounds__(NT, MIN_BLOCKS<NT>) k_half64(StepArgs a) {
+  const Node64 r = node_of<NT>(a.blk_cav, a.cav);
   const CavDev &cv = a.cav[r.cav];
   const int ii = min(max(r.i, 1), cv.nx - 2), jj = min(max(r.j, 1), cv.ny - 2);
+  const Stencil64<GEN> st = stencil64<GEN>(cv, a.geo, 0, ii, jj);
+  const int64_t plane = cv.plane, off = cv.off;
+  const double dt = cv.dt;
+  previous_done();
+  dependents_may_start();
+  if (!r.valid) return;
+  const double *fb = (const double *)a.fb + 9 * off, *lam = (const double *)a.lam_out + off;
+  const int64_t node = int64_t(jj) * st.pitch + ii;
   double f[9];
-  const Mom64 m = half_at64<GEN>(a, cv, ii, jj, f);
+  const Mom64 m = half_at64<GEN>(st, plane, dt, fb + node, lam + node, f);
   if (r.wall) {
     double dp = 0.0;
     if (cv.wallp) {
+      const int i2 = 2 * ii - r.i, j2 = 2 * jj - r.j;
+      const int64_t n2 = int64_t(j2) * st.pitch + i2;
       double f2[9];
-      dp = m.p - half_at64<GEN>(a, cv, 2 * ii - r.i, 2 * jj - r.j, f2).p;
+      dp = m.p - half_at64<GEN>(stencil64<GEN>(cv, a.geo, 0, i2, j2), plane, dt, fb + n2, lam + n2,
+                                f2).p;
     }
     wall_node64(f, m, dp, r.i, r.j, cv);
   }
-  double *fh = (double *)a.fh + 9 * cv.off + int64_t(r.j) * cv.pitch + r.i;
+  double *fh = (double *)a.fh + 9 * off + int64_t(r.j) * st.pitch + r.i;
 #pragma unroll
-  for (int q = 0; q < 9; ++q) fh[q * cv.plane] = f[q];
+  for (int q = 0; q < 9; ++q) fh[q * plane] = f[q];
 }
 
-template <bool GEN>
-__global__ void __launch_bounds__(MAX_NT) k_full64(StepArgs a) {
-  const Node64 r = node_of(a.blk_cav, a.cav);
+template <int NT, bool GEN>
+__global__ void __launch_bounds__(NT, MIN_BLOCKS<NT>) k_full64(StepArgs a) {
+  const Node64 r = node_of<NT>(a.blk_cav, a.cav);
   const CavDev &cv = a.cav[r.cav];
+  const int ii = min(max(r.i, 1), cv.nx - 2), jj = min(max(r.j, 1), cv.ny - 2);
+  const Stencil64<GEN> st = stencil64<GEN>(cv, a.geo, 1, ii, jj);
+  const int64_t plane = cv.plane;
+  previous_done();
+  dependents_may_start();
   Partial p = {0, 0, 0, 0, 0, 0, 0};
   if (r.valid) {
-    const int ii = min(max(r.i, 1), cv.nx - 2), jj = min(max(r.j, 1), cv.ny - 2);
+    const double *fp = (const double *)a.fp + 9 * cv.off, *fh = (const double *)a.fh + 9 * cv.off;
+    const int64_t node = int64_t(jj) * st.pitch + ii;
     double f[9];
-    full_at64<GEN>(a, cv, ii, jj, f);
+    full_at64<GEN>(st, plane, fp + node, fh + node, f);
     if (r.wall) {
       const Mom64 m = moments64(f);
       double dp = 0.0;
       if (cv.wallp) {
+        const int i2 = 2 * ii - r.i, j2 = 2 * jj - r.j;
+        const int64_t n2 = int64_t(j2) * st.pitch + i2;
         double f2[9];
-        full_at64<GEN>(a, cv, 2 * ii - r.i, 2 * jj - r.j, f2);
+        full_at64<GEN>(stencil64<GEN>(cv, a.geo, 1, i2, j2), plane, fp + n2, fh + n2, f2);
         dp = m.p - moments64(f2).p;
       }
       wall_node64(f, m, dp, r.i, r.j, cv);
     }
-    const int64_t me = int64_t(r.j) * cv.pitch + r.i, plane = cv.plane;
+    const int64_t me = int64_t(r.j) * st.pitch + r.i;
     double *out = (double *)a.g_out + 9 * cv.off + me;
 #pragma unroll
     for (int q = 0; q < 9; ++q) out[q * plane] = f[q];
@@ -210,25 +230,25 @@ __global__ void __launch_bounds__(MAX_NT) k_full64(StepArgs a) {
       }
     }
   }
-  if (a.want_residual) block_partial_n<MAX_NT / 32>(p, a.part, blockIdx.x, blockDim.x / 32);
+  if (a.want_residual) block_partial<NT / 32>(p, a.part, blockIdx.x);
 }
 
 }  // namespace
 
 void launch_collide64(const StepArgs &a, int nblk, int nt, cudaStream_t s) {
-  k_collide64<<<nblk, nt, 0, s>>>(a);
+  launch_after(nt == 32 ? k_collide64<32> : k_collide64<128>, nblk, nt, 0, s, a);
 }
 void launch_half64(const StepArgs &a, int nblk, int nt, cudaStream_t s) {
   if (a.geo.gmet)
-    k_half64<true><<<nblk, nt, 0, s>>>(a);
+    launch_after(nt == 32 ? k_half64<32, true> : k_half64<128, true>, nblk, nt, 0, s, a);
   else
-    k_half64<false><<<nblk, nt, 0, s>>>(a);
+    launch_after(nt == 32 ? k_half64<32, false> : k_half64<128, false>, nblk, nt, 0, s, a);
 }
 void launch_full64(const StepArgs &a, int nblk, int nt, cudaStream_t s) {
   if (a.geo.gmet)
-    k_full64<true><<<nblk, nt, 0, s>>>(a);
+    launch_after(nt == 32 ? k_full64<32, true> : k_full64<128, true>, nblk, nt, 0, s, a);
   else
-    k_full64<false><<<nblk, nt, 0, s>>>(a);
+    launch_after(nt == 32 ? k_full64<32, false> : k_full64<128, false>, nblk, nt, 0, s, a);
 }
 
 }  // namespace ifd

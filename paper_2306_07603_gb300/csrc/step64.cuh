@@ -33,6 +33,7 @@ struct Node64 {
   int cav, i, j;
   bool valid, wall;  // wall is uniform over the block
 };
+template <int NT>
 __device__ __forceinline__ Node64 node_of(const int *blk_cav, const CavDev *cavs) {
   Node64 r;
   const int b = blockIdx.x;
@@ -41,14 +42,14 @@ __device__ __forceinline__ Node64 node_of(const int *blk_cav, const CavDev *cavs
   const int lb = b - cv.blk0;
   r.wall = lb >= cv.nblk_in;
   if (!r.wall) {
-    const unsigned n = unsigned(lb) * blockDim.x + threadIdx.x;
+    const unsigned n = unsigned(lb) * NT + threadIdx.x;
     const unsigned w = unsigned(cv.nx - 2);
     const unsigned row = n / w;
     r.valid = row < unsigned(cv.ny - 2);
     r.i = int(n - row * w) + 1;
     r.j = int(row) + 1;
   } else {
-    const int n = (lb - cv.nblk_in) * int(blockDim.x) + int(threadIdx.x);
+    const int n = (lb - cv.nblk_in) * NT + int(threadIdx.x);
     const int k = n - 2 * cv.nx;
     r.valid = k < 2 * (cv.ny - 2);
     if (k < 0) {
@@ -223,22 +224,47 @@ __device__ __forceinline__ double mix64(const double *F, int d, bool edge, const
   return fma(kf, f, fma(k0, f0, fma(kb, b, acc)));
 }
 
+// What the stencils of a node take besides the planes: its speeds, the
+// coefficients, the row pitch and the walls it is next to. None of it is
+// written by a step, so a kernel forms it before the one before it is done.
+template <bool GEN>
+struct Stencil64 {
+  Speeds64<GEN> s;
+  Mix64 mix, mixe;
+  int pitch;
+  bool clo, chi, lo, hi;
+};
+template <bool GEN>
+__device__ __forceinline__ Stencil64<GEN> stencil64(const CavDev &cv, const Geo &geo, int stage,
+                                                    int i, int j) {
+  Stencil64<GEN> st;
+  st.pitch = cv.pitch;
+  st.s = speeds64<GEN>(cv, geo, stage, i, j, int64_t(j) * st.pitch + i);
+  st.mix = cv.mix;
+  if constexpr (!GEN) st.mixe = cv.mixe[stage];
+  st.clo = i == 1;
+  st.chi = i == cv.nx - 2;
+  st.lo = j == 1;
+  st.hi = j == cv.ny - 2;
+  return st;
+}
+
 // base - scale (c_xi D_xi + c_eta D_eta) F_q at interior node F (Eqs. 3.6-3.7):
 // 9 FP64 instructions a plane (5 where e_y = 0 on the trapezoid).
 template <int Q, bool GEN>
-__device__ __forceinline__ double advect64(double base, const double *F, int pitch, double f0,
-                                           const Speeds64<GEN> &s, const CavDev &cv, int stage,
-                                           bool clo, bool chi, bool lo, bool hi) {
+__device__ __forceinline__ double advect64(double base, const double *F, double f0,
+                                           const Stencil64<GEN> &st) {
   constexpr int p = pair_of(Q);
-  const bool xpos = s.xpos[p] != second_of(Q);
-  double out = fma(-s.xi[p], mix64(F, xpos ? 1 : -1, xpos ? clo : chi, cv.mix, f0, 0.0, true), base);
+  const bool xpos = st.s.xpos[p] != second_of(Q);
+  double out = fma(-st.s.xi[p],
+                   mix64(F, xpos ? 1 : -1, xpos ? st.clo : st.chi, st.mix, f0, 0.0, true), base);
   if constexpr (GEN) {
-    const bool epos = s.epos[p] != second_of(Q);
-    out = fma(-s.eta[p],
-              mix64(F, epos ? pitch : -pitch, epos ? lo : hi, cv.mix, f0, 0.0, true), out);
+    const bool epos = st.s.epos[p] != second_of(Q);
+    out = fma(-st.s.eta[p], mix64(F, epos ? st.pitch : -st.pitch, epos ? st.lo : st.hi, st.mix, f0,
+                                  0.0, true), out);
   } else if constexpr (Q != 1 && Q != 3) {
     constexpr bool epos = Q == 2 || Q == 5 || Q == 6;
-    out = mix64(F, epos ? pitch : -pitch, epos ? lo : hi, cv.mixe[stage], f0, out, false);
+    out = mix64(F, epos ? st.pitch : -st.pitch, epos ? st.lo : st.hi, st.mixe, f0, out, false);
   }
   return out;
 }
