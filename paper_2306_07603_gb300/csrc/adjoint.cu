@@ -12,16 +12,36 @@
 // X(F) = E(u_w, P(F)) + F - E(u(F), P(F)). Since dE/dP does not depend on u,
 // X^T(G) = G - c (e_x ubar + e_y vbar) with (ubar, vbar) = (dE/du)^T G at u(F).
 //
-// The reverse sweep runs A3 walls -> A3 stencil gather -> A2 walls -> A2
-// pointwise -> A2 stencil gather -> A1 pointwise, then reduces the parameter
-// partials. Parameters: n (through K = U^(2-n) H^n / Re and the exponent),
-// Re (through K) and theta in degrees (through c_xi of Eq. 3.4 via cot theta,
-// and the Jacobian of the kinetic-energy objective of Eq. 5.1).
+// The reverse sweep of a step takes three launches and a reduction:
+//
+//   k_adj_ring   G' = Gbar + X^T(walls) at the interior nodes next to a wall, in
+//                place (each wall node has one source, so no two threads meet)
+//   k_adj_full   FHbar = -dt A^T(G'), its wall terms by evaluating the gather
+//                again at the wall nodes of a ring node, and the half step's
+//                pointwise adjoint: FBARbar = ah FHbar + M^T E^T (bh FHbar)
+//   k_adj_half   FBbar = FBARbar - dt/2 A^T(FBARbar) and the collision's adjoint,
+//                that of (g_n, lambda_n)
+//
+// Parameters: n (through K = U^(2-n) H^n / Re and the exponent), Re (through K)
+// and theta in degrees (through c_xi of Eq. 3.4 via cot theta, and the
+// Jacobian of the kinetic-energy objective of Eq. 5.1); their partials are
+// summed per block and then per cavity, in a fixed order.
+//
+// Bound: the FP64 pipe, as the forward step (step64.cuh). The gathers take four
+// terms per axis with the coefficients and sides selected by integer
+// instructions, the transposed moments and equilibrium are summed by pairs of
+// opposite directions, and no pass re-forms what another has in registers.
+// FP64 instructions per warp: k_adj_full 305, k_adj_half 412, the ring a small
+// extra; a reverse step at 257^2 takes 126 us, at 65^2 53 us (there the latency
+// of a warp). The nine launches before (wall transposes and additions as
+// kernels of their own, gathers of both upwind sides) took 1980 and 400 us.
 #include <cstdint>
 
 #include "d2q9.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "reduce.cuh"
+#include "step64.cuh"
 
 namespace ifd {
 
@@ -44,190 +64,244 @@ __device__ __forceinline__ Ref tile_ref(const int *tile_cav, const CavDev *cavs)
   return r;
 }
 
-__device__ __forceinline__ bool interior(const CavDev &cv, int i, int j) {
-  return i >= 1 && i <= cv.nx - 2 && j >= 1 && j <= cv.ny - 2;
-}
-
-// (dE/d(u, v, P))^T eb at (ux, uy).
-__device__ __forceinline__ void equilibrium_T(const double eb[9], double ux, double uy,
-                                              const CavDev &cv, double &ub, double &vb,
-                                              double &Pb) {
-  const double c = cv.c, ics2 = cv.inv_cs2;
-  ub = vb = Pb = 0.0;
+// Sum over the block of the N <= 8 values v, written by its first N threads to
+// part[slot * N ..] (fixed order).
+template <int N, int NWARPS>
+__device__ __forceinline__ void block_sum(const double (&v)[N], double *part, int64_t slot) {
+  __shared__ double sh[NWARPS][N];
+  const int lane = threadIdx.x + threadIdx.y * blockDim.x;
+  const int w = lane >> 5, l = lane & 31;
+  double v8[8] = {};
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const double cu = c * (ex(i) * ux + ey(i) * uy);
-    const double w = wgt(i) * eb[i];
-    const double tt = ics2 + cu * ics2 * ics2;
-    ub += w * (c * ex(i) * tt - ux * ics2);
-    vb += w * (c * ey(i) * tt - uy * ics2);
-    Pb += wbar(i) * eb[i] * ics2;
+  for (int k = 0; k < N; ++k) v8[k] = v[k];
+  const double s = warp_sums8(v8);
+  if ((l & 3) == 0 && l < 4 * N) sh[w][l >> 2] = s;
+  __syncthreads();
+  if (lane < N) {
+    double acc = 0.0;
+    for (int k = 0; k < NWARPS; ++k) acc += sh[k][lane];
+    part[slot * N + lane] = acc;
   }
 }
 
-// gb += (dM/dg)^T (ub, vb, Pb) at (ux, uy), M the moments of Eqs. (2.10)-(2.11).
-__device__ __forceinline__ void moments_T(double ub, double vb, double Pb, double ux, double uy,
-                                          const CavDev &cv, double gb[9]) {
-  const double c = cv.c;
-  const double alpha = cv.cs2 / wbar(0), beta = wgt(0) / (2.0 * cv.cs2);
-  const double A = ub + 2.0 * alpha * beta * ux * Pb, B = vb + 2.0 * alpha * beta * uy * Pb;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) gb[i] += c * (ex(i) * A + ey(i) * B) - (i >= 1 ? alpha * Pb : 0.0);
-}
-
-// G <- X^T(G) at F (the wall rule's transpose; u(F) only).
-__device__ __forceinline__ void nee_T(double G[9], const double F[9], const CavDev &cv) {
-  double ux, uy, P;
-  moments(F, cv.c, cv.cs2, ux, uy, P);
-  double ub, vb, Pb;
-  equilibrium_T(G, ux, uy, cv, ub, vb, Pb);
-#pragma unroll
-  for (int i = 0; i < 9; ++i) G[i] -= cv.c * (ex(i) * ub + ey(i) * vb);
-}
-
-// The distinct coefficients of the mixed difference of Eq. (2.5) (times 2 d)
-// for blend eta, formed once per thread: eta, o = 1 - eta, 2 o, 3 o,
-// eta + 2 o and eta + 4 o.
-struct Blend {
-  double e, o, o2, o3, e2, e4;
-};
-__device__ __forceinline__ Blend make_blend(double eta) {
-  const double o = 1.0 - eta;
-  return {eta, o, 2.0 * o, 3.0 * o, eta + 2.0 * o, eta + 4.0 * o};
-}
-
-// Coefficient of F[x + k] in the mixed difference of Eq. (2.5) at node x
-// (times 2 d), for the upwind side `pos` and the near-wall flags lo / hi.
-__device__ __forceinline__ double wmix(int k, bool pos, bool lo, bool hi, const Blend &b) {
-  if (pos) {
-    if (lo) return k == -1 ? -b.e2 : (k == 0 ? b.o2 : (k == 1 ? b.e : 0.0));
-    return k == -2 ? b.o : (k == -1 ? -b.e4 : (k == 0 ? b.o3 : (k == 1 ? b.e : 0.0)));
-  }
-  if (hi) return k == -1 ? -b.e : (k == 0 ? -b.o2 : (k == 1 ? b.e2 : 0.0));
-  return k == -1 ? -b.e : (k == 0 ? -b.o3 : (k == 1 ? b.e4 : (k == 2 ? -b.o : 0.0)));
-}
-
-__device__ __forceinline__ double cxi_at(const CavDev &cv, const Geo &g, int q, int i, int j) {
-  const double A = cv.c * g.xix[cv.goff + j];
-  return ex(q) * A - ey(q) * A * g.xeH[cv.goff + i];
-}
-
-// Per-node terms of c_{q xi} and of its theta derivative, formed once for all
-// planes: with A = c xi_x and x_eta / H of the node, c_{q xi} = e_x A - e_y A
-// x_eta / H (as cxi_at), and, through x_xi = L + 2 H cot eta and x_eta = H cot
-// (2 xi - 1), d c_{q xi} / d theta_deg = e_y t1 - e_x t2 with
-// t1 = (-A (2 xi - 1) + A x_eta/H K) dcot, t2 = A K dcot, K = 2 H eta xi_x.
-struct NodeXi {
-  double A, xe, t1, t2;
-  __device__ __forceinline__ double cxi(int q) const { return ex(q) * A - ey(q) * A * xe; }
-  __device__ __forceinline__ double dcxi(int q) const { return ey(q) * t1 - ex(q) * t2; }
-};
-__device__ __forceinline__ NodeXi node_xi(const CavDev &cv, const Geo &g, int i, int j) {
-  const double xix = g.xix[cv.goff + j];
-  const double A = cv.c * xix, xe = g.xeH[cv.goff + i];
-  const double K = 2.0 * cv.H * (j * cv.deta) * xix;
-  return {A, xe, (-A * (2.0 * (i * cv.dxi) - 1.0) + A * xe * K) * cv.dcot, A * K * cv.dcot};
-}
-
-// D_xi F_q at interior node (i, j) of plane F (as in the forward kernels), on
-// the upwind side of c_{q xi} = cx.
-__device__ __forceinline__ double dxi_with(const CavDev &cv, const double *F, double cx, int i,
-                                           int j) {
-  const int64_t node = int64_t(j) * cv.pitch + i;
-  const int im2 = i >= 2 ? -2 : -1, ip2 = i <= cv.nx - 3 ? 2 : 1;
-  return dmix2(F[node + im2], F[node - 1], F[node], F[node + 1], F[node + ip2], cx >= 0.0, i == 1,
-               i == cv.nx - 2, cv.eta_b) * cv.inv2dxi;
-}
-__device__ __forceinline__ double dxi_at(const CavDev &cv, const Geo &g, const double *F, int q,
-                                         int i, int j) {
-  return dxi_with(cv, F, cxi_at(cv, g, q, i, j), i, j);
-}
-
-// Gather of the transposed advection: sum over interior x on the xi and eta
-// lines through y of Gb_q(x) dA_q(x)/dF_q(y). c_{q xi}(x) is formed as in
-// cxi_at (the row's metric c xi_x loaded once), so that its sign, which picks
-// the upwind side, is the forward step's; the constant factors 1 / (2 dxi)
-// and c_{q eta} / (2 deta) are applied to each line's sum.
-__device__ __forceinline__ double advect_T(const CavDev &cv, const Geo &g, const double *Gb, int q,
-                                           int i, int j, const Blend &bl) {
-  double acc = 0.0;
-  if (j >= 1 && j <= cv.ny - 2) {
-    const double A = cv.c * g.xix[cv.goff + j];
-    const double *row = Gb + int64_t(j) * cv.pitch;
-    double sx = 0.0;
-#pragma unroll
-    for (int k = -2; k <= 2; ++k) {
-      const int xi = i - k;  // F(y) = F(x + k)
-      if (xi < 1 || xi > cv.nx - 2) continue;
-      const double cx = ex(q) * A - ey(q) * A * g.xeH[cv.goff + xi];
-      const double w = wmix(k, cx >= 0.0, xi == 1, xi == cv.nx - 2, bl);
-      if (w != 0.0) sx += row[xi] * cx * w;
+// The interior node of this thread: blocks [0, nblk_core) of a cavity take the
+// nodes away from the walls row by row, the blocks after them the ring of
+// nodes next to a wall (rows 1 and ny-2, then columns 1 and nx-2 in turn).
+template <int NT>
+__device__ __forceinline__ Node64 interior_node(const int *blk_cav, const CavDev *cavs,
+                                                bool ring_only) {
+  Node64 r;
+  r.cav = blk_cav[blockIdx.x];
+  const CavDev &cv = cavs[r.cav];
+  const int lb = int(blockIdx.x) - (ring_only ? cv.ring0 : cv.adj0);
+  const int core = ring_only ? 0 : cv.nblk_core;
+  r.wall = lb >= core;  // a ring node
+  if (!r.wall) {
+    const unsigned n = unsigned(lb) * NT + threadIdx.x, w = unsigned(cv.nx - 4), row = n / w;
+    r.valid = row < unsigned(cv.ny - 4);
+    r.i = int(n - row * w) + 2;
+    r.j = int(row) + 2;
+  } else {
+    const int n = (lb - core) * NT + int(threadIdx.x), w = cv.nx - 2, k = n - 2 * w;
+    r.valid = k < 2 * (cv.ny - 4);
+    if (k < 0) {
+      const bool top = n >= w;
+      r.i = 1 + (top ? n - w : n);
+      r.j = top ? cv.ny - 2 : 1;
+    } else {
+      r.i = (k & 1) ? cv.nx - 2 : 1;
+      r.j = 2 + (k >> 1);
     }
-    acc = sx * cv.inv2dxi;
   }
-  const double ceta = double(ey(q)) * cv.c / cv.H;
-  if (i >= 1 && i <= cv.nx - 2 && ceta != 0.0) {
-    double se = 0.0;
+  return r;
+}
+
+// (dE / d(m_x, m_y, p))^T h at m, E the equilibrium in lattice units
+// (equilibrium64): x, y, p.
+struct Adj64 {
+  double x, y, p;
+};
+__device__ __forceinline__ Adj64 equilibrium_T(const double h[9], double mx, double my) {
+  const double s13 = h[1] + h[3], d13 = h[1] - h[3], s24 = h[2] + h[4], d24 = h[2] - h[4];
+  const double s57 = h[5] + h[7], d57 = h[5] - h[7], s68 = h[6] + h[8], d68 = h[6] - h[8];
+  const double t9 = (1.0 / 9.0) * fma(0.25, s57 + s68, s13 + s24);
+  const double w3 = -3.0 * fma(4.0 / 9.0, h[0], t9);  // -3 sum w_i h_i
+  const double a = (mx + my) * s57, b = (my - mx) * s68;
+  Adj64 r;
+  r.p = fma(-5.0 / 9.0, h[0], t9);
+  r.x = fma(1.0 / 3.0, d13, fma(1.0 / 12.0, d57 - d68, fma(0.25, a - b, mx * (s13 + w3))));
+  r.y = fma(1.0 / 3.0, d24, fma(1.0 / 12.0, d57 + d68, fma(0.25, a + b, my * (s24 + w3))));
+  return r;
+}
+
+// out[i] = k h[i] + (dM/dg)^T (x, y, p), M the moments of moments64 at m.
+__device__ __forceinline__ void moments_T(const Adj64 &b, double mx, double my, double k,
+                                          const double h[9], double out[9]) {
+  const double p2 = -2.4 * b.p, X = fma(p2, mx, b.x), Y = fma(p2, my, b.y), Z = 1.8 * b.p;
+  const double s = X + Y, d = Y - X;
+  out[0] = k * h[0];
+  out[1] = fma(k, h[1], Z + X);
+  out[3] = fma(k, h[3], Z - X);
+  out[2] = fma(k, h[2], Z + Y);
+  out[4] = fma(k, h[4], Z - Y);
+  out[5] = fma(k, h[5], Z + s);
+  out[7] = fma(k, h[7], Z - s);
+  out[6] = fma(k, h[6], Z + d);
+  out[8] = fma(k, h[8], Z - d);
+}
+
+// h += X^T(w), X the wall rule (Sec. 4) at the populations F of the inner
+// neighbour: X^T(w) = w - e (dE/dm)^T w.
+__device__ __forceinline__ void wall_T(double h[9], const double w[9], double mx, double my) {
+  const Adj64 b = equilibrium_T(w, mx, my);
+  const double s = b.x + b.y, d = b.y - b.x;
+  h[0] += w[0];
+  h[1] += w[1] - b.x;
+  h[3] += w[3] + b.x;
+  h[2] += w[2] - b.y;
+  h[4] += w[4] + b.y;
+  h[5] += w[5] - s;
+  h[7] += w[7] + s;
+  h[6] += w[6] - d;
+  h[8] += w[8] + d;
+}
+
+// The wall nodes whose extrapolation source is ring node (i, j), at most three:
+// the node across the side wall, the one across the bottom or lid, and at a
+// corner the diagonal one. `k` in 0..2; false if there is no such node.
+__device__ __forceinline__ bool wall_of(const CavDev &cv, int i, int j, int k, int &wi, int &wj) {
+  const int si = i == 1 ? 0 : (i == cv.nx - 2 ? cv.nx - 1 : -1);
+  const int sj = j == 1 ? 0 : (j == cv.ny - 2 ? cv.ny - 1 : -1);
+  wi = k == 1 ? i : si;
+  wj = k == 0 ? j : sj;
+  return (k == 1 || si >= 0) && (k == 0 || sj >= 0);
+}
+
+// What a gather at node (i, j) takes besides the planes. xi: the nodes x = i + o,
+// o = -2..2, that the transposed stencils of row j reach: which are interior
+// (none if j is a wall row) and which are next to a wall; eta: the same for
+// the rows j + o of column i. Bit o + 2.
+struct Gather64 {
+  const double *G;        // plane 0 at the node
+  int64_t plane;
+  int pitch, ix;          // ix: index of the node in the column tables
+  unsigned xin, xlo, xhi, ein, elo, ehi;
+  double A;               // scale c xi_x / (2 dxi) of the row
+};
+__device__ __forceinline__ unsigned bits5(int at, int lo, int hi) {
+  // bit o + 2 for lo <= at + o <= hi
+  unsigned b = 0;
 #pragma unroll
-    for (int k = -2; k <= 2; ++k) {
-      const int yj = j - k;
-      if (yj < 1 || yj > cv.ny - 2) continue;
-      const double w = wmix(k, ceta >= 0.0, yj == 1, yj == cv.ny - 2, bl);
-      if (w != 0.0) se += Gb[int64_t(yj) * cv.pitch + i] * w;
-    }
-    acc += se * (ceta * cv.inv2deta);
-  }
+  for (int o = -2; o <= 2; ++o) b |= (at + o >= lo && at + o <= hi) ? 1u << (o + 2) : 0u;
+  return b;
+}
+__device__ __forceinline__ Gather64 gather_at(const CavDev &cv, const Geo &geo, int stage, int i,
+                                              int j) {
+  Gather64 g;
+  g.plane = cv.plane;
+  g.pitch = cv.pitch;
+  g.ix = cv.goff + i;
+  const bool row = j >= 1 && j <= cv.ny - 2, col = i >= 1 && i <= cv.nx - 2;
+  g.xin = row ? bits5(i, 1, cv.nx - 2) : 0u;
+  g.xlo = bits5(i, 1, 1);
+  g.xhi = bits5(i, cv.nx - 2, cv.nx - 2);
+  g.ein = col ? bits5(j, 1, cv.ny - 2) : 0u;
+  g.elo = bits5(j, 1, 1);
+  g.ehi = bits5(j, cv.ny - 2, cv.ny - 2);
+  g.A = geo.ax[stage][cv.goff + j];
+  g.G = nullptr;
+  return g;
+}
+
+// Sum over the nodes x = y + o d of one line through y of G(x) m(x) times the
+// coefficient of F(y) in the mixed difference at x, added to acc: x = y is the
+// centre, x one node upwind of y takes y as its downwind neighbour (ka), one
+// node downwind as its upwind one (kb), two downwind as the far one (kf).
+// `pos`: bit o + 2, the side of x; `in`, `lo`, `hi` as in Gather64. UNIT: m = 1.
+// Where the side changes between y - 2 (from above) and y + 2 (from below)
+// both far terms are there; elsewhere there is one at most.
+template <bool UNIT>
+__device__ __forceinline__ double line_T(const double *G, int d, unsigned pos, unsigned in,
+                                         unsigned lo, unsigned hi, const double m[5],
+                                         const Mix64 &c, double acc) {
+  const unsigned edge = (pos & lo) | (~pos & hi);
+  auto side = [&](unsigned b, unsigned bit) { return (b & bit) != 0; };
+  auto put = [&](int o, double k) {
+    const bool on = side(in, 1u << (o + 2));
+    const double w = on ? (UNIT ? k : k * m[o + 2]) : 0.0;
+    acc = fma(w, G[on ? o * d : 0], acc);
+  };
+  const double km = side(edge, 2u) ? c.wb : c.kb, kp = side(edge, 8u) ? c.wb : c.kb;
+  put(0, side(edge, 4u) ? c.w0 : c.k0);
+  put(-1, side(pos, 2u) ? c.ka : km);
+  put(1, side(pos, 8u) ? kp : c.ka);
+  const bool up = side(pos & in, 16u), down = side(~pos & in, 1u);
+  const double mf = UNIT ? 1.0 : (up ? m[4] : m[0]);
+  acc = fma((up || down) ? (UNIT ? c.kf : c.kf * mf) : 0.0, G[up ? 2 * d : (down ? -2 * d : 0)], acc);
+  if (up && down) acc = fma(UNIT ? c.kf : c.kf * m[0], G[-2 * d], acc);
   return acc;
 }
 
-// Adds sum over the wall nodes whose extrapolation source is interior node
-// (i, j) of their adjoints, transposed through the wall rule at F(i, j).
-__device__ __forceinline__ void wall_gather_T(const CavDev &cv, const double *Gplanes,
-                                              const double *Fplanes, int i, int j, double out[9]) {
-  double G[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  bool any = false;
-  const int bi[3] = {i, i == 1 ? 0 : -1, i == cv.nx - 2 ? cv.nx - 1 : -1};
-  const int bj[3] = {j, j == 1 ? 0 : -1, j == cv.ny - 2 ? cv.ny - 1 : -1};
+// out[q] += -scale (A^T G)_q at the gather's node, all moving populations.
+__device__ __forceinline__ void advect_T(const Gather64 &g, const Geo &geo, const Mix64 &mix,
+                                         const Mix64 &mixe, double out[9]) {
+  auto pair = [&](auto pc) {
+    constexpr int p = decltype(pc)::value;
+    constexpr int q0 = p == 0 ? 1 : (p == 1 ? 2 : (p == 2 ? 5 : 6)), q1 = p < 2 ? q0 + 2 : q0 + 2;
+    // side and magnitude of c_xi / (c xi_x) at the five nodes, for q0
+    double m[5] = {1.0, 1.0, 1.0, 1.0, 1.0};
+    unsigned pos = 31u;
+    if constexpr (p > 0) {
+      const double *tab = p == 1 ? geo.xeH : (p == 2 ? geo.xm : geo.xp);
+      pos = 0u;
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      if (a == 0 && b == 0) continue;
-      const int wi = bi[a], wj = bj[b];
-      if (wi < 0 || wj < 0) continue;
-      const int64_t nd = int64_t(wj) * cv.pitch + wi;
-#pragma unroll
-      for (int q = 0; q < 9; ++q) G[q] += Gplanes[q * cv.plane + nd];
-      any = true;
+      for (int o = -2; o <= 2; ++o) {
+        const double v = tab[g.ix + ((g.xin >> (o + 2)) & 1u ? o : 0)];
+        const bool neg = negative(v);
+        pos |= (p == 2 ? !neg : neg) ? 1u << (o + 2) : 0u;
+        m[o + 2] = fabs(v);
+      }
     }
-  if (!any) return;
-  const int64_t node = int64_t(j) * cv.pitch + i;
-  double F[9];
-#pragma unroll
-  for (int q = 0; q < 9; ++q) F[q] = Fplanes[q * cv.plane + node];
-  nee_T(G, F, cv);
-#pragma unroll
-  for (int q = 0; q < 9; ++q) out[q] += G[q];
+    auto one = [&](auto qc, unsigned side) {
+      constexpr int q = decltype(qc)::value;
+      const double *G = g.G + q * g.plane;
+      double r = out[q];
+      if constexpr (p > 0) {
+        constexpr bool epos = q == 2 || q == 5 || q == 6;
+        r = line_T<true>(G, g.pitch, epos ? 31u : 0u, g.ein, g.elo, g.ehi, m, mixe, r);
+      }
+      out[q] = fma(-g.A, line_T<p == 0>(G, 1, side, g.xin, g.xlo, g.xhi, m, mix, 0.0), r);
+    };
+    one(Const<q0>(), pos);
+    one(Const<q1>(), ~pos);
+  };
+  pair(Const<0>()), pair(Const<1>()), pair(Const<2>()), pair(Const<3>());
 }
 
-__device__ __forceinline__ void tile_sum3(double a, double b, double c, double *ppart, int slot) {
-  __shared__ double sh[TILE_X * TILE_Y / 32][3];
-  const int lane = threadIdx.x + threadIdx.y * blockDim.x;
-  const int w = lane >> 5, l = lane & 31;
-  double v[3] = {a, b, c};
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-  if (l == 0)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) sh[w][k] = v[k];
-  __syncthreads();
-  if (lane < 3) {
-    double acc = 0.0;
-    for (int k = 0; k < TILE_X * TILE_Y / 32; ++k) acc += sh[k][lane];
-    ppart[int64_t(blockIdx.x) * 12 + slot * 3 + lane] = acc;
-  }
+// Theta partial of an interior node: sum_q Gb_q dc_{q xi}/dtheta D_xi F_q times
+// dt / (2 dxi). With A = c xi_x and x_xi = L + 2 H cot eta, x_eta = H cot (2 xi - 1),
+// dc_{q xi}/dtheta = e_y t1 - e_x t2, t2 = A 2 H eta xi_x dcot, t1 = t2 x_eta/H -
+// A (2 xi - 1) dcot.
+__device__ __forceinline__ double theta_partial(const CavDev &cv, const Geo &geo, const Mix64 &mix,
+                                                int i, int j, const double *Gb, const double *F) {
+  const double xe = geo.xeH[cv.goff + i];
+  const double t2 = geo.ath2[cv.goff + j];
+  const double t1 = fma(t2, xe, -geo.ath1[cv.goff + j] * geo.z[cv.goff + i]);
+  const int64_t plane = cv.plane;
+  const bool clo = i == 1, chi = i == cv.nx - 2;
+  // k: dc/dtheta of the pair's first member; pos0, pos1: c >= 0 of either (both at c = 0)
+  auto term = [&](int q0, bool pos0, bool pos1, double k, double r) {
+    const double *F0 = F + q0 * plane, *F1 = F0 + 2 * plane;
+    const double a = mix64(F0, pos0 ? 1 : -1, pos0 ? clo : chi, mix, F0[0], 0.0, true);
+    const double b = mix64(F1, pos1 ? 1 : -1, pos1 ? clo : chi, mix, F1[0], 0.0, true);
+    const double g0 = Gb[q0 * plane], g1 = Gb[(q0 + 2) * plane];
+    return fma(fma(pos0 ? g0 : -g0, a, (pos1 ? -g1 : g1) * b), k, r);
+  };
+  const double xm = geo.xm[cv.goff + i], xp = geo.xp[cv.goff + i];
+  double r = term(1, true, false, -t2, 0.0);
+  r = term(2, nonpositive(xe), nonnegative(xe), t1, r);
+  r = term(5, nonnegative(xm), nonpositive(xm), t1 - t2, r);
+  return term(6, nonpositive(xp), nonnegative(xp), t1 + t2, r);
 }
 
 }  // namespace
@@ -257,7 +331,8 @@ __global__ void k_adj_seed_energy(AdjArgs a) {
     const double dJ = 2.0 * cv.H * cv.H * (r.j * cv.deta) * cv.dcot;
     dth = 0.5 * wx * wy * dJ * (ux * ux + uy * uy);
   }
-  tile_sum3(0.0, 0.0, dth, a.ppart, 3);
+  double v[3] = {0.0, 0.0, dth};
+  block_sum<3, TILE_X * TILE_Y / 32>(v, a.ppart, blockIdx.x);
 }
 
 // Seed of J = sum over cavities of psi(i*, j*), the stream function at one
@@ -290,279 +365,255 @@ __global__ void k_adj_seed_psi(AdjArgs a) {
       dth = -w * uy * cv.H * (2.0 * r.i * cv.dxi - 1.0) * cv.dcot;
     }
   }
-  tile_sum3(0.0, 0.0, dth, a.ppart, 3);
+  double v[3] = {0.0, 0.0, dth};
+  block_sum<3, TILE_X * TILE_Y / 32>(v, a.ppart, blockIdx.x);
 }
 
-// A3 walls: adjoint of g_{n+1} at interior nodes next to walls += X^T(walls).
-__global__ void k_adj3_walls(AdjArgs a) {
-  const Ref r = tile_ref(a.tile_cav, a.cav);
+// Threads per block NT and registers as in staged64.cu: up to 255 registers on
+// small batches (8 blocks of a warp on an SM; 10, 12 and 14 blocks with fewer
+// registers ran at 0.96-1.04 of its speed), 168 with 128 threads.
+template <int NT>
+constexpr int ADJ_BLOCKS = NT == 32 ? 8 : 3;
+
+// Ring nodes: Gbar += X^T(sum of the wall nodes' adjoints), at g_{n+1}.
+template <int NT>
+__global__ void __launch_bounds__(NT, ADJ_BLOCKS<NT>) k_adj_ring(AdjArgs a) {
+  const Node64 r = interior_node<NT>(a.ring_cav, a.cav, true);
+  const CavDev &cv = a.cav[r.cav];
+  const int64_t plane = cv.plane, b9 = 9 * cv.off, node = int64_t(r.j) * cv.pitch + r.i;
+  previous_done();
+  dependents_may_start();
   if (!r.valid) return;
-  const CavDev &cv = a.cav[r.cav];
-  if (!interior(cv, r.i, r.j)) return;
-  if (!(r.i == 1 || r.j == 1 || r.i == cv.nx - 2 || r.j == cv.ny - 2)) return;
-  double *ag = a.adj_g + 9 * cv.off;
-  double add[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  wall_gather_T(cv, ag, a.gn + 9 * cv.off, r.i, r.j, add);
-  const int64_t node = int64_t(r.j) * cv.pitch + r.i;
-#pragma unroll
-  for (int q = 0; q < 9; ++q) a.fbarb[q * cv.plane + node + 9 * cv.off] = add[q];
-}
-
-// Applies the wall additions of k_adj3_walls (kept apart so that no thread
-// reads a wall adjoint another thread has changed).
-__global__ void k_adj_add(AdjArgs a, int which) {
-  const Ref r = tile_ref(a.tile_cav, a.cav);
-  if (!r.valid) return;
-  const CavDev &cv = a.cav[r.cav];
-  if (!interior(cv, r.i, r.j)) return;
-  if (!(r.i == 1 || r.j == 1 || r.i == cv.nx - 2 || r.j == cv.ny - 2)) return;
-  const int64_t node = int64_t(r.j) * cv.pitch + r.i;
-  double *dst = (which == 0 ? a.adj_g : a.fhb) + 9 * cv.off;
-  const double *add = a.fbarb + 9 * cv.off;
-#pragma unroll
-  for (int q = 0; q < 9; ++q) dst[q * cv.plane + node] += add[q * cv.plane + node];
-}
-
-// A3 stencil: FHbar(y) = -dt A^T(Gbar') for every node; theta partial (slot 0).
-__global__ void k_adj3_stencil(AdjArgs a) {
-  const Ref r = tile_ref(a.tile_cav, a.cav);
-  const CavDev &cv = a.cav[r.cav];
-  double dth = 0.0;
-  if (r.valid) {
-    const int64_t node = int64_t(r.j) * cv.pitch + r.i;
-    const double *ag = a.adj_g + 9 * cv.off;
-    const double *fh = a.fh + 9 * cv.off;
-    double *fhb = a.fhb + 9 * cv.off;
-    fhb[node] = 0.0;
-    const Blend bl = make_blend(cv.eta_b);
-#pragma unroll
-    for (int q = 1; q < 9; ++q)
-      fhb[q * cv.plane + node] = -cv.dt * advect_T(cv, a.geo, ag + q * cv.plane, q, r.i, r.j, bl);
-    if (interior(cv, r.i, r.j)) {
-      const NodeXi nm = node_xi(cv, a.geo, r.i, r.j);
-#pragma unroll
-      for (int q = 1; q < 9; ++q) {
-        const double gb = ag[q * cv.plane + node];
-        dth += -cv.dt * gb * nm.dcxi(q) * dxi_with(cv, fh + q * cv.plane, nm.cxi(q), r.i, r.j);
-      }
-    }
-  }
-  tile_sum3(0.0, 0.0, dth, a.ppart, 0);
-}
-
-// A2 walls: FHbar at interior nodes next to walls += X^T(FHbar at walls).
-__global__ void k_adj2_walls(AdjArgs a) {
-  const Ref r = tile_ref(a.tile_cav, a.cav);
-  if (!r.valid) return;
-  const CavDev &cv = a.cav[r.cav];
-  if (!interior(cv, r.i, r.j)) return;
-  if (!(r.i == 1 || r.j == 1 || r.i == cv.nx - 2 || r.j == cv.ny - 2)) return;
-  double add[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  wall_gather_T(cv, a.fhb + 9 * cv.off, a.fh + 9 * cv.off, r.i, r.j, add);
-  const int64_t node = int64_t(r.j) * cv.pitch + r.i;
-#pragma unroll
-  for (int q = 0; q < 9; ++q) a.fbarb[q * cv.plane + node + 9 * cv.off] = add[q];
-}
-
-// A2 pointwise at interior x: FBARbar = ah FHbar + M^T E^T (bh FHbar); lambda-bar of K2.
-__global__ void k_adj2_point(AdjArgs a) {
-  const Ref r = tile_ref(a.tile_cav, a.cav);
-  if (!r.valid) return;
-  const CavDev &cv = a.cav[r.cav];
-  const int64_t node = int64_t(r.j) * cv.pitch + r.i;
-  double *fbarb = a.fbarb + 9 * cv.off;
-  if (!interior(cv, r.i, r.j)) {
-#pragma unroll
-    for (int q = 0; q < 9; ++q) fbarb[q * cv.plane + node] = 0.0;
-    a.lamb2[cv.off + node] = 0.0;
-    return;
-  }
-  const double *fh = a.fh + 9 * cv.off;
-  const double *fhb = a.fhb + 9 * cv.off;
-  const double lam = a.lam[cv.off + node];
-  // f-bar(t + dt/2) of the node from the stored f(t + dt/2): Eq. (2.17),
-  // f = f-bar + bh (f^eq - f-bar), keeps u and P, so f^eq is that of f and
-  // f-bar = (f - bh f^eq) / ah, pointwise (no second evaluation of the
-  // half step's stencil)
-  double fhv[9];
-#pragma unroll
-  for (int q = 0; q < 9; ++q) fhv[q] = fh[q * cv.plane + node];
-  double ux, uy, P;
-  moments(fhv, cv.c, cv.cs2, ux, uy, P);
-  double geq[9];
-  equilibrium(P, ux, uy, cv.c, cv.inv_cs2, geq);
-  const double i4 = 1.0 / (4.0 * lam + cv.dt);
-  const double ah = 4.0 * lam * i4, bh = cv.dt * i4;
-  const double iah = (4.0 * lam + cv.dt) / (4.0 * lam);  // 1 / ah
-  double fbar[9];
-#pragma unroll
-  for (int q = 0; q < 9; ++q) fbar[q] = (fhv[q] - bh * geq[q]) * iah;
-  double hb[9], eb[9], out[9];
-  double lb = 0.0;
+  double *ag = a.adj_g + b9;
+  const double *gn = a.gn + b9 + node;
+  double w[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, h[9], F[9];
 #pragma unroll
   for (int q = 0; q < 9; ++q) {
-    hb[q] = fhb[q * cv.plane + node];
-    eb[q] = bh * hb[q];
-    out[q] = ah * hb[q];
-    lb += hb[q] * (fbar[q] - geq[q]);
+    F[q] = gn[q * plane];
+    h[q] = ag[q * plane + node];
   }
-  double ub, vb, Pb;
-  equilibrium_T(eb, ux, uy, cv, ub, vb, Pb);
-  moments_T(ub, vb, Pb, ux, uy, cv, out);
+  for (int k = 0; k < 3; ++k) {
+    int wi, wj;
+    if (!wall_of(cv, r.i, r.j, k, wi, wj)) continue;
+    const double *wn = ag + int64_t(wj) * cv.pitch + wi;
 #pragma unroll
-  for (int q = 0; q < 9; ++q) fbarb[q * cv.plane + node] = out[q];
-  a.lamb2[cv.off + node] = 4.0 * cv.dt * i4 * i4 * lb;  // d ah / d lam = -d bh / d lam
+    for (int q = 0; q < 9; ++q) w[q] += wn[q * plane];
+  }
+  const Mom64 m = moments64(F);
+  wall_T(h, w, m.x, m.y);
+#pragma unroll
+  for (int q = 0; q < 9; ++q) ag[q * plane + node] = h[q];
 }
 
-// A2 stencil: FBbar(y) = FBARbar(y) - dt/2 A^T(FBARbar); theta partial (slot 1).
-__global__ void k_adj2_stencil(AdjArgs a) {
-  const Ref r = tile_ref(a.tile_cav, a.cav);
+// The full step's stencil and the half step's collision (interior nodes; the
+// walls' FBARbar is zero and is not written).
+template <int NT>
+__global__ void __launch_bounds__(NT, ADJ_BLOCKS<NT>) k_adj_full(AdjArgs a) {
+  const Node64 r = interior_node<NT>(a.adj_cav, a.cav, false);
   const CavDev &cv = a.cav[r.cav];
-  double dth = 0.0;
+  const int64_t plane = cv.plane, off = cv.off, b9 = 9 * off;
+  const int i = min(r.i, cv.nx - 2), j = min(r.j, cv.ny - 2);
+  const int64_t node = int64_t(j) * cv.pitch + i;
+  const Mix64 mix = cv.mix, mixe = cv.mixe[1];
+  const double dt = cv.dt;
+  previous_done();
+  dependents_may_start();
+  double dth[1] = {0.0};
   if (r.valid) {
-    const int64_t node = int64_t(r.j) * cv.pitch + r.i;
-    const double *fbarb = a.fbarb + 9 * cv.off;
-    const double *fb = a.fb + 9 * cv.off;
-    double *fbb = a.fbb + 9 * cv.off;
-    const double hdt = 0.5 * cv.dt;
-    fbb[node] = fbarb[node];
-    const Blend bl = make_blend(cv.eta_b);
+    const double *ag = a.adj_g + b9, *fh = a.fh + b9 + node;
+    double f[9];
 #pragma unroll
-    for (int q = 1; q < 9; ++q)
-      fbb[q * cv.plane + node] = fbarb[q * cv.plane + node] -
-                                 hdt * advect_T(cv, a.geo, fbarb + q * cv.plane, q, r.i, r.j, bl);
-    if (interior(cv, r.i, r.j)) {
-      const NodeXi nm = node_xi(cv, a.geo, r.i, r.j);
+    for (int q = 0; q < 9; ++q) f[q] = fh[q * plane];
+    const Mom64 m = moments64(f);                  // those of f-bar too (Eq. 2.17)
+    // FHbar of the node (the rest plane is not advected); for a ring node then the
+    // sum of its wall nodes' and their transposed wall rule
+    double h[9], w[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll 1
+    for (int k = -1; k < (r.wall ? 3 : 0); ++k) {
+      int gi = i, gj = j;
+      if (k >= 0 && !wall_of(cv, i, j, k, gi, gj)) continue;
+      Gather64 g = gather_at(cv, a.geo, 1, gi, gj);
+      g.G = ag + int64_t(gj) * cv.pitch + gi;
+      advect_T(g, a.geo, mix, mixe, w);
+      if (k < 0)
 #pragma unroll
-      for (int q = 1; q < 9; ++q)
-        dth += -hdt * fbarb[q * cv.plane + node] * nm.dcxi(q) *
-               dxi_with(cv, fb + q * cv.plane, nm.cxi(q), r.i, r.j);
+        for (int q = 0; q < 9; ++q) {
+          h[q] = w[q];
+          w[q] = 0.0;
+        }
     }
+    if (r.wall) wall_T(h, w, m.x, m.y);
+    // Eq. (2.17): f = ah f-bar + bh f^eq keeps u and P, so f^eq is that of f and
+    // f-bar - f^eq = (f - f^eq) / ah; d ah / d lam = -d bh / d lam = 4 dt / (4 lam + dt)^2
+    double geq[9], out[9];
+    equilibrium64(m, geq);
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) s = fma(h[q], f[q] - geq[q], s);
+    const double lam = a.lam[off + node];
+    const double bh = dt * recip(fma(4.0, lam, dt));
+    a.lamb2[off + node] = bh * recip(lam) * s;
+    Adj64 b = equilibrium_T(h, m.x, m.y);
+    b.x *= bh;
+    b.y *= bh;
+    b.p *= bh;
+    moments_T(b, m.x, m.y, 1.0 - bh, h, out);
+    double *fbarb = a.fbarb + b9 + node;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) fbarb[q * plane] = out[q];
+    dth[0] = -theta_partial(cv, a.geo, mix, i, j, ag + node, fh);
   }
-  tile_sum3(0.0, 0.0, dth, a.ppart, 1);
+  block_sum<1, NT / 32>(dth, a.pfull, blockIdx.x);
 }
 
-// A1 pointwise: adjoint of (g_n, lambda_n); n and Re partials (slot 2).
-__global__ void k_adj1(AdjArgs a) {
-  const Ref r = tile_ref(a.tile_cav, a.cav);
+// The half step's stencil and the collision: the adjoint of (g_n, lambda_n).
+template <int NT>
+__global__ void __launch_bounds__(NT, ADJ_BLOCKS<NT>) k_adj_half(AdjArgs a) {
+  const Node64 r = node_of<NT>(a.blk_cav, a.cav);
   const CavDev &cv = a.cav[r.cav];
-  double dn = 0.0, dRe = 0.0;
+  const int64_t plane = cv.plane, off = cv.off, b9 = 9 * off;
+  const int i = min(r.i, cv.nx - 1), j = min(r.j, cv.ny - 1);
+  const int64_t node = int64_t(j) * cv.pitch + i;
+  const Mix64 mix = cv.mix, mixe = cv.mixe[0];
+  Gather64 gt = gather_at(cv, a.geo, 0, i, j);
+  const double dt = cv.dt;
+  previous_done();
+  dependents_may_start();
+  double v[3] = {0.0, 0.0, 0.0};  // n, Re, theta
   if (r.valid) {
-    const int64_t node = int64_t(r.j) * cv.pitch + r.i;
-    const double *g = a.g + 9 * cv.off;
-    double gg[9];
+    const double *fbarb = a.fbarb + b9 + node;
+    double *ag = a.adj_g + b9 + node;
+    gt.G = fbarb;
+    double B[9], P[9], d[9];      // FBbar, FPbar (f-hat^+ is read at interior nodes only)
 #pragma unroll
-    for (int q = 0; q < 9; ++q) gg[q] = g[q * cv.plane + node];
-    const double lam_p = a.lam_p[cv.off + node];
-    const double lam = a.lam[cv.off + node];
-    double ux, uy, P;
-    moments(gg, cv.c, cv.cs2, ux, uy, P);
-    double geq[9], d[9];
-    equilibrium(P, ux, uy, cv.c, cv.inv_cs2, geq);
+    for (int q = 0; q < 9; ++q) B[q] = r.wall ? 0.0 : fbarb[q * plane];
+    advect_T(gt, a.geo, mix, mixe, B);
+    const double *gp = a.g + b9 + node;
+    double g[9];
 #pragma unroll
-    for (int q = 0; q < 9; ++q) d[q] = gg[q] - geq[q];
-    double pxx, pxy, pyy;
-    second_moments(d, cv.c, pxx, pxy, pyy);
-    const double D = 2.0 * lam_p + cv.dt;
-    const double k = -2.0 / (D * cv.cs2);
-    const double pp = pxx * pxx + 2.0 * pxy * pxy + pyy * pyy;
-    const double q = 0.5 * k * k * pp;
-    const bool free = q > cv.gmin2;
-    const double qc = free ? q : cv.gmin2;
-
-    const bool in = interior(cv, r.i, r.j);
-    double *ag = a.adj_g + 9 * cv.off;
-    const double *fbb = a.fbb + 9 * cv.off;
-    double pb[9], bb_[9];
-#pragma unroll
-    for (int qq = 0; qq < 9; ++qq) {
-      pb[qq] = in ? ag[qq * cv.plane + node] : 0.0;   // FPbar (FP is read at interior nodes only)
-      bb_[qq] = fbb[qq * cv.plane + node];
+    for (int q = 0; q < 9; ++q) {
+      P[q] = r.wall ? 0.0 : ag[q * plane];
+      g[q] = gp[q * plane];
     }
-    const double i2 = 1.0 / (2.0 * lam + cv.dt);
-    const double ap = (2.0 * lam - cv.dt) * i2, bp = 2.0 * cv.dt * i2;
-    const double ab = (4.0 * lam - cv.dt) * 0.5 * i2, bb = 3.0 * cv.dt * 0.5 * i2;
-    double sP = 0.0, sB = 0.0;
+    const Mom64 m = moments64(g);
+    equilibrium64(m, d);
 #pragma unroll
-    for (int qq = 0; qq < 9; ++qq) {
-      sP += pb[qq] * d[qq];
-      sB += bb_[qq] * d[qq];
+    for (int q = 0; q < 9; ++q) d[q] = g[q] - d[q];
+    const double diag = (d[5] + d[6]) + (d[7] + d[8]);
+    const double pxx = (d[1] + d[3]) + diag, pyy = (d[2] + d[4]) + diag;
+    const double pxy = (d[5] - d[6]) + (d[7] - d[8]);
+    const double pp = fma(pxx, pxx, fma(pyy, pyy, (pxy + pxy) * pxy));
+    const double rD = recip(fma(2.0, a.lam_p[off + node], dt));
+    const double q = cv.strain2 * pp * (rD * rD);       // |gamma-dot|^2 (k_collide64)
+    const bool free = __double_as_longlong(q) > __double_as_longlong(cv.gmin2);
+    const double lam = a.lam[off + node];
+    const double i2 = recip(fma(2.0, lam, dt));
+    const double bp = 2.0 * dt * i2, bb = 0.75 * bp;    // Eqs. (2.15)-(2.16)
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) s = fma(fma(4.0, P[k], 3.0 * B[k]), d[k], s);
+    const double lb = a.adj_lam[off + node] + (r.wall ? 0.0 : a.lamb2[off + node]) +
+                      dt * (i2 * i2) * s;
+    // lam = K/c_s^2 max(q, gmin2)^m, m = (n-1)/2, K = U^(2-n) H^n / Re
+    const double ll = lb * lam;
+    v[0] = ll * fma(0.34657359027997265471, log2_fast(free ? q : cv.gmin2, a.powtab), cv.lnHU);
+    v[1] = -ll * cv.inv_Re;
+    // d lam / d q = m lam / q, q = strain2 pp / (2 lam_p + dt)^2
+    const double lm = free ? ll * cv.half_nm1 : 0.0;
+    const double e = free ? 2.0 * lm * recip(pp) : 0.0;
+    const double xx = e * pxx, yy = e * pyy, xy = 2.0 * e * pxy, t = xx + yy;
+    const double db[9] = {0.0, xx, yy, xx, yy, t + xy, t - xy, t + xy, t - xy};
+    double gb[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const double eb = fma(bp, P[k], bb * B[k]) - db[k];   // f^eq's adjoint
+      gb[k] = (P[k] + B[k]) - eb;
+      d[k] = eb;
     }
-    double lb = a.adj_lam[cv.off + node] + a.lamb2[cv.off + node] + 4.0 * cv.dt * i2 * i2 * sP +
-                3.0 * cv.dt * i2 * i2 * sB;
-    // lam = K/c_s^2 qc^m, m = (n-1)/2, K = U^(2-n) H^n / Re
-    dn = lb * lam * (cv.lnHU + 0.5 * log(qc));
-    dRe = -lb * lam / cv.Re;
-    const double qb = free ? lb * cv.half_nm1 * lam / q : 0.0;
-    const double k2 = k * k;
-    const double pxxb = qb * k2 * pxx, pxyb = qb * k2 * 2.0 * pxy, pyyb = qb * k2 * pyy;
-    const double kb = qb * k * pp;
-    const double lam_pb = kb * 4.0 / (D * D * cv.cs2);
-    const double c2 = cv.c * cv.c;
-    double gb[9], geqb[9];
+    const Adj64 b = equilibrium_T(d, m.x, m.y);
+    double out[9];
+    moments_T(b, m.x, m.y, 1.0, gb, out);
 #pragma unroll
-    for (int qq = 0; qq < 9; ++qq) {
-      const double db = c2 * (ex(qq) * ex(qq) * pxxb + ex(qq) * ey(qq) * pxyb + ey(qq) * ey(qq) * pyyb);
-      gb[qq] = ap * pb[qq] + ab * bb_[qq] + db;
-      geqb[qq] = bp * pb[qq] + bb * bb_[qq] - db;
-    }
-    double ub, vb, Pb;
-    equilibrium_T(geqb, ux, uy, cv, ub, vb, Pb);
-    moments_T(ub, vb, Pb, ux, uy, cv, gb);
-#pragma unroll
-    for (int qq = 0; qq < 9; ++qq) ag[qq * cv.plane + node] = gb[qq];
-    a.adj_lam[cv.off + node] = lam_pb;
+    for (int k = 0; k < 9; ++k) ag[k * plane] = out[k];
+    a.adj_lam[off + node] = -4.0 * lm * rD;
+    if (!r.wall) v[2] = -0.5 * theta_partial(cv, a.geo, mix, i, j, fbarb, a.fb + b9 + node);
   }
-  tile_sum3(dn, dRe, 0.0, a.ppart, 2);
+  block_sum<3, NT / 32>(v, a.phalf, blockIdx.x);
 }
 
-// Per cavity: dparams[cav][0..2] += sums over its tiles of the four slots.
-__global__ void k_adj_reduce(const CavDev *cavs, const double *ppart, double *dparams) {
-  const CavDev &cv = cavs[blockIdx.x];
-  __shared__ double sh[128][3];
-  double acc[3] = {0, 0, 0};
-  for (int t = threadIdx.x; t < cv.tiles_x * cv.tiles_y; t += blockDim.x)
-    for (int s = 0; s < 4; ++s)
+// Per cavity, by a cluster of CS blocks (k_residual_reduce): dparams[cav][0..2]
+// += the sums of n3 triples of p3 and, for theta, of n1 values of p1, in a
+// fixed order.
+template <int CS>
+__device__ __forceinline__ void reduce_params(const double *p3, int n3, const double *p1, int n1,
+                                              double *dparams) {
+  __shared__ double all[CS][3];
+  const int r = blockIdx.x % CS;
+  auto from = [&](int n, int b) { return int(int64_t(n) * b / CS); };
+  double v[8] = {};
+#pragma unroll 2
+  for (int t = from(n3, r) + threadIdx.x; t < from(n3, r + 1); t += 256)
 #pragma unroll
-      for (int k = 0; k < 3; ++k) acc[k] += ppart[int64_t(cv.tile0 + t) * 12 + s * 3 + k];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) sh[threadIdx.x][k] = acc[k];
+    for (int k = 0; k < 3; ++k) v[k] += p3[3 * int64_t(t) + k];
+#pragma unroll 2
+  for (int t = from(n1, r) + threadIdx.x; t < from(n1, r + 1); t += 256) v[2] += p1[t];
+  __shared__ double sh[8][3];
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const double s = warp_sums8(v);
+  if ((l & 3) == 0 && l < 12) sh[w][l >> 2] = s;
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) sh[threadIdx.x][k] += sh[threadIdx.x + w][k];
-    __syncthreads();
+  if (threadIdx.x < 3) {
+    double acc = 0.0;
+    for (int k = 0; k < 8; ++k) acc += sh[k][threadIdx.x];
+    cluster_at<CS>(&all[r][0])[threadIdx.x] = acc;
   }
-  if (threadIdx.x < 3) dparams[3 * blockIdx.x + threadIdx.x] += sh[0][threadIdx.x];
+  cluster_done<CS>();
+  if (r == 0 && threadIdx.x < 3) {
+    double acc = 0.0;
+    for (int b = 0; b < CS; ++b) acc += all[b][threadIdx.x];
+    dparams[threadIdx.x] += acc;
+  }
+}
+__global__ void __launch_bounds__(256) k_adj_reduce_seed(AdjArgs a) {
+  const CavDev &cv = a.cav[blockIdx.x];
+  reduce_params<1>(a.ppart + 3 * int64_t(cv.tile0), cv.tiles_x * cv.tiles_y, nullptr, 0,
+                   a.dparams + 3 * blockIdx.x);
+}
+template <int CS>
+__global__ void __launch_bounds__(256) k_adj_reduce(AdjArgs a) {
+  const CavDev &cv = a.cav[blockIdx.x / CS];
+  previous_done();
+  dependents_may_start();
+  reduce_params<CS>(a.phalf + 3 * int64_t(cv.blk0), cv.nblk, a.pfull + cv.adj0, cv.nblk_adj,
+                    a.dparams + 3 * (blockIdx.x / CS));
 }
 
 static const dim3 kT(TILE_X, TILE_Y);
 
-void launch_adjoint_seed(const AdjArgs &a, int ntiles, int ncav, double *dparams, cudaStream_t s) {
-  cudaMemsetAsync(a.ppart, 0, size_t(ntiles) * 12 * sizeof(double), s);
-  k_adj_seed_energy<<<ntiles, kT, 0, s>>>(a);
-  k_adj_reduce<<<ncav, 128, 0, s>>>(a.cav, a.ppart, dparams);
+void launch_adjoint_seed(const AdjArgs &a, cudaStream_t s) {
+  k_adj_seed_energy<<<a.ntiles, kT, 0, s>>>(a);
+  k_adj_reduce_seed<<<a.ncav, 256, 0, s>>>(a);
 }
 
-void launch_adjoint_seed_psi(const AdjArgs &a, int ntiles, int ncav, double *dparams,
-                             cudaStream_t s) {
-  cudaMemsetAsync(a.ppart, 0, size_t(ntiles) * 12 * sizeof(double), s);
-  k_adj_seed_psi<<<ntiles, kT, 0, s>>>(a);
-  k_adj_reduce<<<ncav, 128, 0, s>>>(a.cav, a.ppart, dparams);
+void launch_adjoint_seed_psi(const AdjArgs &a, cudaStream_t s) {
+  k_adj_seed_psi<<<a.ntiles, kT, 0, s>>>(a);
+  k_adj_reduce_seed<<<a.ncav, 256, 0, s>>>(a);
 }
 
-void launch_adjoint_step(const AdjArgs &a, int ntiles, int ncav, double *dparams, cudaStream_t s) {
-  cudaMemsetAsync(a.ppart, 0, size_t(ntiles) * 12 * sizeof(double), s);
-  k_adj3_walls<<<ntiles, kT, 0, s>>>(a);
-  k_adj_add<<<ntiles, kT, 0, s>>>(a, 0);
-  k_adj3_stencil<<<ntiles, kT, 0, s>>>(a);
-  k_adj2_walls<<<ntiles, kT, 0, s>>>(a);
-  k_adj_add<<<ntiles, kT, 0, s>>>(a, 1);
-  k_adj2_point<<<ntiles, kT, 0, s>>>(a);
-  k_adj2_stencil<<<ntiles, kT, 0, s>>>(a);
-  k_adj1<<<ntiles, kT, 0, s>>>(a);
-  k_adj_reduce<<<ncav, 128, 0, s>>>(a.cav, a.ppart, dparams);
+void launch_adjoint_step(const AdjArgs &a, cudaStream_t s) {
+  if (a.nt == 32) {
+    launch_after(k_adj_ring<32>, a.nblk_ring, 32, 0, s, a);
+    launch_after(k_adj_full<32>, a.nblk_adj, 32, 0, s, a);
+    launch_after(k_adj_half<32>, a.nblk, 32, 0, s, a);
+  } else {
+    launch_after(k_adj_ring<128>, a.nblk_ring, 128, 0, s, a);
+    launch_after(k_adj_full<128>, a.nblk_adj, 128, 0, s, a);
+    launch_after(k_adj_half<128>, a.nblk, 128, 0, s, a);
+  }
+  if (a.most > REDUCE_ONE)
+    launch_after(k_adj_reduce<REDUCE_CS>, a.ncav * REDUCE_CS, 256, 0, s, a, REDUCE_CS);
+  else
+    launch_after(k_adj_reduce<1>, a.ncav, 256, 0, s, a);
 }
 
 }  // namespace ifd

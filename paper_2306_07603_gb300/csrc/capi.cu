@@ -49,6 +49,7 @@ struct ifdlbm_ctx {
   int ntiles = 0;
   int nblk64 = 0;      // FP64 staged kernels: blocks per launch
   int nt64 = 128;      // ... and threads per block
+  int most_parts = 0;  // staged kernels: largest number of residual partials of a cavity
   int ntasks = 0;      // fused kernel tasks
   int fused_nt = 128;  // fused kernel threads per CTA
   int fused_rows = 0;  // rows per task (0: automatic)
@@ -61,9 +62,11 @@ struct ifdlbm_ctx {
   unsigned char *tmaps = nullptr;  // [2][ncav] TMA tensor maps of g[0], g[1] (fused kernel)
   int tma_skip = 0;                // test hook (ifdlbm_inject_tma_timeout)
   // adjoint scratch (allocated on the first adjoint call)
-  double *adj_g1 = nullptr, *adj_l1 = nullptr, *adj_fhb = nullptr, *adj_fbarb = nullptr,
-         *adj_fbb = nullptr, *adj_lamb2 = nullptr, *adj_ppart = nullptr;
+  double *adj_g1 = nullptr, *adj_l1 = nullptr, *adj_fbarb = nullptr, *adj_lamb2 = nullptr,
+         *adj_ppart = nullptr, *adj_pfull = nullptr, *adj_phalf = nullptr, *adj_tab = nullptr;
   int *adj_nodes = nullptr;  // [ncav][2] nodes of the psi objective
+  int *adj_blocks = nullptr;  // block -> cavity of the kernels over the interior and its ring
+  int nblk_adj = 0, nblk_ring = 0;
   int64_t total_plane = 0;
   int64_t geo_len = 0;
   int64_t max_n2 = 0;
@@ -244,7 +247,8 @@ void enqueue_step(ifdlbm_ctx *h, int parity, bool want_residual) {
   }
   if (want_residual)
     timed(h, IFDLBM_KPROF_REDUCE, [&] {
-      ifd::launch_residual_reduce(h->b.cav, h->b.part, h->b.resid, h->ncav, h->stream);
+      ifd::launch_residual_reduce(h->b.cav, h->b.part, h->b.resid, h->ncav, h->most_parts,
+                                  h->stream);
     });
 }
 
@@ -707,7 +711,7 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
       cv.dcot = -(M_PI / 180.0) / (sn * sn);
     }
     cv.lnHU = std::log(H) - std::log(s.U_lid);
-    cv.Re = s.Re;
+    cv.inv_Re = 1.0 / s.Re;
     cv.half_nm1 = 0.5 * cv.nm1;
     cv.Kics2 = cv.K / cv.cs2;
     {  // pow_tab: binomial coefficients of (1 + t)^m, m = (n - 1)/2, and the FP32 clamp
@@ -765,7 +769,9 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
   h->geo_len = goff;
   const bool staged64 = !fused && opt.precision == IFDLBM_FP64;
   std::vector<int> blk_cav;
+  for (const CavDev &cv : h->cav) h->most_parts = std::max(h->most_parts, cv.nparts);
   if (staged64) {
+    h->most_parts = 0;
     // Blocks of the FP64 staged kernels (node_of, step64.cuh): interior nodes,
     // then wall nodes of every cavity.
     int64_t nodes = 0;
@@ -778,8 +784,17 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
       cv.nblk_in = blocks(int64_t(cv.nx - 2) * (cv.ny - 2));
       cv.nblk = cv.nblk_in + blocks(2 * int64_t(cv.nx) + 2 * (cv.ny - 2));
       blk_cav.resize(blk_cav.size() + cv.nblk, k);
+      // adjoint: interior nodes away from the walls, then the ring next to them
+      const int nring = blocks(2 * int64_t(cv.nx - 2) + 2 * (cv.ny - 4));
+      cv.nblk_core = blocks(int64_t(cv.nx - 4) * (cv.ny - 4));
+      cv.nblk_adj = cv.nblk_core + nring;
+      cv.adj0 = h->nblk_adj;
+      cv.ring0 = h->nblk_ring;
+      h->nblk_adj += cv.nblk_adj;
+      h->nblk_ring += nring;
       cv.part0 = cv.blk0;
       cv.nparts = cv.nblk;
+      h->most_parts = std::max(h->most_parts, cv.nparts);
     }
     h->nblk64 = int(blk_cav.size());
   }
@@ -1255,13 +1270,10 @@ int ifdlbm_save_state_dev(ifdlbm_handle h, void *dst) {
   const size_t tsize = h->precision == IFDLBM_FP64 ? sizeof(double) : sizeof(float);
   const size_t gb = 9 * h->total_plane * tsize;
   const size_t lb = h->total_plane * tsize;
-  cudaError_t e = cudaMemcpyAsync(dst, h->b.g[h->cur], gb, cudaMemcpyDeviceToDevice, h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync((char *)dst + gb, h->b.lam[h->cur], lb, cudaMemcpyDeviceToDevice,
-                        h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync((char *)dst + gb + lb, h->b.pref, h->ncav * sizeof(double),
-                        cudaMemcpyDeviceToDevice, h->stream);
+  const cudaError_t e = ifd::launch_copy(
+      {{h->b.g[h->cur], h->b.lam[h->cur], h->b.pref},
+       {dst, (char *)dst + gb, (char *)dst + gb + lb},
+       {int64_t(gb), int64_t(lb), int64_t(h->ncav * sizeof(double))}}, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "save_state_dev");
   return IFDLBM_OK;
 }
@@ -1272,13 +1284,10 @@ int ifdlbm_load_state_dev(ifdlbm_handle h, const void *src) {
   const size_t tsize = h->precision == IFDLBM_FP64 ? sizeof(double) : sizeof(float);
   const size_t gb = 9 * h->total_plane * tsize;
   const size_t lb = h->total_plane * tsize;
-  cudaError_t e = cudaMemcpyAsync(h->b.g[h->cur], src, gb, cudaMemcpyDeviceToDevice, h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(h->b.lam[h->cur], (const char *)src + gb, lb, cudaMemcpyDeviceToDevice,
-                        h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(h->b.pref, (const char *)src + gb + lb, h->ncav * sizeof(double),
-                        cudaMemcpyDeviceToDevice, h->stream);
+  const cudaError_t e = ifd::launch_copy(
+      {{src, (const char *)src + gb, (const char *)src + gb + lb},
+       {h->b.g[h->cur], h->b.lam[h->cur], h->b.pref},
+       {int64_t(gb), int64_t(lb), int64_t(h->ncav * sizeof(double))}}, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "load_state_dev");
   return IFDLBM_OK;
 }
@@ -1337,43 +1346,97 @@ int adjoint_ready(ifdlbm_ctx *h) {
   if (h->opt.wall_pressure != IFDLBM_WALLP_ZEROTH)
     return fail(h, IFDLBM_ERR_INVALID_ARG, "adjoint: differentiates the zeroth-order wall pressure");
   if (h->adj_g1) return IFDLBM_OK;
-  const size_t P = size_t(h->total_plane) * sizeof(double);
+  const size_t P = size_t(h->total_plane) * sizeof(double), GL = size_t(h->geo_len);
   bool ok = true;
-  ok &= (h->adj_g1 = (double *)dalloc(h, 9 * P)) != nullptr;
+  double *g1 = nullptr;
+  ok &= (g1 = (double *)dalloc(h, 9 * P)) != nullptr;
   ok &= (h->adj_l1 = (double *)dalloc(h, P)) != nullptr;
-  ok &= (h->adj_fhb = (double *)dalloc(h, 9 * P)) != nullptr;
   ok &= (h->adj_fbarb = (double *)dalloc(h, 9 * P)) != nullptr;
-  ok &= (h->adj_fbb = (double *)dalloc(h, 9 * P)) != nullptr;
   ok &= (h->adj_lamb2 = (double *)dalloc(h, P)) != nullptr;
-  ok &= (h->adj_ppart = (double *)dalloc(h, size_t(h->ntiles) * 12 * sizeof(double))) != nullptr;
+  ok &= (h->adj_ppart = (double *)dalloc(h, size_t(h->ntiles) * 3 * sizeof(double))) != nullptr;
+  ok &= (h->adj_pfull = (double *)dalloc(h, size_t(h->nblk_adj) * sizeof(double))) != nullptr;
+  ok &= (h->adj_phalf = (double *)dalloc(h, size_t(h->nblk64) * 3 * sizeof(double))) != nullptr;
   ok &= (h->adj_nodes = (int *)dalloc(h, size_t(h->ncav) * 2 * sizeof(int))) != nullptr;
+  ok &= (h->adj_blocks = (int *)dalloc(h, size_t(h->nblk_adj + h->nblk_ring) * sizeof(int))) !=
+        nullptr;
+  ok &= (h->adj_tab = (double *)dalloc(h, 5 * GL * sizeof(double))) != nullptr;
   if (!ok) return fail(h, IFDLBM_ERR_OOM, "adjoint: device allocation failed");
-  for (double *p : {h->adj_fhb, h->adj_fbarb, h->adj_fbb})
-    cudaMemsetAsync(p, 0, 9 * P, h->stream);
-  cudaMemsetAsync(h->adj_lamb2, 0, P, h->stream);
+  // column and row tables of the gathers and of the theta partial (Geo), and
+  // the block tables
+  std::vector<double> tab(5 * GL);
+  std::vector<int> blocks;
+  for (int k = 0; k < h->ncav; ++k) blocks.insert(blocks.end(), h->cav[k].nblk_adj, k);
+  for (int k = 0; k < h->ncav; ++k)
+    blocks.insert(blocks.end(), h->cav[k].nblk_adj - h->cav[k].nblk_core, k);
+  for (int k = 0; k < h->ncav; ++k) {
+    const CavDev &cv = h->cav[k];
+    const ifdlbm_geometry &gm = h->spec[k].geom;
+    const double ct = cot_deg(gm.theta_deg);
+    for (int i = 0; i < cv.nx; ++i) {
+      const double z = 2.0 * (double(i) / (cv.nx - 1)) - 1.0;
+      const double xe = gm.H * ct * z / gm.H;
+      tab[cv.goff + i] = 1.0 - xe;
+      tab[GL + cv.goff + i] = 1.0 + xe;
+      tab[2 * GL + cv.goff + i] = z;
+    }
+    for (int j = 0; j < cv.ny; ++j) {
+      const double eta = double(j) / (cv.ny - 1), xix = 1.0 / (gm.L + 2.0 * gm.H * ct * eta);
+      const double r = cv.sxi[1] * xix * cv.dcot;
+      tab[3 * GL + cv.goff + j] = r;
+      tab[4 * GL + cv.goff + j] = r * 2.0 * gm.H * eta * xix;
+    }
+  }
+  cudaError_t e = cudaMemcpyAsync(h->adj_tab, tab.data(), tab.size() * sizeof(double),
+                                  cudaMemcpyHostToDevice, h->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(h->adj_blocks, blocks.data(), blocks.size() * sizeof(int),
+                        cudaMemcpyHostToDevice, h->stream);
+  for (double *p : {g1, h->adj_fbarb})
+    if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, 9 * P, h->stream);
+  for (double *p : {h->adj_l1, h->adj_lamb2})
+    if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, P, h->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);  // the host tables go out of scope
+  if (e != cudaSuccess) return cuda_fail(h, e, "adjoint set-up");
+  h->b.geo.xm = h->adj_tab;
+  h->b.geo.xp = h->adj_tab + GL;
+  h->b.geo.z = h->adj_tab + 2 * GL;
+  h->b.geo.ath1 = h->adj_tab + 3 * GL;
+  h->b.geo.ath2 = h->adj_tab + 4 * GL;
+  h->adj_g1 = g1;
   return IFDLBM_OK;
 }
 
-ifd::AdjArgs adj_args(ifdlbm_ctx *h, const void *state, void *adj) {
+ifd::AdjArgs adj_args(ifdlbm_ctx *h, const void *state, void *adj, double *dparams) {
   ifd::AdjArgs a{};
   const int64_t n9 = 9 * h->total_plane;
   a.cav = h->b.cav;
   a.geo = h->b.geo;
   a.tile_cav = h->b.tile_cav;
+  a.blk_cav = h->b.blk_cav;
+  a.adj_cav = h->adj_blocks;
+  a.ring_cav = h->adj_blocks + h->nblk_adj;
   a.g = (const double *)state;
   a.lam_p = (const double *)state + n9;
   a.lam = h->adj_l1;
   a.fb = (const double *)h->b.fb;
-  a.fp = (const double *)h->b.fp;
   a.fh = (const double *)h->b.fh;
   a.gn = h->adj_g1;
   a.adj_g = (double *)adj;
   a.adj_lam = (double *)adj + n9;
-  a.fhb = h->adj_fhb;
   a.fbarb = h->adj_fbarb;
-  a.fbb = h->adj_fbb;
   a.lamb2 = h->adj_lamb2;
   a.ppart = h->adj_ppart;
+  a.pfull = h->adj_pfull;
+  a.phalf = h->adj_phalf;
+  a.dparams = dparams;
+  a.powtab = h->b.powtab;
+  a.ntiles = h->ntiles;
+  a.ncav = h->ncav;
+  a.nblk = h->nblk64;
+  a.nblk_adj = h->nblk_adj;
+  a.nblk_ring = h->nblk_ring;
+  a.nt = h->nt64;
+  a.most = h->most_parts;
   return a;
 }
 
@@ -1384,7 +1447,7 @@ int ifdlbm_adjoint_seed_energy(ifdlbm_handle h, const void *state, void *adj, do
   cudaSetDevice(h->device);
   int rc = adjoint_ready(h);
   if (rc) return rc;
-  ifd::launch_adjoint_seed(adj_args(h, state, adj), h->ntiles, h->ncav, dparams, h->stream);
+  ifd::launch_adjoint_seed(adj_args(h, state, adj, dparams), h->stream);
   g_launches += 2;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e, "adjoint seed");
@@ -1407,9 +1470,9 @@ int ifdlbm_adjoint_seed_psi(ifdlbm_handle h, const void *state, const int *nodes
   cudaError_t e = cudaMemcpyAsync(h->adj_nodes, nodes, size_t(h->ncav) * 2 * sizeof(int),
                                   cudaMemcpyHostToDevice, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "adjoint_seed_psi nodes");
-  ifd::AdjArgs a = adj_args(h, state, adj);
+  ifd::AdjArgs a = adj_args(h, state, adj, dparams);
   a.psi_nodes = h->adj_nodes;
-  ifd::launch_adjoint_seed_psi(a, h->ntiles, h->ncav, dparams, h->stream);
+  ifd::launch_adjoint_seed_psi(a, h->stream);
   g_launches += 2;
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e, "adjoint seed psi");
@@ -1444,8 +1507,8 @@ int ifdlbm_adjoint_step(ifdlbm_handle h, const void *state_n, void *adj, double 
   ifd::launch_collide64(f, h->nblk64, h->nt64, h->stream);
   ifd::launch_half64(f, h->nblk64, h->nt64, h->stream);
   ifd::launch_full64(f, h->nblk64, h->nt64, h->stream);
-  ifd::launch_adjoint_step(adj_args(h, state_n, adj), h->ntiles, h->ncav, dparams, h->stream);
-  g_launches += 3 + 9;
+  ifd::launch_adjoint_step(adj_args(h, state_n, adj, dparams), h->stream);
+  g_launches += 3 + 4;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e, "adjoint step");
   return IFDLBM_OK;
@@ -1464,11 +1527,10 @@ int ifdlbm_save_intermediates_dev(ifdlbm_handle h, void *dst) {
   if (rc) return rc;
   // the staged kernels' scratch planes hold the last step's f-bar^+, f-hat^+
   // and f(t + dt/2), in the order the adjoint reads them
-  const size_t P9 = 9 * size_t(h->total_plane) * sizeof(double);
-  cudaError_t e = cudaSuccess;
-  const void *src[3] = {h->b.fb, h->b.fp, h->b.fh};
-  for (int k = 0; k < 3 && e == cudaSuccess; ++k)
-    e = cudaMemcpyAsync((char *)dst + k * P9, src[k], P9, cudaMemcpyDeviceToDevice, h->stream);
+  const int64_t P9 = 9 * h->total_plane * int64_t(sizeof(double));
+  const cudaError_t e = ifd::launch_copy({{h->b.fb, h->b.fp, h->b.fh},
+                                          {dst, (char *)dst + P9, (char *)dst + 2 * P9},
+                                          {P9, P9, P9}}, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "save_intermediates_dev");
   return IFDLBM_OK;
 }
@@ -1483,14 +1545,13 @@ int ifdlbm_adjoint_step_saved(ifdlbm_handle h, const void *state_n, const void *
   // step n's outputs (state n + 1: its populations and lambda(t), which the
   // step stores as the next step's lagged value) and intermediates, as saved
   const int64_t n9 = 9 * h->total_plane;
-  ifd::AdjArgs a = adj_args(h, state_n, adj);
+  ifd::AdjArgs a = adj_args(h, state_n, adj, dparams);
   a.gn = (const double *)state_np1;
   a.lam = (const double *)state_np1 + n9;
-  a.fb = (const double *)inter;
-  a.fp = (const double *)inter + n9;
+  a.fb = (const double *)inter;            // (f-hat^+, the planes between, is not needed)
   a.fh = (const double *)inter + 2 * n9;
-  ifd::launch_adjoint_step(a, h->ntiles, h->ncav, dparams, h->stream);
-  g_launches += 9;
+  ifd::launch_adjoint_step(a, h->stream);
+  g_launches += 4;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e, "adjoint step (saved)");
   return IFDLBM_OK;

@@ -26,10 +26,9 @@ namespace ifd {
 // T_j = 2^(j/256).
 constexpr int POW_TABLE_SIZE = 3 * 256;
 
-__device__ __forceinline__ double pow_fast(double x, double m, const double *__restrict__ tab) {
+// log2 x for normal x > 0 (the first half of pow_fast).
+__device__ __forceinline__ double log2_fast(double x, const double *__restrict__ tab) {
   constexpr double K1 = 1.4426950408889634074;       // 1/ln 2
-  constexpr double LN2 = 0.69314718055994530942;
-  constexpr double MAGIC = 6755399441055744.0;       // 1.5 * 2^52
   // log2 x: x = 2^e f, f in [1, 2); j = top 8 bits of the fraction
   const int hi = __double2hiint(x), lo = __double2loint(x);
   const int e = ((hi >> 20) & 0x7FF) - 1023;
@@ -41,7 +40,13 @@ __device__ __forceinline__ double pow_fast(double x, double m, const double *__r
   const float tf = float(t);
   const float c32 = float(K1 / 3.0) + tf * (float(-K1 / 4.0) + tf * float(K1 / 5.0));
   s = fma(t2 * t, double(c32), s);                   // + t^3 (1/3 - t/4 + t^2/5)/ln2
-  const double lg = (double(e) + __ldg(tab + 256 + j)) + s;
+  return (double(e) + __ldg(tab + 256 + j)) + s;
+}
+
+__device__ __forceinline__ double pow_fast(double x, double m, const double *__restrict__ tab) {
+  constexpr double LN2 = 0.69314718055994530942;
+  constexpr double MAGIC = 6755399441055744.0;       // 1.5 * 2^52
+  const double lg = log2_fast(x, tab);
   // 2^y, y = m log2 x: N = round(256 y), r = y - N/256
   const double y = m * lg;
   const double v = fma(y, 256.0, MAGIC);

@@ -38,7 +38,7 @@ struct CavDev {
   double Kics2;             // K / c_s^2
   double dcot;              // d cot(theta) / d theta_deg (adjoint)
   double lnHU;              // ln H - ln U: d ln K / d n (adjoint)
-  double Re;                // Reynolds number (adjoint)
+  double inv_Re;            // 1 / Reynolds number (adjoint)
   int implicit;             // 1: lambda from the implicit form of Eq. (2.14), 0: lagged
   int general;              // 1: general quadrilateral, per-node metrics in Geo::gmet
   int pow32;                // FP32 storage only: 1 power law (and implicit solve) in FP32
@@ -54,6 +54,7 @@ struct CavDev {
   // of the mixed difference (xi, unscaled; eta of the trapezoid, times -scale
   // c / (2 deta H)) and scale c / (2 dxi), scale c / (2 deta)
   int blk0, nblk_in, nblk;
+  int adj0, nblk_core, nblk_adj, ring0;  // adjoint: blocks over the interior, over its ring
   Mix64 mix, mixe[2];
   double sxi[2], seta[2];
   double strain2;           // 2 c^4 / c_s^4: |gamma-dot|^2 = strain2 pp / (2 lam_prev + dt)^2
@@ -69,6 +70,9 @@ struct CavDev {
 struct Geo {
   const double *xix, *xeH, *xxi, *xeta;
   const double *ax[2];  // scale c xi_x(eta_j) / (2 dxi), scale = dt/2 and dt (FP64 staged kernels)
+  // adjoint: 1 - x_eta/H, 1 + x_eta/H and 2 xi - 1 per column; dt c xi_x dcot / (2 dxi) and
+  // that times 2 H eta xi_x per row (dcot = d cot(theta) / d theta_deg)
+  const double *xm, *xp, *z, *ath1, *ath2;
   const float *cxix_f, *jac_f;
   // general quadrilaterals (staged kernels): per node, at 7 * off + k * plane,
   // k = 0..6: xi_x, xi_y, eta_x, eta_y, x_eta, y_eta, J (Eqs. 3.2-3.3)
@@ -172,28 +176,47 @@ void launch_full(const StepArgs &a, int ntiles, cudaStream_t s);
 void launch_collide64(const StepArgs &a, int nblk, int nt, cudaStream_t s);
 void launch_half64(const StepArgs &a, int nblk, int nt, cudaStream_t s);
 void launch_full64(const StepArgs &a, int nblk, int nt, cudaStream_t s);
+// (most: the largest number of partials a cavity has; above REDUCE_ONE a cluster
+// of REDUCE_CS blocks reduces a cavity's, below it one block)
+constexpr int REDUCE_ONE = 512, REDUCE_CS = 8;
 void launch_residual_reduce(const CavDev *cav, const double *part, double *resid, int ncav,
-                            cudaStream_t s);
+                            int most, cudaStream_t s);
+
+// Device-to-device copies of up to three segments: one kernel while they are
+// small (COPY_MOST bytes in all), where the launches of three copies cost more
+// than the bytes.
+struct CopyArgs {
+  const void *src[3];
+  void *dst[3];
+  int64_t bytes[3];
+};
+constexpr int64_t COPY_MOST = int64_t(64) << 20;
+cudaError_t launch_copy(const CopyArgs &a, cudaStream_t s);
 
 // Discrete adjoint of one staged FP64 step (adjoint.cu). Buffers use the
 // state layout: 9 planes then 1 plane per cavity at the usual offsets.
 struct AdjArgs {
   const CavDev *cav;
   Geo geo;
-  const int *tile_cav;
+  const int *tile_cav;       // tiles of the seeds
+  const int *blk_cav, *adj_cav, *ring_cav;  // block -> cavity of the step's kernels
   const double *g, *lam_p;   // state n
   const double *lam;         // lambda(t) of step n (forward output)
-  const double *fb, *fp, *fh;  // forward intermediates of step n
+  const double *fb, *fh;     // forward intermediates of step n
   const double *gn;          // state n + 1 (forward output)
   double *adj_g, *adj_lam;   // in: adjoint of state n + 1; out: of state n
-  double *fhb, *fbarb, *fbb, *lamb2;  // adjoint scratch
-  double *ppart;             // [ntiles][4 slots][3] parameter partials
+  double *fbarb, *lamb2;     // adjoint scratch (zero at the wall nodes)
+  double *ppart;             // [ntiles][3] parameter partials of a seed
+  double *pfull, *phalf;     // [nblk_adj], [nblk][3] parameter partials of a step
+  double *dparams;           // [ncav][3]
+  const double *powtab;
   const int *psi_nodes;      // [ncav][2] (i, j) of the psi objective (seed_psi only)
+  int ntiles, ncav, nblk, nblk_adj, nblk_ring, nt;
+  int most;                  // largest number of blocks of a cavity (launch_residual_reduce)
 };
-void launch_adjoint_seed(const AdjArgs &a, int ntiles, int ncav, double *dparams, cudaStream_t s);
-void launch_adjoint_seed_psi(const AdjArgs &a, int ntiles, int ncav, double *dparams,
-                             cudaStream_t s);
-void launch_adjoint_step(const AdjArgs &a, int ntiles, int ncav, double *dparams, cudaStream_t s);
+void launch_adjoint_seed(const AdjArgs &a, cudaStream_t s);
+void launch_adjoint_seed_psi(const AdjArgs &a, cudaStream_t s);
+void launch_adjoint_step(const AdjArgs &a, cudaStream_t s);
 
 // Host-built tables of pow_fast and of pow_tab (capi.cu) and their self-tests (staged.cu)
 void fill_pow_tables(double *tab);

@@ -11,6 +11,7 @@
 // first access to memory that any kernel or copy of the stream writes (tables
 // uploaded at creation are not), and none returns before it.
 #pragma once
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 namespace ifd {
@@ -22,19 +23,39 @@ __device__ __forceinline__ void dependents_may_start() {
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
+// Address of p, in this block's shared memory, in that of the first block of the
+// cluster of CS blocks; and the barrier after which the first block reads what
+// the others wrote there.
+template <int CS>
+__device__ __forceinline__ double *cluster_at(double *p) {
+  if constexpr (CS == 1)
+    return p;
+  else
+    return cooperative_groups::this_cluster().map_shared_rank(p, 0);
+}
+template <int CS>
+__device__ __forceinline__ void cluster_done() {
+  if constexpr (CS == 1)
+    __syncthreads();
+  else
+    cooperative_groups::this_cluster().sync();
+}
+
 template <class Args>
 inline void launch_after(void (*kernel)(Args), int grid, int block, int smem, cudaStream_t s,
-                         const Args &args) {
+                         const Args &args, int cluster = 1) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(grid));
   cfg.blockDim = dim3(unsigned(block));
   cfg.dynamicSmemBytes = size_t(smem);
   cfg.stream = s;
-  cudaLaunchAttribute attr = {};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute attr[2] = {};
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim = {unsigned(cluster), 1, 1};
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   cudaLaunchKernelEx(&cfg, kernel, args);
 }
 

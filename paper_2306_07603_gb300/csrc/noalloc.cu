@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(kThreads)
 __global__ void __launch_bounds__(kThreads) k_field_reduce(const double *part, int nslots,
                                                            double *out) {
   __shared__ double res[4];
-  ifd::reduce_partials(part, nslots, res);
+  ifd::reduce_partials_block<kThreads / 32>(part, nslots, res);
   __syncthreads();
   if (threadIdx.x < 3) out[threadIdx.x] = res[threadIdx.x];
 }

@@ -14,13 +14,21 @@
 // ny-2)): the adjacent node along the grid normal on a side, the diagonal
 // node at a corner. The lid nodes 0 < i < nx-1 of row ny-1 move at (U, 0);
 // every other wall node, the two top corners included, is at rest.
+#include <algorithm>
 #include <cstdint>
 
 #include "d2q9.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "reduce.cuh"
 
 namespace ifd {
+
+struct ReduceArgs {
+  const CavDev *cav;
+  const double *part;
+  double *resid;
+};
 
 struct NodeRef {
   int cav, i, j;
@@ -309,10 +317,30 @@ __global__ void __launch_bounds__(TILE_X *TILE_Y) k_full(StepArgs a) {
   if (a.want_residual) block_partial<TILE_X * TILE_Y / 32>(p, a.part, blockIdx.x);
 }
 
-// One block per cavity: fixed-order reduction of that cavity's partials.
-__global__ void k_residual_reduce(const CavDev *cavs, const double *part, double *resid) {
-  const CavDev &cv = cavs[blockIdx.x];
-  reduce_partials(part + int64_t(cv.part0) * NPART, cv.nparts, resid + 4 * blockIdx.x);
+// A cluster of CS blocks per cavity: fixed-order reduction of that cavity's
+// partials, each block over a contiguous share of the slots, the last sums in
+// the first block's shared memory. One block takes 2.5 us of FP64 additions
+// alone for the 2065 slots of a 257^2 cavity (12 us in all); eight take an eighth.
+template <int CS>
+__global__ void __launch_bounds__(256) k_residual_reduce(ReduceArgs a) {
+  __shared__ double all[CS][7];
+  const int k = blockIdx.x / CS, r = blockIdx.x % CS;
+  const CavDev &cv = a.cav[k];
+  const int s0 = int(int64_t(cv.nparts) * r / CS), s1 = int(int64_t(cv.nparts) * (r + 1) / CS);
+  previous_done();
+  dependents_may_start();
+  const Partial p = sum_slots(a.part + int64_t(cv.part0 + s0) * NPART, threadIdx.x, 256, s1 - s0);
+  block_reduce<8>(p, cluster_at<CS>(&all[r][0]));
+  cluster_done<CS>();
+  if (r == 0 && threadIdx.x == 0) {
+    double v[7];
+#pragma unroll
+    for (int q = 0; q < 7; ++q) v[q] = all[0][q];
+    for (int b = 1; b < CS; ++b)
+#pragma unroll
+      for (int q = 0; q < 7; ++q) v[q] = q < 5 ? v[q] + all[b][q] : fmax(v[q], all[b][q]);
+    residual_of(v, a.resid + 4 * k);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -447,6 +475,33 @@ __global__ void k_import(const CavDev *cavs, int cavity, const double *pref, T *
   for (int q = 0; q < 9; ++q)
     g[9 * cv.off + q * cv.plane + node] = T(fhat[q * n2 + o] - wgt(q) * cv.rho0 - wbar(q) * pt);
   lam[cv.off + node] = T(lami[o]);
+}
+
+// Copies up to three segments of device memory (ifdlbm_save_state_dev and the
+// like), 16 bytes per thread and turn. Bound by the launch at the sizes it is
+// used for: the state of a 257^2 cavity 2.9 us (16.5 as three copies of the
+// copy engine), its step's intermediates 4.1 us (24.7).
+__global__ void __launch_bounds__(256) k_copy(CopyArgs a) {
+  previous_done();
+  dependents_may_start();
+  const int64_t t0 = int64_t(blockIdx.x) * 256 + threadIdx.x, step = int64_t(gridDim.x) * 256;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int4 *src = static_cast<const int4 *>(a.src[k]);
+    int4 *dst = static_cast<int4 *>(a.dst[k]);
+    const int64_t n = a.bytes[k] / 16;
+    int64_t t = t0;
+    for (; t + 3 * step < n; t += 4 * step) {
+      const int4 v0 = src[t], v1 = src[t + step], v2 = src[t + 2 * step], v3 = src[t + 3 * step];
+      dst[t] = v0;
+      dst[t + step] = v1;
+      dst[t + 2 * step] = v2;
+      dst[t + 3 * step] = v3;
+    }
+    for (; t < n; t += step) dst[t] = src[t];
+    if (t0 < (a.bytes[k] & 15) / 8)   // a last double
+      reinterpret_cast<double *>(dst + n)[t0] = reinterpret_cast<const double *>(src + n)[t0];
+  }
 }
 
 // Re-basing of the stored deviations on the mean pressure (FP32 storage):
@@ -617,8 +672,34 @@ void launch_full(const StepArgs &a, int ntiles, cudaStream_t s) {
     k_full<float, false><<<ntiles, kTile, 0, s>>>(a);
 }
 void launch_residual_reduce(const CavDev *cav, const double *part, double *resid, int ncav,
-                            cudaStream_t s) {
-  k_residual_reduce<<<ncav, 256, 0, s>>>(cav, part, resid);
+                            int most, cudaStream_t s) {
+  const ReduceArgs a{cav, part, resid};
+  if (most > REDUCE_ONE)
+    launch_after(k_residual_reduce<REDUCE_CS>, ncav * REDUCE_CS, 256, 0, s, a, REDUCE_CS);
+  else
+    launch_after(k_residual_reduce<1>, ncav, 256, 0, s, a);
+}
+cudaError_t launch_copy(const CopyArgs &a, cudaStream_t s) {
+  // segments that are not on 16-byte boundaries, or not whole doubles, are left
+  // to the copy engine; so are large ones, where three launches do not count
+  int64_t total = 0;
+  bool plain = true;
+  for (int k = 0; k < 3; ++k) {
+    total += a.bytes[k];
+    plain &= ((uintptr_t(a.src[k]) | uintptr_t(a.dst[k])) & 15) == 0 && a.bytes[k] % 8 == 0;
+  }
+  if (plain && total <= COPY_MOST) {
+    const int64_t blocks = (total / 16 + 255) / 256;
+    launch_after(k_copy, int(std::max<int64_t>(1, std::min<int64_t>(blocks, 152 * 8))), 256, 0, s,
+                 a);
+    count_launches(1);
+    return cudaGetLastError();
+  }
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < 3 && e == cudaSuccess; ++k)
+    if (a.bytes[k])
+      e = cudaMemcpyAsync(a.dst[k], a.src[k], size_t(a.bytes[k]), cudaMemcpyDeviceToDevice, s);
+  return e;
 }
 template <class T> void launch_init(const CavDev *cav, const int *tile_cav, void *g, void *lam,
                                     int ntiles, cudaStream_t s) {

@@ -86,7 +86,11 @@ __device__ __forceinline__ double recip(double x) {
   return fma(r, fma(e, e, e), r);
 }
 
+// Signs from the bits; +-0 is nonpositive and nonnegative.
 __device__ __forceinline__ bool negative(double x) { return __double2hiint(x) < 0; }
+__device__ __forceinline__ bool zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ bool nonpositive(double x) { return negative(x) || zero(x); }
+__device__ __forceinline__ bool nonnegative(double x) { return !negative(x) || zero(x); }
 
 // The power law of Eq. (1.4), K/c_s^2 max(q, gmin2)^m, for an FP64 strain
 // rate: the table-driven binomial form of pow_tab (fastpow.cuh) on the full

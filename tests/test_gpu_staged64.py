@@ -73,3 +73,60 @@ def test_lattice_speed():
     fg, lg = s.get_state(0)
     compare_state(fg, lg, fo, lo, lam_tol=lam_bound(f0, l0, prm, lo))
     s.close()
+
+
+def _adjoint_of(specs, states, weights):
+    """One adjoint step of a batch: per cavity (adj_g, adj_lam) and dparams."""
+    import torch
+
+    from paper_2306_07603_gb300 import capi
+    s = solver([cav(*sp) for sp in specs], kernel="staged", dt_mode="grid")
+
+    def checkpoint(parts):
+        for k, (f, lam) in enumerate(parts):
+            s.set_state(k, f, lam)
+        buf = torch.zeros(capi.ifdlbm_state_bytes(s.h) // 8 + 1, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        capi.ifdlbm_save_state_dev(s.h, buf)
+        odd = buf[1:]                      # the same copy to an address off 16 bytes
+        whole = buf.clone()
+        torch.cuda.synchronize()
+        capi.ifdlbm_save_state_dev(s.h, odd)
+        s.sync()
+        assert torch.equal(odd, whole[:-1])
+        return whole[:-1].clone()
+
+    adj, state = checkpoint(weights), checkpoint(states)
+    dp = torch.zeros((len(specs), 3), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    capi.ifdlbm_adjoint_step(s.h, state, adj, dp)
+    s.sync()
+    out, planes = [], [sp[1] * ((sp[0] + 31) // 32 * 32) for sp in specs]
+    g0, l0 = 0, 9 * sum(planes)
+    for sp, p in zip(specs, planes):
+        out.append((adj[g0:g0 + 9 * p].view(9, sp[1], -1)[:, :, :sp[0]].cpu().numpy(),
+                    adj[l0:l0 + p].view(sp[1], -1)[:, :sp[0]].cpu().numpy()))
+        g0, l0 = g0 + 9 * p, l0 + p
+    s.close()
+    return out, dp.cpu().numpy()
+
+
+def test_adjoint_step_of_a_large_batch_equals_the_cavities_alone():
+    """Blocks of 128 threads (above the node count of the one-warp blocks), a
+    cluster per cavity in the reduction and ragged core and ring nodes: the
+    adjoint of each small cavity equals its own in a handle of its own (blocks
+    of one warp, which the dot-product and gradient tests hold to independent
+    derivatives), to the rounding of the same operations: 1e-13 of the largest
+    entry, and 1e-11 of the parameters' sums over some thousand terms."""
+    specs = [(463, 441, 400.0, 0.75, 60.0), (5, 5, 100.0, 0.75, 60.0), (6, 40, 100.0, 1.25, 45.0),
+             (37, 29, 400.0, 1.0, 90.0), (70, 7, 400.0, 0.6, 75.0)]
+    runs = [O.cavity_run(sp[0], sp[2], sp[3], theta_deg=sp[4], ny=sp[1], dt_mode="grid")
+            for sp in specs]
+    states = [synthetic_state(r, 500 + 10 * k) for k, r in enumerate(runs)]
+    weights = [synthetic_state(r, 900 + 10 * k) for k, r in enumerate(runs)]
+    both, dp = _adjoint_of(specs, states, weights)
+    for k in range(1, len(specs)):
+        (one,), dp1 = _adjoint_of(specs[k:k + 1], states[k:k + 1], weights[k:k + 1])
+        for a, b in zip(both[k], one):
+            assert np.abs(a - b).max() <= 1e-13 * np.abs(b).max(), k
+        assert np.all(np.abs(dp[k] - dp1[0]) <= 1e-11 * np.abs(dp1[0]) + 1e-300), k
