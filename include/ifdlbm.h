@@ -55,11 +55,13 @@ extern "C" {
                             equilibrium at a reference pressure (Eq. 2.8 at
                             u = 0), P_ref re-based on the cavity's mean
                             pressure every 1024 steps (a uniform pressure
-                            offset is a neutral, drifting mode). The metrics,
-                            the power law of Eq. (1.4) (on the FP32 strain
-                            rate) and all reductions are FP64 (see power_fp32
-                            for an FP32 power); the relaxation-time plane is
-                            stored in FP32. Every output includes P_ref. */
+                            offset is a neutral, drifting mode). The metrics
+                            and all reductions are FP64; the power law of Eq.
+                            (1.4), on the FP32 strain rate, is FP64 or, in the
+                            fused kernel, pairs of floats (2^-40 before its one
+                            rounding; see power_fp32 for a plain FP32 power);
+                            the relaxation-time plane is stored in FP32. Every
+                            output includes P_ref. */
 
 /* Step kernel organisation. */
 #define IFDLBM_KERNEL_AUTO 0   /* FUSED for FP32DEV, STAGED for FP64 */
@@ -492,6 +494,15 @@ int ifdlbm_inject_tma_timeout(ifdlbm_handle h, int enable);
  * `out` is a DEVICE array of 2n doubles; on the handle's stream (no sync).
  * Errors: INVALID_ARG for a bad handle, cavity or pointers. */
 int ifdlbm_selftest_pow_tab(ifdlbm_handle h, int cavity, int n, const double *x, double *out);
+
+/* Self-test of the same power as the fused kernel evaluates it, in pairs of
+ * floats, rounded once to the FP32 relaxation-time plane: for n DEVICE doubles
+ * x[k] whose float roundings are normal and > 0, writes out[k] = that value and
+ * out[n + k] = the FP64 one of ifdlbm_selftest_pow_tab rounded to FP32, both
+ * widened to double. `out` is a DEVICE array of 2n doubles; on the handle's
+ * stream (no sync). Errors: INVALID_ARG for a bad handle, cavity or pointers, or
+ * an FP64 handle. */
+int ifdlbm_selftest_pow_pair(ifdlbm_handle h, int cavity, int n, const double *x, double *out);
 
 /* Self-test of the FP32 power the FP32-power opt-in uses for Eq. (1.4):
  * for n DEVICE doubles x[k] (finite, > 0 after rounding to float) writes

@@ -55,6 +55,7 @@ struct ifdlbm_ctx {
   int fused_rows = 0;  // rows per task (0: automatic)
   int schedule = IFDLBM_SCHED_GRID;
   int grid = 0;        // CTAs per fused launch
+  int early = 0;       // overlap the launches of consecutive fused steps (build_fused_tasks)
   int task_cap = 0;    // capacity of tasks / order / partial slots
   ifd::Task *tasks = nullptr;
   int *order = nullptr;
@@ -204,12 +205,14 @@ void enqueue_step(ifdlbm_ctx *h, int parity, bool want_residual) {
     f.status = h->b.status;
     f.powtab = h->b.powtab;
     f.powt = h->b.powt;
+    f.powp = h->b.powp;
     f.pref = h->b.pref;
     f.cav_done = h->b.cav_done;
     f.implicit = h->opt.lambda_mode == IFDLBM_LAMBDA_IMPLICIT ? 1 : 0;
     f.general = h->quad.empty() ? 0 : 1;
     f.pow32 = h->opt.power_fp32 ? 1 : 0;
     f.tma_skip = h->tma_skip;
+    f.early = h->early;
     f.resid = h->b.resid;
     f.want_residual = want_residual ? 1 : 0;
     if (h->schedule == IFDLBM_SCHED_DYNAMIC) cudaMemsetAsync(h->counter, 0, sizeof(int), h->stream);
@@ -350,27 +353,84 @@ int build_tmaps(ifdlbm_ctx *h, size_t tsize) {
 
 bool cavity_ok(ifdlbm_ctx *h, int cavity) { return h && cavity >= 0 && cavity < h->ncav; }
 
+// Balanced strips of at most W columns of a cavity nx columns wide: their
+// number and common width, a multiple of 4 columns (W is one too), so that every
+// strip starts on a 16-byte boundary: the fused kernel's TMA row loads start at
+// column i0 - 4 (+ 32 per warp).
+int strips(int nx, int W, int *w4) {
+  const int sx0 = (nx + W - 1) / W;
+  *w4 = (((nx + sx0 - 1) / sx0) + 3) / 4 * 4;
+  return (nx + *w4 - 1) / *w4;
+}
+// Row segments of about `rows` rows (at least 2 rows each) of a cavity.
+int segments(int ny, int rows) { return std::max(1, std::min((ny + rows - 1) / rows, ny / 2)); }
+
+int count_tasks(const ifdlbm_ctx *h, int nt, int rows) {
+  int n = 0, w4;
+  for (const CavDev &cv : h->cav)
+    n += strips(cv.nx, ifd::fused_strip_width(nt), &w4) * segments(cv.ny, rows);
+  return n;
+}
+
+// CTAs of the fused kernel that fit on the device at once, and SMs.
+int fused_resident(const ifdlbm_ctx *h, int nt, int *sms) {
+  const int per_sm = h->precision == IFDLBM_FP64 ? ifd::fused_blocks_per_sm<double>(nt)
+                                                 : ifd::fused_blocks_per_sm<float>(nt);
+  *sms = 0;
+  cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, h->device);
+  return per_sm;
+}
+
+// Rows per task where the caller leaves them open. A task of r rows marches
+// (r + 7) / 2 + 1 iterations (8 halo rows, two rows at a time), and an iteration
+// takes an SM the longer the more CTAs it holds: measured at 128 threads (4 on an
+// SM) 2.0, 2.4, 3.0 and 3.5 us with 1 to 4, which 1.4 + 2.1 f follows, f the share
+// of its slots in use. With `full` rounds of all slots and a rest, a step takes
+//   iterations x (full x 3.5 + (1.4 + 2.1 f_rest)) + 5.8 us,
+// within 7 % of the best of 19 row counts on 22 batches from one 65^2 cavity to
+// 64 of up to 513^2. Few rows fill the chip from a small grid (65^2: 2 rows 14.3
+// us a step, 32 rows 34.5; 257^2: 5 rows 22.4, 32 rows 44.6), many keep the
+// halo's share low on a large one (2049^2: 48 rows 255 us, 12 rows 350).
+int automatic_rows(const ifdlbm_ctx *h, int nt) {
+  int sms = 0, w4;
+  const int per_sm = fused_resident(h, nt, &sms), slots = std::max(1, sms * per_sm);
+  int best = 32;
+  double least = 1e300;
+  for (int rows : {2, 3, 4, 5, 6, 8, 10, 12, 14, 16, 20, 24, 28, 32, 40, 48, 64, 96, 128}) {
+    double its = 0;
+    int n = 0;
+    for (const CavDev &cv : h->cav) {
+      const int sx = strips(cv.nx, ifd::fused_strip_width(nt), &w4), sy = segments(cv.ny, rows);
+      n += sx * sy;
+      its += sx * sy * ((double(cv.ny) / sy + 7) / 2 + 1);
+    }
+    const int full = n / slots, rest = n % slots;
+    const double f = double((rest + sms - 1) / std::max(sms, 1)) / std::max(per_sm, 1);
+    const double t = its / n * (full * 3.5 + (rest ? 1.4 + 2.1 * f : 0.0));
+    if (t < least) {
+      least = t;
+      best = rows;
+    }
+  }
+  return best;
+}
+
 // (Re)builds the fused kernel's tasks: per cavity, balanced strips of at most
 // nt/2 - 8 columns times balanced segments of about `rows` rows (0: automatic),
 // partial slots per cavity contiguous, and the scheduling order (largest
 // tasks first). Uploads the tasks, the order and the cavity table; drops
 // captured graphs. Asynchronous on the handle's stream.
 int build_fused_tasks(ifdlbm_ctx *h, int nt, int rows, int sched) {
-  const int W = ifd::fused_strip_width(nt);
+  const int hs = rows ? rows : automatic_rows(h, nt);
   std::vector<ifd::Task> tasks;
   for (int k = 0; k < h->ncav; ++k) {
     CavDev &cv = h->cav[k];
-    const int hs = rows ? rows : (h->total_plane < (int64_t(8) << 20) ? 32 : 64);
-    // strips of a common width, a multiple of 4 columns (W is one too), so
-    // that every strip starts on a 16-byte boundary: the fused kernel's TMA
-    // row loads start at column i0 - 4 (+ 32 per warp)
-    const int sx0 = (cv.nx + W - 1) / W;
-    const int w4 = (((cv.nx + sx0 - 1) / sx0) + 3) / 4 * 4;
-    const int sx = (cv.nx + w4 - 1) / w4;
+    int w4;
+    const int sx = strips(cv.nx, ifd::fused_strip_width(nt), &w4);
     // a last strip of one column (the right wall alone) would not form column
     // nx - 2, from which the wall column extrapolates: its start moves 4 left
     const int shift = (sx >= 2 && cv.nx - (sx - 1) * w4 < 2) ? 4 : 0;
-    const int sy = std::max(1, std::min((cv.ny + hs - 1) / hs, cv.ny / 2));
+    const int sy = segments(cv.ny, hs);
     cv.part0 = int(tasks.size());
     for (int b = 0; b < sy; ++b)
       for (int a = 0; a < sx; ++a) {
@@ -393,16 +453,21 @@ int build_fused_tasks(ifdlbm_ctx *h, int nt, int rows, int sched) {
     return int64_t(t.i1 - t.i0 + 8) * (t.j1 - t.j0 + 8);
   };
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost(a) > cost(b); });
-  const bool fp64 = h->precision == IFDLBM_FP64;
-  const int per_sm = fp64 ? ifd::fused_blocks_per_sm<double>(nt) : ifd::fused_blocks_per_sm<float>(nt);
-  if (per_sm < 1) return fail(h, IFDLBM_ERR_INVALID_ARG, "fused layout does not fit on an SM");
   int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+  const int per_sm = fused_resident(h, nt, &sms);
+  if (per_sm < 1) return fail(h, IFDLBM_ERR_INVALID_ARG, "fused layout does not fit on an SM");
   h->ntasks = int(tasks.size());
   h->fused_nt = nt;
   h->fused_rows = rows;
   h->schedule = sched;
   h->grid = sched == IFDLBM_SCHED_GRID ? h->ntasks : std::min(h->ntasks, sms * per_sm);
+  // Consecutive steps overlap (launch.cuh) where the next step's CTAs find room
+  // that does not unbalance it: idle SMs of a small grid (65^2: 14.2 -> 12.0 us a
+  // step), or the slots that the last round of a large one leaves (2049^2 257 ->
+  // 252, 64 cavities 499 -> 491). In between they would double up on some SMs
+  // while others have none (129^2 16.6 -> 17.6, 1025^2 87 -> 98).
+  h->early = sched == IFDLBM_SCHED_GRID &&
+             (3 * h->ntasks <= 2 * sms || 5 * h->ntasks >= 4 * sms * per_sm);
   for (int p = 0; p < 2; ++p)
     if (h->gexec[p]) {
       cudaGraphExecDestroy(h->gexec[p]);
@@ -449,6 +514,35 @@ void ifd::fill_cavity_pow_table(double *tab, double m, double C) {
     tab[2 * j + 1] = double(1.0L / c);
   }
   for (int e = 0; e < 256; ++e) tab[512 + e] = double(Cl * exp2l(ml * (e - 127)));
+}
+// Table of pow_pair from pow_tab's: each double split into a pair of floats, and
+// the range of exponents whose factor lies in [2^-60, 2^60] (a contiguous one:
+// the factor is monotonic in the exponent; 0 and 255 are no normal floats).
+void ifd::fill_cavity_pair_table(float *tab, const double *powt, CavDev &cv) {
+  auto split = [](double v, float *hi) {
+    hi[0] = float(v);
+    hi[1] = std::isfinite(hi[0]) ? float(v - double(hi[0])) : 0.0f;
+  };
+  for (int j = 0; j < 256; ++j) {
+    split(powt[2 * j], tab + 4 * j);
+    split(powt[2 * j + 1], tab + 4 * j + 2);
+  }
+  int lo = 256, hi = -1;
+  for (int e = 0; e < 256; ++e) {
+    const double A = powt[512 + e];
+    split(A, tab + 1024 + 2 * e);
+    if (e >= 1 && e <= 254 && A >= 0x1p-60 && A <= 0x1p60) {
+      lo = std::min(lo, e);
+      hi = e;
+    }
+  }
+  cv.pe_lo = unsigned(lo);
+  cv.pe_n = unsigned(std::max(0, hi - lo + 1));
+  float b1[2];
+  split(cv.half_nm1, b1);
+  cv.pb1h = b1[0];
+  cv.pb1l = b1[1];
+  cv.pb2f = float(cv.pb2);
 }
 void ifd::count_launches(int64_t n) { g_launches += n; }
 
@@ -806,6 +900,8 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
       cap += ((cv.nx + wmin - 1) / wmin) *
              std::max(1, std::min((cv.ny + rmin - 1) / rmin, cv.ny / 2));
     h->task_cap = std::max(cap, 1);
+    if (!opt.fused_rows)
+      h->task_cap = std::max(h->task_cap, count_tasks(h, h->fused_nt, automatic_rows(h, h->fused_nt)));
   }
   auto A = [&](size_t bytes) { return dalloc(h, bytes); };
   bool ok = true;
@@ -838,6 +934,9 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
   ok &= (h->stage = (double *)A(size_t(10 * h->max_n2) * sizeof(double))) != nullptr;
   ok &= (h->b.powtab = (double *)A(ifd::POW_TABLE_SIZE * sizeof(double))) != nullptr;
   ok &= (h->b.powt = (double *)A(size_t(ncav) * ifd::POWT_SIZE * sizeof(double))) != nullptr;
+  const bool pairs = opt.precision == IFDLBM_FP32DEV;
+  if (pairs)
+    ok &= (h->b.powp = (float *)A(size_t(ncav) * ifd::POWP_SIZE * sizeof(float))) != nullptr;
   ok &= (h->b.pref = (double *)A(size_t(ncav) * sizeof(double))) != nullptr;
   ok &= (h->b.cav_done = (int *)A(size_t(ncav) * sizeof(int))) != nullptr;
   ok &= (h->b.ptile = (double *)A(size_t(h->ntiles + ncav) * sizeof(double))) != nullptr;
@@ -950,6 +1049,19 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
       for (int t = 0; t < nth; ++t) pool.emplace_back(fill, ncav * t / nth, ncav * (t + 1) / nth);
       for (auto &th : pool) th.join();
     }
+  }
+  std::vector<float> powp_h(pairs ? size_t(ncav) * ifd::POWP_SIZE : 0);
+  if (pairs) {
+    for (int k = 0; k < ncav; ++k)
+      ifd::fill_cavity_pair_table(powp_h.data() + size_t(k) * ifd::POWP_SIZE,
+                                  powt_h.data() + size_t(k) * ifd::POWT_SIZE, h->cav[k]);
+    h->h2d_bytes += int64_t(powp_h.size() * sizeof(float) + h->cav.size() * sizeof(CavDev));
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(h->b.powp, powp_h.data(), powp_h.size() * sizeof(float),
+                          cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)   // with the tables' ranges
+      e = cudaMemcpyAsync(h->b.cav, h->cav.data(), h->cav.size() * sizeof(CavDev),
+                          cudaMemcpyHostToDevice, s);
   }
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->b.powt, powt_h.data(), powt_h.size() * sizeof(double),
@@ -1654,6 +1766,20 @@ int ifdlbm_selftest_pow_tab(ifdlbm_handle h, int cavity, int n, const double *x,
   g_launches += 1;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e, "selftest_pow_tab");
+  return IFDLBM_OK;
+}
+
+int ifdlbm_selftest_pow_pair(ifdlbm_handle h, int cavity, int n, const double *x, double *out) {
+  if (!cavity_ok(h, cavity) || n < 0 || (n > 0 && (!x || !out)) || !h->b.powp)
+    return fail(h, IFDLBM_ERR_INVALID_ARG, "selftest_pow_pair: bad arguments or not an FP32 handle");
+  if (n == 0) return IFDLBM_OK;
+  cudaSetDevice(h->device);
+  ifd::launch_pow_pair_selftest(n, x, h->b.cav, cavity,
+                                h->b.powt + size_t(cavity) * ifd::POWT_SIZE,
+                                h->b.powp + size_t(cavity) * ifd::POWP_SIZE, out, h->stream);
+  g_launches += 1;
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(h, e, "selftest_pow_pair");
   return IFDLBM_OK;
 }
 

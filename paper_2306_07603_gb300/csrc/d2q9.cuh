@@ -42,6 +42,7 @@ struct F2 {
 };
 __host__ __device__ constexpr F2 f2_of(double x) { return {float(x), float(x - double(float(x)))}; }
 constexpr F2 INV36 = f2_of(1.0 / 36.0);
+constexpr F2 INV36x4 = {4.0f * INV36.hi, 4.0f * INV36.lo};
 constexpr F2 INV5 = f2_of(1.0 / 5.0);
 __device__ __forceinline__ float mul_f2(float x, F2 k) { return fmaf(x, k.hi, x * k.lo); }
 __host__ __device__ constexpr int w36(int i) { return i == 0 ? 16 : (i <= 4 ? 4 : 1); }
@@ -75,8 +76,9 @@ __device__ __forceinline__ void equilibrium(T P, T ux, T uy, T c, T inv_cs2, T g
   for (int i = 0; i < 9; ++i) {
     const T cu = c * (T(ex(i)) * ux + T(ey(i)) * uy);
     const T quad = cu * inv_cs2 + cu * cu * half_inv_cs4 + base;
-    if constexpr (sizeof(T) == 4)
-      geq[i] = mul_f2(T(wbar36(i)) * pterm + T(w36(i)) * quad, INV36);
+    if constexpr (sizeof(T) == 4)   // wbar_i = w_i for i > 0; 4/36 scales the pair exactly
+      geq[i] = i == 0 ? mul_f2(T(wbar36(0)) * pterm + T(w36(0)) * quad, INV36)
+                      : (i <= 4 ? mul_f2(pterm + quad, INV36x4) : mul_f2(pterm + quad, INV36));
     else
       geq[i] = T(wbar(i)) * pterm + T(wgt(i)) * quad;
   }

@@ -103,6 +103,55 @@ __device__ __forceinline__ double pow_tab(float x, const double *__restrict__ ta
   return fma(P, t * w, P);
 }
 
+// The same C x^m rounded to float, with every product and sum that matters to
+// more than 40 bits carried as a pair of floats (hi + lo; T. J. Dekker, "A
+// floating-point technique for extending the available precision", Numer. Math.
+// 18, 1971) instead of a double: GB300 issues one FP64 warp instruction per 64
+// cycles and sub-partition, so that pow_tab's FP64 chain (7 instructions, its
+// conversions, their latency) is the slowest part of the FP32 step's collision;
+// these ~32 FP32 instructions take half a cycle each per lane group. With
+// delta = f - c_j (exact) and t = delta (1/c_j),
+//
+//   C x^m = P (1 + t w),  P = [C 2^(m (e - 127))] [c_j^m],
+//   w = b1 + t (b2 + t (b3 + t b4)),
+//
+// table entries, 1/c_j and b1 as pairs, t, P, w and t w as pairs, the
+// polynomial's tail (below 2^-9 of w) in one float: every term is held to 2^-40
+// of the result or better (the first one dropped is t^5 b5 < 2^-45), then rounded
+// once. The float it gives differs from pow_tab's rounded one where the exact
+// value lies within 2^-40 of a rounding boundary (about one argument in 2^16)
+// and nowhere else; its error is 0.5 ulp as pow_tab's.
+// Table (POWP_SIZE floats): [4j ..] = c_j^m hi, lo, 1/c_j hi, lo; [1024 + 2e ..] =
+// C 2^(m (e - 127)) hi, lo. Entries e outside [pe_lo, pe_lo + pe_n) are not in
+// [2^-60, 2^60] (their low parts or products could underflow): pow_tab.
+constexpr int POWP_SIZE = 1536;
+
+struct PowPair {
+  const float *tab;         // the cavity's table
+  float b1h, b1l, b2, b3, b4;
+  unsigned pe_lo, pe_n;     // exponents the table covers
+};
+
+__device__ __forceinline__ bool pow_pair_covers(float x, const PowPair &c) {
+  return (__float_as_uint(x) >> 23) - c.pe_lo < c.pe_n;
+}
+__device__ __forceinline__ float pow_pair(float x, const PowPair &c) {
+  const unsigned bits = __float_as_uint(x), e = bits >> 23, j = (bits >> 15) & 255u;
+  const float4 B = __ldg(reinterpret_cast<const float4 *>(c.tab) + j);
+  const float2 A = __ldg(reinterpret_cast<const float2 *>(c.tab + 1024) + e);
+  const float d = __uint_as_float(0x3F800000u | (bits & 0x7FFFFFu)) -
+                  __uint_as_float(0x3F804000u | (j << 15));     // f - c_j, exact
+  const float th = d * B.z, tl = fmaf(d, B.w, fmaf(d, B.z, -th));
+  const float v = fmaf(th, fmaf(th, fmaf(th, c.b4, c.b3), c.b2), c.b1l);
+  const float wh = c.b1h + v, wl = v - (wh - c.b1h);             // |v| <= |b1|
+  const float sh = th * wh, sl = fmaf(th, wl, fmaf(tl, wh, fmaf(th, wh, -sh)));
+  const float Ph = A.x * B.x, Pl = fmaf(A.x, B.y, fmaf(A.y, B.x, fmaf(A.x, B.x, -Ph)));
+  const float yh = Ph * sh;
+  const float yl = fmaf(Ph, sl, fmaf(Pl, sh, fmaf(Ph, sh, -yh) + Pl));
+  const float r = Ph + yh;
+  return r + ((yh - (r - Ph)) + yl);
+}
+
 // x^m in FP32 for the FP32-deviation form: 2^(m log2 x) with CUDA's log2f
 // and exp2f (1 and 2 ulp by the CUDA math documentation). For normal x > 0
 // its relative error is about ln2 2^-24 (2 |m log2 x| + |m log2 x|) from the

@@ -45,7 +45,9 @@
 
 #include "d2q9.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "reduce.cuh"
+#include "step64.cuh"
 #include "tma.cuh"
 
 namespace ifd {
@@ -76,10 +78,14 @@ constexpr int fused_smem_size() {
   return int(sizeof(FusedSmem<T, NT>)) + 128;
 }
 
-// Ring slot of row r (r >= -12) and prefetch slot of iteration it (it >= 0):
-// unsigned remainders by constants, a multiply-high and a shift each.
+// Ring slot of row r (r >= -12): an unsigned remainder by a constant.
 __device__ __forceinline__ int slot6(int r) { return int(unsigned(r + 12) % unsigned(RING)); }
-__device__ __forceinline__ int pf_slot(int it) { return int(unsigned(it) % unsigned(PF)); }
+// (s + d) mod N for slot s and 0 <= d < N, in two instructions: the difference
+// s + d - N wraps to a large unsigned value where it is negative.
+template <int N>
+__device__ __forceinline__ int slot_add(int s, int d) {
+  return int(min(unsigned(s + d), unsigned(s + d - N)));
+}
 
 // a / b for the relaxation weights and the strain-rate factor, whose
 // denominators (2 lam + dt, 4 lam + dt, (2 lam + dt) c_s^2) are positive and
@@ -124,28 +130,45 @@ __device__ __forceinline__ T mixed_sum(T a, T b, T cf, T f0, bool edge, T kb, T 
   return kb * (a - b) + (ku3 * d2 + ku * d3);
 }
 
+// The xi side of a column of the trapezoid: c_{q xi} = c xi_x (e_x - e_y x_eta / H)
+// has the row's positive factor c xi_x, so that the upwind side of every
+// population is the column's. Per pair of opposite directions (pair_of), the
+// step to the downwind neighbour of the first member (the second's is the
+// opposite): the neighbours are loaded from the right side instead of selected
+// after loading both. (Where rounding makes xs zero although e_x - e_y x_eta / H
+// is not, the side does not matter.)
+template <class T>
+struct XiCol {
+  T xeH;     // x_eta / H
+  int d[4];
+};
+template <class T>
+__device__ __forceinline__ XiCol<T> xi_col(T xe) {
+  return {xe, {1, xe <= T(0) ? 1 : -1, xe <= T(1) ? 1 : -1, xe <= T(-1) ? 1 : -1}};
+}
+// |xs_q| = |e_x As - e_y Bs| of the four pairs.
+template <class T>
+__device__ __forceinline__ void xi_speeds(T As, T Bs, T xs[4]) {
+  xs[0] = As;
+  xs[1] = fabs(Bs);
+  xs[2] = fabs(As - Bs);
+  xs[3] = fabs(-As - Bs);
+}
+
 // base_q - scale (c_{q xi} D_xi F + c_{q eta} D_eta F) at an interior node of
-// the trapezoid (Eq. 3.7 with scale = dt/2, Eq. 3.6 with scale = dt):
-// `row` is the xi row of plane q at this thread's lane l, `col` the five eta
-// neighbours. xs = scale c_{q xi} / (2 dxi) = e_x As - e_y Bs, whose sign is
-// the upwind side along xi (it absorbs sigma: xs D = |xs| sum); along eta the
-// side is the sign of e_y (c_{q eta} = c e_y / H) and the factor is
-// Es = scale (c / H) / (2 deta). As = scale c xi_x / (2 dxi) is positive, so
-// the planes with e_y = 0 have the side of e_x. With EDGE the near-wall
-// first-order form is selected by the flags; without it the far upwind
-// neighbour outside the cavity holds the linear extrapolation (a ghost value,
-// written by the caller), which gives the same difference.
-template <int Q, bool EDGE, class T>
-__device__ __forceinline__ T advect_out(T base, const T *row, int l, const T col[5], T As, T Bs,
-                                        T Es, bool clo, bool chi, bool lo, bool hi, T kb, T ku3,
-                                        T ku) {
-  const T xs = T(ex(Q)) * As - T(ey(Q)) * Bs;
+// the trapezoid (Eq. 3.7 with scale = dt/2, Eq. 3.6 with scale = dt): `node` is
+// plane 0 at the node, planes RS apart, `col` the five eta neighbours. xs = scale
+// c |e_x - e_y x_eta/H| xi_x / (2 dxi); along eta the side is the sign of e_y
+// (c_{q eta} = c e_y / H) and the factor is Es = scale (c / H) / (2 deta). With
+// EDGE the near-wall first-order form is selected by the flags; without it the
+// far upwind neighbour outside the cavity holds the linear extrapolation (a
+// ghost value, written by the caller), which gives the same difference.
+template <int Q, int RS, bool EDGE, class T>
+__device__ __forceinline__ T advect_out(T base, const T *node, int d, const T col[5], T xs, T Es,
+                                        bool clo, bool chi, bool lo, bool hi, T kb, T ku3, T ku) {
+  const T *F = node + Q * RS;
   const T f0 = col[2];
-  const T fm1 = row[l - 1], fp1 = row[l + 1];
-  const bool pos = ey(Q) == 0 ? ex(Q) > 0 : xs >= T(0);
-  const T sx = mixed_sum(pos ? fp1 : fm1, pos ? fm1 : fp1, pos ? row[l - 2] : row[l + 2], f0,
-                         EDGE && (pos ? clo : chi), kb, ku3, ku);
-  T out = base - fabs(xs) * sx;
+  T out = base - xs * mixed_sum(F[d], F[-d], F[-2 * d], f0, EDGE && (d > 0 ? clo : chi), kb, ku3, ku);
   if constexpr (ey(Q) > 0)
     out -= Es * mixed_sum(col[3], col[1], col[0], f0, EDGE && lo, kb, ku3, ku);
   else if constexpr (ey(Q) < 0)
@@ -188,19 +211,22 @@ __device__ __forceinline__ void write_ghosts(T *row, int l, bool clo, bool chi, 
   }
 }
 
-// out[q] for q = Q..8; ring planes are RS apart, base planes BS apart.
+// out[q] for q = Q..8; ring planes are RS apart, base planes BS apart; xs: the
+// xi factors of the four pairs.
 template <class T, int Q, int RS, int BS, bool EDGE>
 struct AdvectAll {
-  __device__ __forceinline__ static void run(const T *rows, const T *const cols[5], int l, T As,
-                                             T Bs, T Es, bool clo, bool chi, bool lo, bool hi,
-                                             T kb, T ku3, T ku, const T *base, T out[9]) {
+  __device__ __forceinline__ static void run(const T *const cols[5], const XiCol<T> &xc,
+                                             const T xs[4], T Es, bool clo, bool chi, bool lo,
+                                             bool hi, T kb, T ku3, T ku, const T *base, T out[9]) {
     const T col[5] = {cols[0][Q * RS], cols[1][Q * RS], cols[2][Q * RS], cols[3][Q * RS],
                       cols[4][Q * RS]};
-    out[Q] = advect_out<Q, EDGE>(base[Q * BS], rows + Q * RS, l, col, As, Bs, Es, clo, chi, lo,
-                                 hi, kb, ku3, ku);
+    constexpr int p = pair_of(Q);
+    const int d = p == 0 ? (second_of(Q) ? -1 : 1) : (second_of(Q) ? -xc.d[p] : xc.d[p]);
+    out[Q] = advect_out<Q, RS, EDGE>(base[Q * BS], cols[2], d, col, xs[p], Es, clo, chi, lo, hi,
+                                     kb, ku3, ku);
     if constexpr (Q < 8)
-      AdvectAll<T, Q + 1, RS, BS, EDGE>::run(rows, cols, l, As, Bs, Es, clo, chi, lo, hi, kb, ku3,
-                                             ku, base, out);
+      AdvectAll<T, Q + 1, RS, BS, EDGE>::run(cols, xc, xs, Es, clo, chi, lo, hi, kb, ku3, ku, base,
+                                             out);
   }
 };
 
@@ -257,8 +283,8 @@ __device__ __forceinline__ void leaf_flush(Leaf<T> &l, Partial &p) {
   l.n = 0;
 }
 
-// P1, P0 are pressures of the stored deviations; Pr their reference (the
-// pressure of Eq. 2.11 is Pr + P), which cancels in the difference.
+// In units of c. P1, P0 are pressures of the stored deviations; Pr their
+// reference (the pressure of Eq. 2.11 is Pr + P), which cancels in the difference.
 template <class T>
 __device__ __forceinline__ void leaf_add(Leaf<T> &l, Partial &p, T u1, T v1, T P1, T u0, T v0,
                                          T P0, T Pr, T wJ, unsigned *status) {
@@ -278,7 +304,7 @@ __device__ __forceinline__ void leaf_add(Leaf<T> &l, Partial &p, T u1, T v1, T P
 
 }  // namespace
 
-template <class T, int NT, bool IMPL, bool GEN, bool P32>
+template <class T, int NT, bool IMPL, bool GEN, bool P32, bool PERSIST>
 __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> &S, int ti,
                                            unsigned &phase) {
   constexpr int NC = NT / 2;
@@ -292,8 +318,8 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
   const int nx = cv.nx, ny = cv.ny, pitch = cv.pitch;
   const int64_t plane = cv.plane, goff = cv.goff;
   const double cvc = cv.c, cvH = cv.H;
-  const T Uw = GEN ? T(cv.lid_ux) : T(cv.U);        // lid velocity
-  const T Uwy = GEN ? T(cv.lid_uy) : T(0);
+  const T Uw = GEN ? T(cv.lid_ux / cvc) : T(cv.U / cvc);  // lid velocity / c
+  const T Uwy = GEN ? T(cv.lid_uy / cvc) : T(0);
   const int part0 = cv.part0, nparts = cv.nparts;
   // c xi_x of row j and the Jacobian x_xi H: FP64 metrics for FP64
   // arithmetic, their rounded float copies for FP32 arithmetic.
@@ -318,25 +344,27 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
   const bool own = colv && c >= i0 && c < i1;        // output column (i1 - i0 <= NC - 8)
   const bool inner_c = c >= 1 && c <= nx - 2;
   const bool wall_c = c == 0 || c == nx - 1;
-  const bool clo = c == 1, chi = c == nx - 2;
+  const bool clo = c == 1, chi = c == nx - 2, nearc = clo || chi;
 
   const int64_t b9 = 9 * cv.off;
   T *gout = (T *)a.g_out + b9;
   const T *lam_in = (const T *)a.lam_in + cv.off;   // relaxation time, storage type T
   T *lam_out = (T *)a.lam_out + cv.off;
 
-  const T c_ = T(cv.c), cs2 = T(cv.cs2), ics2 = T(cv.inv_cs2);
+  // Populations do not depend on c: in units of c (u / c, P / c^2) every relation
+  // of the step but the speeds of the differences is that of c = 1, and the
+  // moments' and the equilibrium's constants are compile-time ones.
+  constexpr T c_ = T(1), cs2 = T(1.0 / 3.0), ics2 = T(3);
   const T dt = T(cv.dt), hdt = T(0.5 * cv.dt);
   const T eta_b = T(cv.eta_b);
   const T i2dxi = T(cv.inv2dxi), i2deta = T(cv.inv2deta);
-  const T ceta_unit = T(cv.c / cv.H);
   // factors of the trapezoid's advection (advect_out): scale / (2 dxi) and
   // scale (c / H) / (2 deta) with scale = dt/2 (half step) and dt (full step);
   // the blend weights of Eq. (2.5)
   const T hxs = T(0.5 * cv.dt * cv.inv2dxi), fxs = T(cv.dt * cv.inv2dxi);
   const T Es1 = T(0.5 * cv.dt * cv.inv2deta * cv.c / cv.H), Es2 = T(cv.dt * cv.inv2deta * cv.c / cv.H);
   const T ku = T(1.0 - cv.eta_b), ku3 = T(3.0 * (1.0 - cv.eta_b));
-  const T xeH = GEN ? T(0) : T(a.geo.xeH[goff + cc]);  // x_eta / H of this column
+  const XiCol<T> xc = xi_col<T>(GEN ? T(0) : T(a.geo.xeH[goff + cc]));
   // general quadrilateral: the node's c xi_x, c xi_y, c eta_x, c eta_y and J of
   // Eqs. (3.2)-(3.3), formed in FP64 at creation and rounded to FP32 planes
   const float *qm = GEN ? a.geo.qmet_f + 5 * cv.off : nullptr;
@@ -349,7 +377,6 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
   // registers are at the cap, keeps the division (the approximation's extra
   // live values spill there)
   constexpr bool FASTQ = !GEN;
-  const T Pr = T(a.pref[task.cav]);                  // reference pressure of the deviations
 
   Partial p = {0, 0, 0, 0, 0, 0, 0};
   Leaf<T> leaf;
@@ -371,10 +398,10 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
   const void *tmap = static_cast<const char *>(a.tmap_in) + size_t(task.cav) * TMAP_BYTES;
   const bool aligned = (tx & 3) == 0;
   const bool issue = aligned && !a.tma_skip;
-  auto prefetch = [&](int it) {
+  auto prefetch = [&](int it, int s) {
     const int r = row_of(it);
     if (lane == 0 && r >= rlo && r <= rhi && issue)
-      tma_load_box3(&S.sf[pf_slot(it)][wid][0][0], tmap, tx, r, &S.bar[pf_slot(it)][wid],
+      tma_load_box3(&S.sf[s][wid][0][0], tmap, tx, r, &S.bar[s][wid],
                     uint32_t(9 * 32 * sizeof(T)));
   };
   // A wait that runs out is reported in the status word; the warp then waits
@@ -383,10 +410,9 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
   // waits, bounded too, for the last copy it issued into each slot. The phase
   // bits follow the issued copies only.
   bool gave_up = false;
-  auto wait_row = [&](int it) {
+  auto wait_row = [&](int it, int s) {
     const int r = row_of(it);
     if (r >= rlo && r <= rhi) {
-      const int s = pf_slot(it);
       const bool ok = aligned && !gave_up && mbar_wait(&S.bar[s][wid], (phase >> s) & 1u);
       if (!ok && !gave_up && lane == 0) atomicOr(a.status, STATUS_TMA_TIMEOUT);
       gave_up = gave_up || !ok;
@@ -398,81 +424,69 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
     return (r >= rlo && r <= rhi) ? lam_in[int64_t(r) * pitch + cc] : T(0);
   };
   // per-cavity constants of the relaxation time
-  const double gmin2 = cv.gmin2, half_nm1 = cv.half_nm1, Kics2 = cv.Kics2;
+  const double half_nm1 = cv.half_nm1;
   // the FP32 strain rate's clamp: the largest float not above gamma_min^2 (so
   // that every clamped q is >= it), and not below FLT_MIN
   const float gmin2_f = cv.gmin2_f;
-  const float half_nm1_f = float(half_nm1), Kics2_f = float(Kics2);
-  // pow_tab of the FP32 form: the cavity's table and binomial coefficients
+  const float half_nm1_f = float(half_nm1), Kics2_f = float(cv.Kics2);
   const double *powt = a.powt + int64_t(task.cav) * POWT_SIZE;
-  const double pb2 = cv.pb2;
-  const float pb3 = cv.pb3, pb4 = cv.pb4, pb5 = cv.pb5;
+  const PowPair pw = {a.powp + int64_t(task.cav) * POWP_SIZE, cv.pb1h, cv.pb1l, cv.pb2f, cv.pb3,
+                      cv.pb4, cv.pe_lo, cv.pe_n};
   const T wy_in = T(cv.deta), wy_edge = T(0.5 * cv.deta);
-  // Step (2) for this thread's row of iteration `it`: moments, f^eq and
+  // Step (2) for this thread's row of iteration `it`: moments, f^eq - f-hat and
   // lambda(t). The row of iteration it + 1 is formed during the full step of
   // iteration it, so that the power overlaps the stencil work.
-  T nux = 0, nuy = 0, nP = 0, ngeq[9];
-  T nlam = T(0);
   struct Collided {
-    T ux, uy, P, geq[9];
+    T ux, uy, P, d[9];
     T lam;
   };
-  auto collide = [&](int it, T lam_prev) {
+  Collided now = {};
+  auto collide = [&](int s, T lam_prev) {  // s: prefetch slot of the row
     Collided o;
-    const int s = pf_slot(it);
     T g[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) g[q] = sfme[s * SLOT + q * 32];
     moments(g, c_, cs2, o.ux, o.uy, o.P);                 // Eqs. (2.10)-(2.11)
-    equilibrium(o.P, o.ux, o.uy, c_, ics2, o.geq);        // Eq. (2.8)
-    T d[9];
+    equilibrium(o.P, o.ux, o.uy, c_, ics2, o.d);          // Eq. (2.8)
 #pragma unroll
-    for (int q = 0; q < 9; ++q) d[q] = g[q] - o.geq[q];
-    T pxx, pxy, pyy;
-    second_moments(d, c_, pxx, pxy, pyy);
+    for (int q = 0; q < 9; ++q) o.d[q] -= g[q];
+    T pxx, pxy, pyy;                                      // of f^eq - f-hat: the sign drops out below
+    second_moments(o.d, c_, pxx, pxy, pyy);
     if constexpr (IMPL) {                                  // implicit form of Eq. (2.14)
       const T G2 = T(0.5) * (pxx * pxx + T(2) * pxy * pxy + pyy * pyy);
       if constexpr (P32)
         o.lam = T(lambda_implicit_f32(float(T(2) * sqrt(G2) * ics2), float(lam_prev), cv));
       else
-        o.lam = T(lambda_implicit(2.0 * sqrt(double(G2)) * cv.inv_cs2, double(lam_prev), cv,
-                                  a.powtab));
+        o.lam = T(lambda_implicit(2.0 * sqrt(double(G2)) * 3.0, double(lam_prev), cv, a.powtab));
       return o;
     }
-    // Eqs. (2.12)-(2.14), (1.4): strain rate in T, power in FP64 (as
-    // relaxation_time), or in FP32 with the pow32 opt-in
+    // Eqs. (2.12)-(2.14), (1.4): strain rate in T, power in FP64, by pairs of
+    // floats rounded once to the FP32 plane, or in FP32 with the pow32 opt-in
     const T k = quot<FASTQ>(T(-2), (T(2) * lam_prev + dt) * cs2);
     const T Sxx = k * pxx, Sxy = k * pxy, Syy = k * pyy;
     if constexpr (sizeof(T) == 4) {
-      // the strain rate is FP32 here: clamped in FP32, then C q^m in FP64 by
-      // pow_tab (7 FP64 instructions) and rounded to the FP32 plane
       const float qf = fmaxf(T(0.5) * (Sxx * Sxx + T(2) * Sxy * Sxy + Syy * Syy), gmin2_f);
       if constexpr (P32)
         o.lam = Kics2_f * pow_f32(qf, half_nm1_f);
+      else if (pow_pair_covers(qf, pw))
+        o.lam = pow_pair(qf, pw);
       else
-        o.lam = float(pow_tab(qf, powt, half_nm1, pb2, pb3, pb4, pb5));
+        o.lam = float(pow_tab(qf, powt, half_nm1, cv.pb2, cv.pb3, cv.pb4, cv.pb5));
     } else {
-      double q = double(T(0.5) * (Sxx * Sxx + T(2) * Sxy * Sxy + Syy * Syy));
-      q = q > gmin2 ? q : gmin2;
-      o.lam = Kics2 * pow_fast(q, half_nm1, a.powtab);
+      o.lam = power_law64(T(0.5) * (Sxx * Sxx + T(2) * Sxy * Sxy + Syy * Syy), cv, a.powtab, powt);
     }
     return o;
   };
-  auto take = [&](const Collided &o) {
-    nux = o.ux;
-    nuy = o.uy;
-    nP = o.P;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) ngeq[q] = o.geq[q];
-    nlam = o.lam;
-  };
   auto in_a = [&](int r) { return r >= rlo && r <= rhi; };
 
+  // everything so far is the same in every step; what follows the step before writes
+  if constexpr (!PERSIST) previous_done();
+  const T Pr = T(a.pref[task.cav] / (cvc * cvc));  // reference pressure of the deviations / c^2
   if (lane == 0) tmap_acquire(tmap);
-  prefetch(0);
-  prefetch(1);
-  wait_row(0);
-  if (in_a(row_of(0))) take(collide(0, lam_load(row_of(0))));
+  prefetch(0, 0);
+  prefetch(1, 1);
+  wait_row(0, 0);
+  if (in_a(row_of(0))) now = collide(0, lam_load(row_of(0)));
   T lp_next = lam_load(row_of(1));       // lambda_prev of the next row
   T Lprev = T(0);                        // lambda(t) of this thread's previous row
   // metrics of this iteration's half-step and full-step rows, loaded one
@@ -485,16 +499,21 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
     A1 = row_cxix(crow(kb - 2 + h)), A2 = row_cxix(crow(kb - 4 + h)), J2 = row_jac(crow(kb - 4 + h));
   }
 
-  for (int it = 0; it < nit; ++it) {
+  // Slots of iteration it, advanced with it: s0 the ring slot of row k + h (the
+  // six rows k + h - 5 .. k + h that an iteration touches have the six slots
+  // s0 + 1 .. s0 + 6 mod 6), pf its prefetch slot (it mod PF).
+  int s0 = slot6(kb + h), pf = 0;
+  for (int it = 0; it < nit; ++it, s0 = slot_add<RING>(s0, 2), pf = slot_add<PF>(pf, 1)) {
     const int k = kb + 2 * it;
+    auto ring = [&](int d) { return slot_add<RING>(s0, d); };  // slot of row k + h + d - 6 or + d
 
     // ---------------- stage A: row k + h (lambda formed in the previous iteration) ----------------
     const int ar = k + h;
     T Lcur = T(0);
     if (in_a(ar)) {
-      const int s = pf_slot(it), sb = slot6(ar);
-      if (own && ar >= j0 && ar < j1) lam_out[int64_t(ar) * pitch + c] = nlam;
-      const T L = nlam;
+      const int s = pf, sb = s0;
+      if (own && ar >= j0 && ar < j1) lam_out[int64_t(ar) * pitch + c] = now.lam;
+      const T L = now.lam;
       Lcur = L;
       const T i2 = quot<FASTQ>(T(1), T(2) * L + dt);
       const T bp = T(2) * dt * i2;     // Eq. (2.15): (2 lam - dt)/(2 lam + dt) = 1 - bp
@@ -502,31 +521,31 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
 #pragma unroll
       for (int q = 0; q < 9; ++q) {
         const T gq = sfme[s * SLOT + q * 32];
-        S.fb[sb][q][l] = toward(gq, ngeq[q], bb);
-        sfme[s * SLOT + q * 32] = toward(gq, ngeq[q], bp);  // f-hat^+ in place of g
+        S.fb[sb][q][l] = gq + bb * now.d[q];
+        sfme[s * SLOT + q * 32] = gq + bp * now.d[q];  // f-hat^+ in place of g
       }
       if (ar == 0 || ar == ny - 1) {
         const int e = ar == 0 ? 0 : 1;
-        S.edge[e][0][l] = nux;
-        S.edge[e][1][l] = nuy;
-        S.edge[e][2][l] = nP;
+        S.edge[e][0][l] = now.ux;
+        S.edge[e][1][l] = now.uy;
+        S.edge[e][2][l] = now.P;
       }
     }
     __syncthreads();  // f-bar^+ of rows k, k + 1
     // the slot this prefetch fills was last read before the barrier above
-    prefetch(it + 2);
+    prefetch(it + 2, slot_add<PF>(pf, 2));
 
     // ---------------- stage 1: row m = k - 2 + h ----------------
     const int m = k - 2 + h;
     const bool do1 = m >= mlo && m <= mhi;
     if (do1 && inner_c && l >= 2 && l < NC - 2) {
-      const int sm = slot6(m);
+      const int sm = ring(4);
       const bool lo = m == 1, hi = m == ny - 2;
       T fbar[9];
       fbar[0] = S.fb[sm][0][l];
       {
-        const T *cols[5] = {&S.fb[slot6(m - 2)][0][l], &S.fb[slot6(m - 1)][0][l], &S.fb[sm][0][l],
-                            &S.fb[slot6(m + 1)][0][l], &S.fb[slot6(m + 2)][0][l]};
+        const T *cols[5] = {&S.fb[ring(2)][0][l], &S.fb[ring(3)][0][l], &S.fb[sm][0][l],
+                            &S.fb[ring(5)][0][l], &S.fb[s0][0][l]};
         if constexpr (GEN) {
           AdvectAllGen<T, 1, NC, NC>::run(&S.fb[sm][0][0], cols, l, qmet(0, m), qmet(1, m),
                                           qmet(2, m), qmet(3, m), clo, chi, lo, hi, eta_b, i2dxi,
@@ -534,14 +553,14 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
                                           &S.fb[sm][0][l], fbar);  // Eq. (3.7)
         } else {
           const T As = A1 * hxs;                         // dt/2 c xi_x / (2 dxi) of row m
-          const T Bs = As * xeH;                         // ... times x_eta / H
-          if constexpr (GHOST)
+          T xs[4];
+          xi_speeds(As, As * xc.xeH, xs);
+          if (GHOST && (nearc || lo || hi))
             write_ghosts<T, NC>(&S.fb[sm][0][0], l, clo, chi, lo, hi, &S.fb[slot6(-1)][0][l],
                                 &S.fb[slot6(0)][0][l], &S.fb[slot6(ny)][0][l],
                                 &S.fb[slot6(ny - 1)][0][l]);
-          AdvectAll<T, 1, NC, NC, !GHOST>::run(&S.fb[sm][0][0], cols, l, As, Bs, Es1, clo, chi, lo,
-                                               hi, eta_b, ku3, ku, &S.fb[sm][0][l],
-                                               fbar);  // Eq. (3.7)
+          AdvectAll<T, 1, NC, NC, !GHOST>::run(cols, xc, xs, Es1, clo, chi, lo, hi, eta_b, ku3, ku,
+                                               &S.fb[sm][0][l], fbar);  // Eq. (3.7)
         }
       }
       T ux, uy, P;
@@ -587,20 +606,21 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
     // ---------------- stage 2: row o = k - 4 + h ----------------
     const int o = k - 4 + h;
     const bool do2 = o >= olo && o <= ohi;
-    const int sp = pf_slot(it + PF - 2);             // f-hat^+ of row o (iteration it - 2)
-    wait_row(it + 1);                                // this warp's row of iteration it + 1
+    const int sp = slot_add<PF>(pf, PF - 2);         // f-hat^+ of row o (iteration it - 2)
+    wait_row(it + 1, slot_add<PF>(pf, 1));           // this warp's row of iteration it + 1
     T gnv[9];
     if (do2 && inner_c && l >= 4 && l < NC - 4) {
-      const int so = slot6(o);
+      const int so = ring(2);
       const bool lo = o == 1, hi = o == ny - 2;
       gnv[0] = sfme[sp * SLOT];
       {
         // rows o-2..o+2 of f(t + dt/2); the lid row ny-1 has a buffer of its own
-        auto fhrow = [&](int r) -> const T * {
-          return r == ny - 1 ? &S.lid[0][l] : &S.fh[slot6(r)][0][l];
+        // (a row of the full step is at most ny - 2)
+        auto fhrow = [&](int r, int s) -> const T * {
+          return r == ny - 1 ? &S.lid[0][l] : &S.fh[s][0][l];
         };
-        const T *cols[5] = {fhrow(o - 2), fhrow(o - 1), &S.fh[so][0][l], fhrow(o + 1),
-                            fhrow(o + 2)};
+        const T *cols[5] = {&S.fh[s0][0][l], &S.fh[ring(1)][0][l], &S.fh[so][0][l],
+                            fhrow(o + 1, ring(3)), fhrow(o + 2, ring(4))};
         if constexpr (GEN) {
           AdvectAllGen<T, 1, NC, 32>::run(&S.fh[so][0][0], cols, l, qmet(0, o), qmet(1, o),
                                           qmet(2, o), qmet(3, o), clo, chi, lo, hi, eta_b, i2dxi,
@@ -608,13 +628,13 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
                                           sfme + sp * SLOT, gnv);  // Eq. (3.6)
         } else {
           const T As = A2 * fxs;                         // dt c xi_x / (2 dxi) of row o
-          const T Bs = As * xeH;
-          if constexpr (GHOST)
+          T xs[4];
+          xi_speeds(As, As * xc.xeH, xs);
+          if (GHOST && (nearc || lo || hi))
             write_ghosts<T, NC>(&S.fh[so][0][0], l, clo, chi, lo, hi, &S.fh[slot6(-1)][0][l],
                                 &S.fh[slot6(0)][0][l], &S.fh[slot6(ny)][0][l], &S.lid[0][l]);
-          AdvectAll<T, 1, NC, 32, !GHOST>::run(&S.fh[so][0][0], cols, l, As, Bs, Es2, clo, chi, lo,
-                                               hi, eta_b, ku3, ku, sfme + sp * SLOT,
-                                               gnv);  // Eq. (3.6)
+          AdvectAll<T, 1, NC, 32, !GHOST>::run(cols, xc, xs, Es2, clo, chi, lo, hi, eta_b, ku3, ku,
+                                               sfme + sp * SLOT, gnv);  // Eq. (3.6)
         }
       }
       if (clo || chi) {                                // values the wall columns extrapolate
@@ -622,7 +642,7 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
         for (int q = 0; q < 9; ++q) S.gw[h][chi ? 1 : 0][q] = gnv[q];
       }
     }
-    if (in_a(row_of(it + 1))) take(collide(it + 1, lp_next));  // lambda of the next row
+    if (in_a(row_of(it + 1))) now = collide(slot_add<PF>(pf, 1), lp_next);  // lambda of the next row
     lp_next = lam_load(row_of(it + 2));
     [[maybe_unused]] const T J2o = J2;               // Jacobian of row o (trapezoid)
     if constexpr (!GEN) {
@@ -701,8 +721,15 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
     for (int s = 0; s < PF; ++s) mbar_wait(&S.bar[s][wid], ((phase >> s) & 1u) ^ 1u);
   if (a.want_residual) {
     leaf_flush(leaf, p);
-    p.du2max = double(leaf.du2max);
-    p.u2max = double(leaf.u2max);
+    // from units of c
+    const double c2 = cvc * cvc, c4 = c2 * c2;
+    p.du2 *= c2;
+    p.u2 *= c2;
+    p.ek *= c2;
+    p.dP2 *= c4;
+    p.P2 *= c4;
+    p.du2max = c2 * double(leaf.du2max);
+    p.u2max = c2 * double(leaf.u2max);
     block_partial<NT / 32>(p, a.part, ti);
     // The last task of the cavity to finish reduces the cavity's partials
     // (a counter, no waiting: every other CTA just moves on).
@@ -734,7 +761,7 @@ struct Occ {
 // blockIdx.x, blockIdx.x + gridDim.x, ... of the largest-first order;
 // 2 persistent CTAs taking positions from an atomic counter (no waiting on
 // other CTAs: a CTA that finds the list exhausted returns).
-template <class T, int NT, bool IMPL, bool GEN, bool P32>
+template <class T, int NT, bool IMPL, bool GEN, bool P32, bool PERSIST>
 __global__ void __launch_bounds__(NT, Occ<T, NT>::blocks) k_fused(FusedArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // the TMA boxes want 128-byte aligned shared memory: align the struct
@@ -747,39 +774,51 @@ __global__ void __launch_bounds__(NT, Occ<T, NT>::blocks) k_fused(FusedArgs a) {
   mbar_init_fence();
   __syncthreads();
   unsigned phase = 0;  // bit s: parity of the next completion of slot s's barrier (this warp)
-  if (a.schedule == 0) {
-    fused_task<T, NT, IMPL, GEN, P32>(a, S, blockIdx.x, phase);
-    return;
-  }
-  for (int it = 0;; ++it) {
-    int pos;
-    if (a.schedule == 1) {
-      pos = blockIdx.x + it * gridDim.x;
-    } else {
-      if (threadIdx.x == 0) next = atomicAdd(a.counter, 1);
-      __syncthreads();
-      pos = next;
-      __syncthreads();
+  // (kernels of their own for one task per CTA and for a loop over tasks, so that
+  // each holds the code of a task once)
+  if constexpr (!PERSIST) {
+    if (a.early) dependents_may_start();
+    fused_task<T, NT, IMPL, GEN, P32, PERSIST>(a, S, blockIdx.x, phase);
+  } else {
+    for (int it = 0;; ++it) {
+      int pos;
+      if (a.schedule == 1) {
+        pos = blockIdx.x + it * gridDim.x;
+      } else {
+        if (threadIdx.x == 0) next = atomicAdd(a.counter, 1);
+        __syncthreads();
+        pos = next;
+        __syncthreads();
+      }
+      if (pos >= a.ntasks) return;
+      fused_task<T, NT, IMPL, GEN, P32, PERSIST>(a, S, a.order[pos], phase);
     }
-    if (pos >= a.ntasks) return;
-    fused_task<T, NT, IMPL, GEN, P32>(a, S, a.order[pos], phase);
   }
 }
 
-template <class T, int NT, bool IMPL, bool GEN = false, bool P32 = false>
+template <class T, int NT, bool IMPL, bool GEN, bool P32, bool PERSIST>
 static void configure_nt() {
   static bool configured = false;  // the attribute is per function
   if (!configured) {
-    cudaFuncSetAttribute(k_fused<T, NT, IMPL, GEN, P32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         fused_smem_size<T, NT>());
+    cudaFuncSetAttribute(k_fused<T, NT, IMPL, GEN, P32, PERSIST>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, fused_smem_size<T, NT>());
     configured = true;
   }
 }
 
 template <class T, int NT, bool IMPL, bool GEN, bool P32>
 static void launch_variant(const FusedArgs &a, int grid, cudaStream_t s) {
-  configure_nt<T, NT, IMPL, GEN, P32>();
-  k_fused<T, NT, IMPL, GEN, P32><<<grid, NT, fused_smem_size<T, NT>(), s>>>(a);
+  constexpr int smem = fused_smem_size<T, NT>();
+  if (a.schedule == 0) {
+    configure_nt<T, NT, IMPL, GEN, P32, false>();
+    if (a.early)
+      launch_after(k_fused<T, NT, IMPL, GEN, P32, false>, grid, NT, smem, s, a);
+    else
+      k_fused<T, NT, IMPL, GEN, P32, false><<<grid, NT, smem, s>>>(a);
+  } else {
+    configure_nt<T, NT, IMPL, GEN, P32, true>();
+    k_fused<T, NT, IMPL, GEN, P32, true><<<grid, NT, smem, s>>>(a);
+  }
 }
 
 template <class T, int NT>
@@ -810,9 +849,9 @@ static void launch_fused_nt(const FusedArgs &a, int grid, cudaStream_t s) {
 
 template <class T, int NT>
 static int blocks_per_sm_nt() {
-  configure_nt<T, NT, false>();
+  configure_nt<T, NT, false, false, false, true>();
   int n = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused<T, NT, false, false, false>, NT,
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused<T, NT, false, false, false, true>, NT,
                                                 fused_smem_size<T, NT>());
   return n;
 }

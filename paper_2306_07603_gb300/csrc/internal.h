@@ -49,6 +49,8 @@ struct CavDev {
   // the clamp of the FP32 strain rate, max(largest float <= gamma_min^2, FLT_MIN)
   double pb2;
   float pb3, pb4, pb5, gmin2_f;
+  float pb1h, pb1l, pb2f;   // pow_pair: b1 = m as a pair of floats, b2 rounded
+  unsigned pe_lo, pe_n;     // ... and the exponents its table covers
   // FP64 staged kernels (staged64.cu): thread blocks of this cavity and, for the
   // half step [0] and the full step [1] (scale dt/2 and dt), the coefficients
   // of the mixed difference (xi, unscaled; eta of the trapezoid, times -scale
@@ -101,6 +103,7 @@ struct Bufs {
   Geo geo;
   double *powtab;    // tables of pow_fast (fastpow.cuh)
   double *powt;      // [ncav][POWT_SIZE] per-cavity tables of pow_tab (fastpow.cuh)
+  float *powp;       // [ncav][POWP_SIZE] per-cavity tables of pow_pair (fused kernel)
   double *pref;      // [ncav] reference pressure: f-hat = w rho0 + wbar pref / c_s^2 + g
   int *cav_done;     // [ncav] fused kernel: tasks finished in the current step
   double *ptile;     // [ntiles + ncav] scratch of the re-basing reduction
@@ -151,11 +154,13 @@ struct FusedArgs {
   unsigned *status;
   const double *powtab;
   const double *powt;  // [ncav][POWT_SIZE] tables of pow_tab
+  const float *powp;   // [ncav][POWP_SIZE] tables of pow_pair
   const double *pref;  // [ncav] reference pressure of the stored deviations
   int *cav_done;       // [ncav] tasks of the step finished (zero between steps)
   int implicit;        // 1: implicit form of Eq. (2.14) (kernel variant), 0: lagged
   int general;         // 1: general quadrilaterals (kernel variant; FP32, lagged)
   int pow32;           // 1: FP32 power law (opt-in of the FP32 form; kernel variant)
+  int early;           // 1: the CTAs of the next step may start before this one is done
   int tma_skip;        // test hook: 1 issues no TMA row loads, so that every row wait runs out
   double *resid;       // [ncav][4] residual outputs (formed by each cavity's last task)
   int want_residual;
@@ -221,8 +226,11 @@ void launch_adjoint_step(const AdjArgs &a, cudaStream_t s);
 // Host-built tables of pow_fast and of pow_tab (capi.cu) and their self-tests (staged.cu)
 void fill_pow_tables(double *tab);
 void fill_cavity_pow_table(double *tab, double m, double C);
+void fill_cavity_pair_table(float *tab, const double *powt, CavDev &cv);
 void launch_pow_tab_selftest(int n, const double *x, double m, double C, const double *tab,
                              double b2, float b3, float b4, float b5, double *out, cudaStream_t s);
+void launch_pow_pair_selftest(int n, const double *x, const CavDev *cav, int cavity,
+                              const double *powt, const float *powp, double *out, cudaStream_t s);
 void launch_pow_f32_selftest(int n, const double *x, double m, double *out, cudaStream_t s);
 
 // Metrics of the bilinear map of a general quadrilateral at (xi, eta),

@@ -599,6 +599,25 @@ void launch_pow_tab_selftest(int n, const double *x, double m, double C, const d
   k_pow_tab_selftest<<<(n + 255) / 256, 256, 0, s>>>(n, x, m, C, tab, b2, b3, b4, b5, out);
 }
 
+// The FP32 form's power of Eq. (1.4) as the fused kernel evaluates it (pow_pair
+// where its table covers the argument, else pow_tab): out[k] of the FP32
+// rounding of x[k], and out[n + k] = pow_tab's value rounded to FP32.
+__global__ void k_pow_pair_selftest(int n, const double *x, const CavDev *cavs, int cavity,
+                                    const double *powt, const float *powp, double *out) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= n) return;
+  const CavDev &cv = cavs[cavity];
+  const PowPair pw = {powp, cv.pb1h, cv.pb1l, cv.pb2f, cv.pb3, cv.pb4, cv.pe_lo, cv.pe_n};
+  const float xf = float(x[k]);
+  const float t = float(pow_tab(xf, powt, cv.half_nm1, cv.pb2, cv.pb3, cv.pb4, cv.pb5));
+  out[k] = double(pow_pair_covers(xf, pw) ? pow_pair(xf, pw) : t);
+  out[n + k] = double(t);
+}
+void launch_pow_pair_selftest(int n, const double *x, const CavDev *cav, int cavity,
+                              const double *powt, const float *powp, double *out, cudaStream_t s) {
+  k_pow_pair_selftest<<<(n + 255) / 256, 256, 0, s>>>(n, x, cav, cavity, powt, powp, out);
+}
+
 __global__ void k_pow_f32_selftest(int n, const double *x, double m, double *out) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
