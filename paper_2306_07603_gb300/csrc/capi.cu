@@ -817,6 +817,13 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
       float g = float(cv.gmin2);
       if (double(g) > cv.gmin2) g = std::nextafter(g, 0.0f);
       cv.gmin2_f = std::max(g, FLT_MIN);
+      // implicit form (ImplPair): the root is the clamp value where 6 sqrt(G2) <=
+      // gmin (2 lam_c + dt), for a float G2 where it is at most this bound rounded down
+      auto mid = [](double v) { return v > 1e-25 && v < 1e25; };
+      cv.impl_f32 = cv.nm1 != 0.0 && mid(cv.Kics2) && mid(cv.lam0) && mid(cv.dt) ? 1 : 0;
+      const double a0 = cv.gmin * (2.0 * cv.lam0 + cv.dt), g2 = a0 * a0 / 36.0;
+      cv.g2c_f = float(g2);
+      if (double(cv.g2c_f) > g2) cv.g2c_f = std::nextafter(cv.g2c_f, 0.0f);
     }
     h->max_n2 = std::max<int64_t>(h->max_n2, int64_t(s.nx) * s.ny);
     // 1-D metric arrays of Eq. (3.8.2)

@@ -93,49 +93,7 @@ __device__ __forceinline__ T toward(T F, T feq, T b) {
   return F + b * (feq - F);
 }
 
-// Implicit form of Eq. (2.14): lam = C max(a / (2 lam + dt), gamma_min)^(n-1)
-// with C = K / c_s^2 and a = 2 sqrt((Pxx^2 + 2 Pxy^2 + Pyy^2) / 2) / c_s^2,
-// Pxx.. the second moments of f-hat - f^eq (Eq. 2.18 at the same lam turns
-// them into gamma-dot(lam) = a / (2 lam + dt)). F(lam) = lam - C max(...)^(n-1)
-// increases strictly, so the root is unique: it is the clamp value
-// lam_c = C gamma_min^(n-1) when gamma-dot(lam_c) <= gamma_min, and otherwise
-// lies in [0, lam_c] (n < 1) or [lam_c, C (a/dt)^(n-1)] (n > 1) with
-// gamma-dot > gamma_min. Newton from lam_start, kept inside the bracket by
-// bisection, one FP64 power per iteration; it stops once the Newton step is
-// below 4e-15 of lam (F = lam - P is itself a difference of nearly equal
-// numbers, so steps much smaller than that are rounding). Kept out of line so
-// that the lagged path is compiled as without it.
-static __device__ __noinline__ double lambda_implicit(double a, double lam_start, const CavDev &cv,
-                                                      const double *powtab) {
-  const double C = cv.Kics2, dt = cv.dt, m = cv.nm1, lamc = cv.lam0;
-  if (m == 0.0) return C;
-  if (a <= cv.gmin * (2.0 * lamc + dt)) return lamc;
-  double lo, hi;
-  if (m < 0.0) {
-    lo = 0.0;
-    hi = lamc;
-  } else {
-    lo = lamc;
-    hi = C * pow_fast((a / dt) * (a / dt), cv.half_nm1, powtab);
-  }
-  double lam = (lam_start > lo && lam_start < hi) ? lam_start : 0.5 * (lo + hi);
-  for (int it = 0; it < 20; ++it) {
-    const double x = 2.0 * lam + dt;
-    const double g = a / x;
-    const double P = C * pow_fast(g * g, cv.half_nm1, powtab);
-    const double F = lam - P;
-    if (F == 0.0) break;                                   // the root itself
-    if (F > 0.0) hi = lam; else lo = lam;
-    double next = lam - F / (1.0 + 2.0 * m * P / x);
-    if (!(next >= lo && next <= hi)) next = 0.5 * (lo + hi);
-    const bool done = fabs(next - lam) <= 4e-15 * next;
-    lam = next;
-    if (done) break;
-  }
-  return lam;
-}
-
-// The same solve in FP32 for the FP32-deviation form, with the FP32 power
+// The implicit form of Eq. (2.14) (implicit.cuh) in FP32, the FP32-power opt-in's, with the FP32 power
 // (pow_f32, relative error ~1e-6 for these arguments): F is then known to
 // about 1e-6 of lam, so the iteration stops once the Newton step is below
 // 4e-6 of lam, after at most 10 iterations. As with the power, this error
@@ -170,36 +128,6 @@ static __device__ __noinline__ float lambda_implicit_f32(float a, float lam_star
     if (done) break;
   }
   return lam;
-}
-
-// Relaxation time of Step (2) of the FP32 staged kernels: strain rate from f^ne
-// (Eqs. 2.12-2.13, with f = f(f-hat, lam_prev) of Eq. 2.18), q = |gamma-dot|^2 =
-// 2 D:D, the clamped power law mu = K max(|gamma-dot|, gamma_min)^(n-1)
-// evaluated as K max(q, gamma_min^2)^((n-1)/2) (Eq. 1.4), and lam = mu / c_s^2
-// (Eq. 2.14). Pxx, Pxy, Pyy are sum_i c_ia c_ib (g_i - geq_i). The strain rate
-// is formed in FP32, clamped at cv.gmin2_f; the power law of Eq. (1.4)
-// (pow_tab, FP64 result, error within 6e-16) and the implicit form's solve are
-// FP64, as the FP32-deviation form specifies. With cv.pow32 (an opt-in) they
-// are FP32 instead (pow_f32, lambda_implicit_f32; the clamp at the largest
-// float not above gamma_min^2). powt: the cavity's pow_tab table.
-__device__ __forceinline__ double relaxation_time(float Pxx, float Pxy, float Pyy,
-                                                  float lam_prev, const CavDev &cv,
-                                                  const double *powtab, const double *powt) {
-  if (cv.implicit) {
-    const float G2 = 0.5f * (Pxx * Pxx + 2.0f * Pxy * Pxy + Pyy * Pyy);
-    if (cv.pow32)
-      return double(lambda_implicit_f32(2.0f * sqrtf(G2) * float(cv.inv_cs2), lam_prev, cv));
-    return lambda_implicit(2.0 * sqrt(double(G2)) * cv.inv_cs2, double(lam_prev), cv, powtab);
-  }
-  // f^ne = 2 lam_prev/(2 lam_prev + dt) (f-hat - f^eq);  S = -sum c c f^ne / (lam_prev c_s^2)
-  const float k = -2.0f / ((2.0f * lam_prev + float(cv.dt)) * float(cv.cs2));
-  const float Sxx = k * Pxx, Sxy = k * Pxy, Syy = k * Pyy;
-  const float q2 = 0.5f * (Sxx * Sxx + 2.0f * Sxy * Sxy + Syy * Syy);
-  if (cv.pow32) {
-    const float q = fmaxf(q2, __double2float_rd(cv.gmin2));
-    return double(float(cv.Kics2) * pow_f32(q, float(cv.half_nm1)));
-  }
-  return pow_tab(fmaxf(q2, cv.gmin2_f), powt, cv.half_nm1, cv.pb2, cv.pb3, cv.pb4, cv.pb5);
 }
 
 // Second moments of the non-equilibrium deviation d_i = g_i - geq_i.

@@ -135,7 +135,7 @@ struct PowPair {
 __device__ __forceinline__ bool pow_pair_covers(float x, const PowPair &c) {
   return (__float_as_uint(x) >> 23) - c.pe_lo < c.pe_n;
 }
-__device__ __forceinline__ float pow_pair(float x, const PowPair &c) {
+__device__ __forceinline__ void pow_pair_parts(float x, const PowPair &c, float &hi, float &lo) {
   const unsigned bits = __float_as_uint(x), e = bits >> 23, j = (bits >> 15) & 255u;
   const float4 B = __ldg(reinterpret_cast<const float4 *>(c.tab) + j);
   const float2 A = __ldg(reinterpret_cast<const float2 *>(c.tab + 1024) + e);
@@ -148,8 +148,13 @@ __device__ __forceinline__ float pow_pair(float x, const PowPair &c) {
   const float Ph = A.x * B.x, Pl = fmaf(A.x, B.y, fmaf(A.y, B.x, fmaf(A.x, B.x, -Ph)));
   const float yh = Ph * sh;
   const float yl = fmaf(Ph, sl, fmaf(Pl, sh, fmaf(Ph, sh, -yh) + Pl));
-  const float r = Ph + yh;
-  return r + ((yh - (r - Ph)) + yl);
+  hi = Ph + yh;
+  lo = (yh - (hi - Ph)) + yl;
+}
+__device__ __forceinline__ float pow_pair(float x, const PowPair &c) {
+  float hi, lo;
+  pow_pair_parts(x, c, hi, lo);
+  return hi + lo;
 }
 
 // x^m in FP32 for the FP32-deviation form: 2^(m log2 x) with CUDA's log2f

@@ -44,6 +44,7 @@
 #include <cstdint>
 
 #include "d2q9.cuh"
+#include "implicit.cuh"
 #include "internal.h"
 #include "launch.cuh"
 #include "reduce.cuh"
@@ -433,6 +434,13 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
   const PowPair pw = {a.powp + int64_t(task.cav) * POWP_SIZE, cv.pb1h, cv.pb1l, cv.pb2f, cv.pb3,
                       cv.pb4, cv.pe_lo, cv.pe_n};
   const T wy_in = T(cv.deta), wy_edge = T(0.5 * cv.deta);
+  [[maybe_unused]] const ImplPair ip = impl_pair(cv);
+  [[maybe_unused]] auto solve = [&](T G2, T lam_prev) -> T {  // implicit form of Eq. (2.14)
+    if constexpr (sizeof(T) == 4)
+      return lambda_implicit_pair(G2, lam_prev, ip, pw, cv, a.powtab, powt);
+    else
+      return lambda_implicit(6.0 * sqrt(G2), lam_prev, cv, a.powtab, powt);
+  };
   // Step (2) for this thread's row of iteration `it`: moments, f^eq - f-hat and
   // lambda(t). The row of iteration it + 1 is formed during the full step of
   // iteration it, so that the power overlaps the stencil work.
@@ -457,7 +465,7 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
       if constexpr (P32)
         o.lam = T(lambda_implicit_f32(float(T(2) * sqrt(G2) * ics2), float(lam_prev), cv));
       else
-        o.lam = T(lambda_implicit(2.0 * sqrt(double(G2)) * 3.0, double(lam_prev), cv, a.powtab));
+        o.lam = solve(G2, lam_prev);
       return o;
     }
     // Eqs. (2.12)-(2.14), (1.4): strain rate in T, power in FP64, by pairs of

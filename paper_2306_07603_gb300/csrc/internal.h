@@ -49,6 +49,8 @@ struct CavDev {
   // the clamp of the FP32 strain rate, max(largest float <= gamma_min^2, FLT_MIN)
   double pb2;
   float pb3, pb4, pb5, gmin2_f;
+  int impl_f32;             // implicit form: 1 where its values lie in a float's range
+  float g2c_f;              // ... the largest float G2 whose root is the clamp value (ImplPair)
   float pb1h, pb1l, pb2f;   // pow_pair: b1 = m as a pair of floats, b2 rounded
   unsigned pe_lo, pe_n;     // ... and the exponents its table covers
   // FP64 staged kernels (staged64.cu): thread blocks of this cavity and, for the

@@ -18,11 +18,43 @@
 #include <cstdint>
 
 #include "d2q9.cuh"
+#include "implicit.cuh"
 #include "internal.h"
 #include "launch.cuh"
 #include "reduce.cuh"
 
 namespace ifd {
+
+// Relaxation time of Step (2) of the FP32 staged kernels: strain rate from f^ne
+// (Eqs. 2.12-2.13, with f = f(f-hat, lam_prev) of Eq. 2.18), q = |gamma-dot|^2 =
+// 2 D:D, the clamped power law mu = K max(|gamma-dot|, gamma_min)^(n-1)
+// evaluated as K max(q, gamma_min^2)^((n-1)/2) (Eq. 1.4), and lam = mu / c_s^2
+// (Eq. 2.14). Pxx, Pxy, Pyy are sum_i c_ia c_ib (g_i - geq_i). The strain rate
+// is formed in FP32, clamped at cv.gmin2_f; the power law of Eq. (1.4)
+// (pow_tab, FP64 result, error within 6e-16) and the implicit form's solve are
+// FP64, as the FP32-deviation form specifies. With cv.pow32 (an opt-in) they
+// are FP32 instead (pow_f32, lambda_implicit_f32; the clamp at the largest
+// float not above gamma_min^2). powt: the cavity's pow_tab table.
+__device__ __forceinline__ double relaxation_time(float Pxx, float Pxy, float Pyy,
+                                                  float lam_prev, const CavDev &cv,
+                                                  const double *powtab, const double *powt) {
+  if (cv.implicit) {
+    const float G2 = 0.5f * (Pxx * Pxx + 2.0f * Pxy * Pxy + Pyy * Pyy);
+    if (cv.pow32)
+      return double(lambda_implicit_f32(2.0f * sqrtf(G2) * float(cv.inv_cs2), lam_prev, cv));
+    return lambda_implicit(2.0 * sqrt(double(G2)) * cv.inv_cs2, double(lam_prev), cv, powtab,
+                           powt);
+  }
+  // f^ne = 2 lam_prev/(2 lam_prev + dt) (f-hat - f^eq);  S = -sum c c f^ne / (lam_prev c_s^2)
+  const float k = -2.0f / ((2.0f * lam_prev + float(cv.dt)) * float(cv.cs2));
+  const float Sxx = k * Pxx, Sxy = k * Pxy, Syy = k * Pyy;
+  const float q2 = 0.5f * (Sxx * Sxx + 2.0f * Sxy * Sxy + Syy * Syy);
+  if (cv.pow32) {
+    const float q = fmaxf(q2, __double2float_rd(cv.gmin2));
+    return double(float(cv.Kics2) * pow_f32(q, float(cv.half_nm1)));
+  }
+  return pow_tab(fmaxf(q2, cv.gmin2_f), powt, cv.half_nm1, cv.pb2, cv.pb3, cv.pb4, cv.pb5);
+}
 
 struct ReduceArgs {
   const CavDev *cav;

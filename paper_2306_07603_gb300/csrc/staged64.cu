@@ -24,6 +24,7 @@
 #include <cstdint>
 
 #include "d2q9.cuh"
+#include "implicit.cuh"
 #include "internal.h"
 #include "launch.cuh"
 #include "reduce.cuh"
@@ -64,7 +65,8 @@ __global__ void __launch_bounds__(NT, MIN_BLOCKS<NT>) k_collide64(StepArgs a) {
   const double pp = fma(pxx, pxx, fma(pyy, pyy, (pxy + pxy) * pxy));
   double lam;
   if (cv.implicit) {
-    lam = lambda_implicit(2.0 * cv.c * cv.c * sqrt(0.5 * pp) * cv.inv_cs2, lam_prev, cv, a.powtab);
+    lam = lambda_implicit(2.0 * cv.c * cv.c * sqrt(0.5 * pp) * cv.inv_cs2, lam_prev, cv, a.powtab,
+                          a.powt + int64_t(r.cav) * POWT_SIZE);
   } else {
     // Eqs. (2.12)-(2.13) with f = f(f-hat, lam_prev) of Eq. (2.18): |gamma-dot|^2 =
     // 2 D:D = k^2 pp c^4 / 2 with k = -2 / ((2 lam_prev + dt) c_s^2)

@@ -92,20 +92,18 @@ __device__ __forceinline__ bool zero(double x) { return (__double_as_longlong(x)
 __device__ __forceinline__ bool nonpositive(double x) { return negative(x) || zero(x); }
 __device__ __forceinline__ bool nonnegative(double x) { return !negative(x) || zero(x); }
 
-// The power law of Eq. (1.4), K/c_s^2 max(q, gmin2)^m, for an FP64 strain
-// rate: the table-driven binomial form of pow_tab (fastpow.cuh) on the full
-// FP64 fraction f of q = 2^e f. As there, t = f (1/c_j) - 1 carries the
-// rounding of 1/c_j (<= 1.2e-16 absolute) and one of its own below 2^-62, the
-// tail's coefficient is FP32, and the result is within 6e-16: closer than
-// pow_fast's 5e-16 + 2.2e-16 |m log2 q|, with 6 FP64 instructions instead of
-// ~22. The table covers the exponents of a normal float; an argument
-// beyond them (or a NaN, which the clamp replaces) takes pow_fast.
-__device__ __forceinline__ double power_law64(double q, const CavDev &cv, const double *powtab,
-                                              const double *__restrict__ powt) {
-  const double qc = __double_as_longlong(q) > __double_as_longlong(cv.gmin2) ? q : cv.gmin2;
-  const int hi = __double2hiint(qc), lo = __double2loint(qc);
+// K/c_s^2 q^m, m = (n-1)/2, for an FP64 argument q > 0: the table-driven binomial
+// form of pow_tab (fastpow.cuh) on the full FP64 fraction f of q = 2^e f. As
+// there, t = f (1/c_j) - 1 carries the rounding of 1/c_j (<= 1.2e-16 absolute) and
+// one of its own below 2^-62, the tail's coefficient is FP32, and the result is
+// within 6e-16: closer than pow_fast's 5e-16 + 2.2e-16 |m log2 q|, with 6 FP64
+// instructions instead of ~22. The table covers the exponents of a normal
+// float; an argument beyond them (or a NaN) takes pow_fast.
+__device__ __forceinline__ double power64(double q, const CavDev &cv, const double *powtab,
+                                          const double *__restrict__ powt) {
+  const int hi = __double2hiint(q), lo = __double2loint(q);
   if (unsigned(hi - (897 << 20)) >= unsigned(254 << 20))
-    return cv.Kics2 * pow_fast(q > cv.gmin2 ? q : cv.gmin2, cv.half_nm1, powtab);
+    return cv.Kics2 * pow_fast(q, cv.half_nm1, powtab);
   const unsigned e = (unsigned(hi) >> 20) - 896u, j = (unsigned(hi) >> 12) & 255u;
   const int fh = (hi & 0x000FFFFF) | 0x3FF00000;
   const double2 dr = __ldg(reinterpret_cast<const double2 *>(powt) + j);
@@ -116,6 +114,13 @@ __device__ __forceinline__ double power_law64(double q, const CavDev &cv, const 
   const double w = fma(t, fma(t, widen(c3), cv.pb2), cv.half_nm1);
   const double P = __ldg(powt + 512 + e) * dr.x;
   return fma(P, t * w, P);
+}
+// The power law of Eq. (1.4), K/c_s^2 max(q, gmin2)^m (a NaN is clamped).
+__device__ __forceinline__ double power_law64(double q, const CavDev &cv, const double *powtab,
+                                              const double *__restrict__ powt) {
+  const long long b = __double_as_longlong(q);
+  const bool above = b > __double_as_longlong(cv.gmin2) && b <= 0x7FF0000000000000ll;
+  return power64(above ? q : cv.gmin2, cv, powtab, powt);
 }
 
 // Moments of a deviation set in lattice units: m = sum e_i g_i (u = c m) and
