@@ -42,11 +42,11 @@ __device__ __forceinline__ void cluster_done() {
 }
 
 template <class Args>
-inline void launch_after(void (*kernel)(Args), int grid, int block, int smem, cudaStream_t s,
+inline void launch_after(void (*kernel)(Args), int grid, dim3 block, int smem, cudaStream_t s,
                          const Args &args, int cluster = 1) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(grid));
-  cfg.blockDim = dim3(unsigned(block));
+  cfg.blockDim = block;
   cfg.dynamicSmemBytes = size_t(smem);
   cfg.stream = s;
   cudaLaunchAttribute attr[2] = {};

@@ -6,6 +6,7 @@
 // Host code never uses the array's name as a pointer: its device address is
 // taken once per device with cudaGetSymbolAddress (with that device current)
 // and passed to the kernels.
+#include <algorithm>
 #include <cstdio>
 #include <mutex>
 
@@ -18,6 +19,12 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kMaxBlocks = IFDLBM_STATIC_MAX_NODES / kThreads;  // 8192 partial slots
 constexpr int kMaxDevices = 64;
+// Blocks of k_field_partials: 4 on each of the 152 SMs, each thread taking every
+// 608 x 256th node. A block's reduction then costs the FP64 pipe once per some
+// nodes instead of once per node, and the second kernel has 608 slots at most
+// (1025^2: 89 + 24 -> 40 + 10 us, from a cold cache).
+constexpr int kBlocks = 608;
+static_assert(kBlocks <= kMaxBlocks, "partial slots");
 
 // 8192 slots x 8 doubles = 512 KiB per device.
 static __device__ __align__(256) double g_static_partials[kMaxBlocks * ifd::NPART];
@@ -28,17 +35,22 @@ double *g_addr[kMaxDevices] = {nullptr};
 __global__ void __launch_bounds__(kThreads)
     k_field_partials(int64_t n, const double *u1, const double *v1, const double *p1,
                      const double *u0, const double *v0, const double *p0, double *part) {
-  const int64_t k = int64_t(blockIdx.x) * kThreads + threadIdx.x;
   ifd::Partial p = {0, 0, 0, 0, 0, 0, 0};
-  if (k < n) {
-    const double du = u1[k] - u0[k], dv = v1[k] - v0[k], dP = p1[k] - p0[k];
-    p.du2 = du * du + dv * dv;
-    p.u2 = u1[k] * u1[k] + v1[k] * v1[k];
-    p.dP2 = dP * dP;
-    p.P2 = p1[k] * p1[k];
-    p.du2max = p.du2;
-    p.u2max = p.u2;
+  long long m0 = -1, m1 = -1;   // maxima as max_key (no node: as a NaN)
+  for (int64_t k = int64_t(blockIdx.x) * kThreads + threadIdx.x; k < n;
+       k += int64_t(gridDim.x) * kThreads) {
+    const double u = u1[k], v = v1[k], P = p1[k];
+    const double du = u - u0[k], dv = v - v0[k], dP = P - p0[k];
+    const double du2 = du * du + dv * dv, u2 = u * u + v * v;
+    p.du2 += du2;
+    p.u2 += u2;
+    p.dP2 += dP * dP;
+    p.P2 += P * P;
+    m0 = max(m0, ifd::max_key(du2));
+    m1 = max(m1, ifd::max_key(u2));
   }
+  p.du2max = __longlong_as_double(m0);
+  p.u2max = __longlong_as_double(m1);
   ifd::block_partial<kThreads / 32>(p, part, blockIdx.x);
 }
 
@@ -100,7 +112,7 @@ extern "C" int ifdlbm_residual_fields_static(int nx, int ny, const double *u1, c
   double *part = nullptr;
   int rc = scratch_address(&part);
   if (rc) return rc;
-  const int nblocks = int((n + kThreads - 1) / kThreads);
+  const int nblocks = int(std::min<int64_t>((n + kThreads - 1) / kThreads, kBlocks));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   (void)cudaGetLastError();  // a launch error left by earlier, unrelated work is not this call's
   k_field_partials<<<nblocks, kThreads, 0, s>>>(n, u1, v1, p1, u0, v0, p0, part);

@@ -393,64 +393,109 @@ __global__ void __launch_bounds__(TILE_X *TILE_Y) k_init(const CavDev *cavs, con
   lam[cv.off + node] = T(cv.lam0);
 }
 
-// Macros at every node and the stream function. A block is 32 xi = const
-// lines x MSEG row segments. Pass 1: rho, u, v and the integrand
-// I = u y_eta - v x_eta at every node (I parked in psi). Pass 2: each thread
-// sums the trapezoid intervals (I_j + I_{j-1}) deta / 2 of its segment. The
-// segment sums are scanned in a fixed order in shared memory, and pass 3
-// writes psi_j = psi_{j-1} + (I_j + I_{j-1}) deta / 2 from the segment's
-// offset (psi = 0 on the bottom wall).
-constexpr int MSEG = 32;
+// double(x) by integer instructions (the conversion would take the FP64 pipe):
+// normal arguments by widen, infinities and NaNs with the largest exponent, zeros
+// and subnormals scaled by 2^64 first.
+__device__ __forceinline__ double to_double(float x) {
+  const int b = __float_as_int(x), s = b & int(0x80000000u), m = b & 0x7FFFFFFF;
+  const int t = __float_as_int(x * 0x1p64f) & 0x7FFFFFFF;
+  const bool small = m < 0x00800000, large = m >= 0x7F800000;
+  const int f = small ? t : m;
+  const int e = large ? (2047 - 255) << 20 : (small ? (896 - 64) << 20 : 896 << 20);
+  const int hi = f == 0 ? 0 : (f >> 3) + e;
+  return __hiloint2double(s | hi, f << 29);
+}
+__device__ __forceinline__ double to_double(double x) { return x; }
 
-template <class T>
-__global__ void __launch_bounds__(32 * MSEG)
-    k_macros(const CavDev *cavs, Geo geo, int cavity, const double *pref, const T *g,
-             double *rho, double *u, double *v, double *psi) {
-  const CavDev &cv = cavs[cavity];
-  const double p0 = pref[cavity];
-  const int i = blockIdx.x * 32 + threadIdx.x;
-  const int seg = (cv.ny + MSEG - 1) / MSEG;
-  const int j0 = threadIdx.y * seg, j1 = min(cv.ny, j0 + seg);
+struct MacrosArgs {
+  const CavDev *cav;
+  Geo geo;
+  int cavity;
+  const double *pref;
+  const void *g;
+  double *rho, *u, *v, *psi;
+};
+
+// Macros at every node and the stream function psi_j = deta (sum_{k <= j} I_k -
+// (I_0 + I_j) / 2), I = u y_eta - v x_eta (trapezoidal rule, psi = 0 on the bottom
+// wall). A cluster of CS blocks holds 32 xi = const lines, each block a share of
+// the rows in MSEG segments. Pass 1: rho, u, v and I at every node (I parked in
+// psi), and the segment's sum of I. The sums of the segments below, in the block
+// and in the cluster's blocks before it, give each segment its offset, and pass
+// 2 writes psi. Bound by the FP64 pipe (8 instructions a node) and the bytes
+// about alike; one block per 32 lines left 119 of the 152 SMs
+// idle (1025^2: 157 us, now 71, both from a cold cache).
+constexpr int MSEG = 32;
+constexpr int MACROS_CS = 8;
+
+template <class T, int CS, bool GEN>
+__global__ void __launch_bounds__(32 * MSEG) k_macros(MacrosArgs a) {
+  const CavDev &cv = a.cav[a.cavity];
+  const int i = int(blockIdx.x / CS) * 32 + threadIdx.x, r = blockIdx.x % CS;
+  const int w = threadIdx.y;
+  const int seg = (cv.ny + CS * MSEG - 1) / (CS * MSEG);
+  const int j0 = min(cv.ny, (r * MSEG + w) * seg), j1 = min(cv.ny, j0 + seg);
   const bool col = i < cv.nx;
-  const T *gb = g + 9 * cv.off;
-  const double *gm = cv.general ? geo.gmet + 7 * cv.off : nullptr;
-  __shared__ double part[MSEG][32];
+  const int64_t plane = cv.plane, pitch = cv.pitch, nx = cv.nx;
+  const double rho0 = cv.rho0, ics2 = cv.inv_cs2, H = cv.H, deta = cv.deta;
+  const T c = T(cv.c), cs2 = T(cv.cs2);
+  const double xeta = col && !GEN ? a.geo.xeta[cv.goff + i] : 0.0;
+  const double *gm = GEN ? a.geo.gmet + 7 * cv.off : nullptr;
+  __shared__ double part[MSEG][33];  // (a line's sums are read along it too)
+  __shared__ double below[CS][32];   // (first block's: the blocks' totals)
+  previous_done();
+  dependents_may_start();
+  const double p0 = a.pref[a.cavity];
+  const T *gb = (const T *)a.g + 9 * cv.off;
+  double sum = 0.0;
   for (int j = j0; col && j < j1; ++j) {
     T gg[9];
-    load9(gb, cv.plane, int64_t(j) * cv.pitch + i, gg);
+    const int64_t nd = j * pitch + i, o = j * nx + i;
+    load9(gb, plane, nd, gg);
     T ux, uy, P;
-    moments(gg, T(cv.c), T(cv.cs2), ux, uy, P);
-    const int64_t o = int64_t(j) * cv.nx + i;
-    if (rho) rho[o] = cv.rho0 + (p0 + double(P)) * cv.inv_cs2;
-    if (u) u[o] = double(ux);
-    if (v) v[o] = double(uy);
-    const int64_t nd = int64_t(j) * cv.pitch + i;
-    if (psi)
-      psi[o] = cv.general ? double(ux) * gm[5 * cv.plane + nd] - double(uy) * gm[4 * cv.plane + nd]
-                          : double(ux) * cv.H - double(uy) * geo.xeta[cv.goff + i];
-  }
-  if (!psi) return;  // uniform over the launch
-  __syncthreads();   // every integrand of the block's lines is written
-  double sum = 0.0, Iprev = 0.0;
-  if (col && j0 < j1) {
-    Iprev = j0 > 0 ? psi[int64_t(j0 - 1) * cv.nx + i] : 0.0;
-    double Ip = Iprev;
-    for (int j = j0; j < j1; ++j) {
-      const double I = psi[int64_t(j) * cv.nx + i];
-      if (j > 0) sum += 0.5 * (I + Ip) * cv.deta;
-      Ip = I;
+    moments(gg, c, cs2, ux, uy, P);
+    const double ud = to_double(ux), vd = to_double(uy);
+    if (a.rho) a.rho[o] = rho0 + (p0 + to_double(P)) * ics2;
+    if (a.u) a.u[o] = ud;
+    if (a.v) a.v[o] = vd;
+    if (a.psi) {
+      double I;
+      if constexpr (GEN)
+        I = ud * gm[5 * plane + nd] - vd * gm[4 * plane + nd];
+      else
+        I = ud * H - vd * xeta;
+      a.psi[o] = I;
+      sum += I;
     }
   }
-  part[threadIdx.y][threadIdx.x] = sum;
-  __syncthreads();   // segment sums published; every integrand has been read
+  if (!a.psi) return;  // uniform over the launch
   double acc = 0.0;
-  for (int k = 0; k < int(threadIdx.y); ++k) acc += part[k][threadIdx.x];
+  if (r == 0 && w == 0 && col) acc = -0.5 * a.psi[i];  // I_0 counts half
+  part[w][threadIdx.x] = sum + acc;
+  __syncthreads();
+  {  // sums of the segments up to each, along every line: warp w takes line w
+    double v = part[threadIdx.x][w];
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2) {
+      const double b = __shfl_up_sync(0xffffffffu, v, o);
+      if (int(threadIdx.x) >= o) v += b;
+    }
+    part[threadIdx.x][w] = v;
+  }
+  __syncthreads();
+  if (w > 0) acc = part[w - 1][threadIdx.x];
+  if constexpr (CS > 1) {
+    if (w == MSEG - 1) cluster_at<CS>(&below[r][0])[threadIdx.x] = part[w][threadIdx.x];
+    cluster_done<CS>();
+    const double *all = cluster_at<CS>(&below[0][0]);
+    for (int b = 0; b < r; ++b) acc += all[b * 32 + threadIdx.x];
+    cluster_done<CS>();   // the first block's memory is there until all have read it
+  }
   for (int j = j0; col && j < j1; ++j) {
-    const int64_t o = int64_t(j) * cv.nx + i;
-    const double I = psi[o];
-    if (j > 0) acc += 0.5 * (I + Iprev) * cv.deta;
-    Iprev = I;
-    psi[o] = acc;
+    const int64_t o = j * nx + i;
+    const double I = a.psi[o];
+    acc += I;
+    a.psi[o] = deta * (acc - 0.5 * I);
   }
 }
 
@@ -759,9 +804,15 @@ template <class T> void launch_init(const CavDev *cav, const int *tile_cav, void
 template <class T> void launch_macros(const CavDev *cav, Geo geo, int cavity, const double *pref,
                                       const void *g, double *rho, double *u, double *v,
                                       double *psi, int nx, int ny, cudaStream_t s) {
-  (void)ny;
-  k_macros<T><<<(nx + 31) / 32, dim3(32, MSEG), 0, s>>>(cav, geo, cavity, pref, (const T *)g,
-                                                        rho, u, v, psi);
+  // (a cluster's blocks get a row per thread from 8 x 32 rows on)
+  const MacrosArgs a{cav, geo, cavity, pref, g, rho, u, v, psi};
+  const int lines = (nx + 31) / 32;
+  const dim3 block(32, MSEG);
+  if (ny >= MACROS_CS * MSEG)
+    launch_after(geo.gmet ? k_macros<T, MACROS_CS, true> : k_macros<T, MACROS_CS, false>,
+                 lines * MACROS_CS, block, 0, s, a, MACROS_CS);
+  else
+    launch_after(geo.gmet ? k_macros<T, 1, true> : k_macros<T, 1, false>, lines, block, 0, s, a);
 }
 template <class T> void launch_export(const CavDev *cav, int cavity, const double *pref,
                                       const void *g, const void *lam, double *fhat,
