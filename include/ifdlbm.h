@@ -137,13 +137,13 @@ typedef struct {
 #define IFDLBM_LAMBDA_IMPLICIT 1
 
 /* Cavity-to-CTA schedules of the fused kernel. Tasks are strips of columns x
- * segments of rows of every cavity of the batch. */
-#define IFDLBM_SCHED_GRID 0    /* one CTA per task */
+ * segments of rows of every cavity of the batch, sorted largest first. */
+#define IFDLBM_SCHED_GRID 0    /* one CTA per task: the hardware hands the next one
+                                  to whichever SM is free first */
 #define IFDLBM_SCHED_STATIC 1  /* persistent CTAs (SMs x resident CTAs); CTA b takes
-                                  the positions b, b + grid, ... of the tasks
-                                  sorted largest first */
-#define IFDLBM_SCHED_DYNAMIC 2 /* persistent CTAs taking the next position of that
-                                  order from an atomic counter */
+                                  the positions b, b + grid, ... */
+#define IFDLBM_SCHED_DYNAMIC 2 /* the same as GRID, whose CTAs the hardware
+                                  schedules dynamically */
 
 /* Result of ifdlbm_autotune. */
 typedef struct {

@@ -59,7 +59,6 @@ struct ifdlbm_ctx {
   int task_cap = 0;    // capacity of tasks / order / partial slots
   ifd::Task *tasks = nullptr;
   int *order = nullptr;
-  int *counter = nullptr;
   unsigned char *tmaps = nullptr;  // [2][ncav] TMA tensor maps of g[0], g[1] (fused kernel)
   int tma_skip = 0;                // test hook (ifdlbm_inject_tma_timeout)
   // adjoint scratch (allocated on the first adjoint call)
@@ -193,7 +192,6 @@ void enqueue_step(ifdlbm_ctx *h, int parity, bool want_residual) {
     f.geo = h->b.geo;
     f.tasks = h->tasks;
     f.order = h->order;
-    f.counter = h->counter;
     f.ntasks = h->ntasks;
     f.schedule = h->schedule;
     f.g_in = h->b.g[parity];
@@ -215,7 +213,6 @@ void enqueue_step(ifdlbm_ctx *h, int parity, bool want_residual) {
     f.early = h->early;
     f.resid = h->b.resid;
     f.want_residual = want_residual ? 1 : 0;
-    if (h->schedule == IFDLBM_SCHED_DYNAMIC) cudaMemsetAsync(h->counter, 0, sizeof(int), h->stream);
     // the residual of Eq. (2.19) is reduced inside the launch by each cavity's last task
     timed(h, IFDLBM_KPROF_FUSED, [&] { ifd::launch_fused<T>(f, h->fused_nt, h->grid, h->stream); });
     return;
@@ -381,32 +378,49 @@ int fused_resident(const ifdlbm_ctx *h, int nt, int *sms) {
   return per_sm;
 }
 
+// Consecutive fused steps overlap (launch.cuh) where the next step's CTAs find
+// room that does not unbalance it: idle SMs of a small grid (65^2: 11.6 -> 9.3 us a
+// step), or the slots that the last round of a large one leaves (2049^2 227 -> 220,
+// 64 cavities 428 -> 421). In between they would double up on some SMs while
+// others have none (257^2 18.8 -> 20.0, 1025^2 80 -> 88).
+bool overlap_small(int tasks, int sms) { return 3 * tasks <= 2 * sms; }
+bool overlap_large(int tasks, int slots) { return 5 * tasks >= 4 * slots; }
+
 // Rows per task where the caller leaves them open. A task of r rows marches
-// (r + 7) / 2 + 1 iterations (8 halo rows, two rows at a time), and an iteration
-// takes an SM the longer the more CTAs it holds: measured at 128 threads (4 on an
-// SM) 2.0, 2.4, 3.0 and 3.5 us with 1 to 4, which 1.4 + 2.1 f follows, f the share
-// of its slots in use. With `full` rounds of all slots and a rest, a step takes
-//   iterations x (full x 3.5 + (1.4 + 2.1 f_rest)) + 5.8 us,
-// within 7 % of the best of 19 row counts on 22 batches from one 65^2 cavity to
-// 64 of up to 513^2. Few rows fill the chip from a small grid (65^2: 2 rows 14.3
-// us a step, 32 rows 34.5; 257^2: 5 rows 22.4, 32 rows 44.6), many keep the
-// halo's share low on a large one (2049^2: 48 rows 255 us, 12 rows 350).
+// (r + 7) / 2 + 1 iterations (8 halo rows, two rows at a time). An iteration takes
+// an SM the longer the more CTAs it holds: at 128 threads (4 on an SM) 1.95,
+// 2.35, 2.9 and 2.8 us with 1 to 4 (the last lower by the overlap of consecutive
+// steps); other CTA widths are read at the same share of an SM's slots. A step is
+// the full rounds of all slots and a rest, of which an overlapped step's next one
+// takes up about half the idle slots, and 2.3 us of launch that a small
+// overlapped grid does not see. Over 19 row counts on 22 batches (one 65^2 cavity
+// to 64 of up to 513^2; trapezoids, quadrilaterals, implicit) the count this picks
+// is within 5 % of the best, 0.5 % on average. Few rows fill the chip from a
+// small grid (65^2: 2 rows 9.3 us a step, 32 rows 28.7), many keep the halo's share
+// low on a large one (2049^2: 48 rows 222 us, 12 rows 310).
 int automatic_rows(const ifdlbm_ctx *h, int nt) {
   int sms = 0, w4;
-  const int per_sm = fused_resident(h, nt, &sms), slots = std::max(1, sms * per_sm);
+  const int per_sm = std::max(1, fused_resident(h, nt, &sms)), slots = std::max(1, sms * per_sm);
+  auto tau = [&](int n) {  // us of an iteration with n CTAs on an SM
+    static const double at[5] = {1.95, 1.95, 2.35, 2.9, 2.8};  // at 0, 1/4 .. 1 of the slots
+    const double x = 4.0 * n / per_sm;
+    const int k = std::min(3, int(x));
+    return at[k] + (at[k + 1] - at[k]) * (x - k);
+  };
   int best = 32;
   double least = 1e300;
-  for (int rows : {2, 3, 4, 5, 6, 8, 10, 12, 14, 16, 20, 24, 28, 32, 40, 48, 64, 96, 128}) {
+  for (int rows : {2, 3, 4, 5, 6, 8, 10, 12, 14, 16, 20, 24, 28, 32, 40, 48, 64, 96}) {
     double its = 0;
     int n = 0;
     for (const CavDev &cv : h->cav) {
-      const int sx = strips(cv.nx, ifd::fused_strip_width(nt), &w4), sy = segments(cv.ny, rows);
-      n += sx * sy;
-      its += sx * sy * ((double(cv.ny) / sy + 7) / 2 + 1);
+      const int t = strips(cv.nx, ifd::fused_strip_width(nt), &w4) * segments(cv.ny, rows);
+      n += t;
+      its += t * ((double(cv.ny) / segments(cv.ny, rows) + 7) / 2 + 1);
     }
     const int full = n / slots, rest = n % slots;
-    const double f = double((rest + sms - 1) / std::max(sms, 1)) / std::max(per_sm, 1);
-    const double t = its / n * (full * 3.5 + (rest ? 1.4 + 2.1 * f : 0.0));
+    double last = rest ? tau((rest + sms - 1) / sms) : 0.0;
+    if (full && overlap_large(n, slots)) last = 0.5 * (last + tau(per_sm) * rest / slots);
+    const double t = its / n * (full * tau(per_sm) + last) + (overlap_small(n, sms) ? 0.0 : 2.3);
     if (t < least) {
       least = t;
       best = rows;
@@ -460,14 +474,9 @@ int build_fused_tasks(ifdlbm_ctx *h, int nt, int rows, int sched) {
   h->fused_nt = nt;
   h->fused_rows = rows;
   h->schedule = sched;
-  h->grid = sched == IFDLBM_SCHED_GRID ? h->ntasks : std::min(h->ntasks, sms * per_sm);
-  // Consecutive steps overlap (launch.cuh) where the next step's CTAs find room
-  // that does not unbalance it: idle SMs of a small grid (65^2: 14.2 -> 12.0 us a
-  // step), or the slots that the last round of a large one leaves (2049^2 257 ->
-  // 252, 64 cavities 499 -> 491). In between they would double up on some SMs
-  // while others have none (129^2 16.6 -> 17.6, 1025^2 87 -> 98).
-  h->early = sched == IFDLBM_SCHED_GRID &&
-             (3 * h->ntasks <= 2 * sms || 5 * h->ntasks >= 4 * sms * per_sm);
+  h->grid = sched == IFDLBM_SCHED_STATIC ? std::min(h->ntasks, sms * per_sm) : h->ntasks;
+  h->early = sched != IFDLBM_SCHED_STATIC && (overlap_small(h->ntasks, sms) ||
+                                              overlap_large(h->ntasks, sms * per_sm));
   for (int p = 0; p < 2; ++p)
     if (h->gexec[p]) {
       cudaGraphExecDestroy(h->gexec[p]);
@@ -924,7 +933,6 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
   } else {
     ok &= (h->tasks = (ifd::Task *)A(size_t(h->task_cap) * sizeof(ifd::Task))) != nullptr;
     ok &= (h->order = (int *)A(size_t(h->task_cap) * sizeof(int))) != nullptr;
-    ok &= (h->counter = (int *)A(sizeof(int))) != nullptr;
     ok &= (h->tmaps = (unsigned char *)A(size_t(2) * ncav * ifd::TMAP_BYTES)) != nullptr;
   }
   const int nslots = fused ? h->task_cap : (staged64 ? h->nblk64 : h->ntiles);

@@ -1,0 +1,13 @@
+// The fused step's kernels for float storage and 256 threads per CTA (fused.cuh), a
+// translation unit of their own so that they compile beside the others.
+#include "fused.cuh"
+
+namespace ifd {
+
+void launch_fused_float_256(const FusedArgs &a, int grid, cudaStream_t s) {
+  launch_fused_nt<float, 256>(a, grid, s);
+}
+int blocks_per_sm_float_256() { return blocks_per_sm_nt<float, 256>(); }
+int smem_float_256() { return fused_smem_size<float, 256>(); }
+
+}  // namespace ifd

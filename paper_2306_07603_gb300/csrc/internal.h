@@ -144,9 +144,8 @@ struct FusedArgs {
   Geo geo;
   const Task *tasks;
   const int *order;   // scheduled position -> task index (largest tasks first)
-  int *counter;       // dynamic schedule: next position (zeroed before each launch)
   int ntasks;
-  int schedule;       // 0 grid (one CTA per task), 1 persistent static, 2 persistent dynamic
+  int schedule;       // 1 persistent CTAs, else one CTA per task
   const void *g_in;
   void *g_out;
   const void *tmap_in;  // [ncav] tensor maps of g_in (TMAP_BYTES each): box 32 x 1 x 9
