@@ -191,10 +191,11 @@ class ClockSampler:
 # kernel source it was taken from
 # ---------------------------------------------------------------------------
 KERNEL_SOURCES = {
-    "fused": ["fused.cu", "d2q9.cuh", "fastpow.cuh", "reduce.cuh", "internal.h", "tma.cuh"],
-    "collide": ["staged.cu", "d2q9.cuh", "fastpow.cuh", "reduce.cuh", "internal.h"],
-    "half": ["staged.cu", "d2q9.cuh", "fastpow.cuh", "reduce.cuh", "internal.h"],
-    "full": ["staged.cu", "d2q9.cuh", "fastpow.cuh", "reduce.cuh", "internal.h"],
+    "fused": ["fused.cuh", "d2q9.cuh", "fastpow.cuh", "implicit.cuh", "step64.cuh", "reduce.cuh",
+              "launch.cuh", "internal.h", "tma.cuh"],
+    "collide": ["staged64.cu", "step64.cuh", "implicit.cuh", "fastpow.cuh", "internal.h"],
+    "half": ["staged64.cu", "step64.cuh", "launch.cuh", "internal.h"],
+    "full": ["staged64.cu", "step64.cuh", "reduce.cuh", "launch.cuh", "internal.h"],
 }
 
 
@@ -672,7 +673,7 @@ def run_adjoint_measure(nx=257, ny=257, T=2000, every=100, n=0.75, Re=400.0, the
             "backward_s": round(t_bwd, 4), "gradient_over_forward": round((t_fwd + t_bwd) / t_plain, 2),
             "checkpoint_bytes": ckpt * state_bytes,
             "segment_bytes": every * (state_bytes + inter_bytes),   # states + intermediates
-            "handle_bytes": handle_bytes, "adjoint_scratch_bytes": 4 * 9 * state_bytes // 10,
+            "handle_bytes": handle_bytes, "adjoint_scratch_bytes": 2 * state_bytes,
             "dJ": {"n": float(p.grad[0]), "Re": float(p.grad[1]), "theta_deg": float(p.grad[2])},
             "J": float(J.detach()),
             "keep_all": {"forward_s": round(t_fwd1, 4), "backward_s": round(t_bwd1, 4),

@@ -369,6 +369,28 @@ __global__ void k_adj_seed_psi(AdjArgs a) {
   block_sum<3, TILE_X * TILE_Y / 32>(v, a.ppart, blockIdx.x);
 }
 
+// Column and row tables of the gathers and of the theta partial (Geo), and the
+// cavity of every block of the step's kernels; one block per cavity.
+__global__ void __launch_bounds__(256) k_adj_setup(const CavDev *cavs, Geo geo, int *adj_cav,
+                                                   int *ring_cav) {
+  const CavDev &cv = cavs[blockIdx.x];
+  for (int i = threadIdx.x; i < cv.nx; i += 256) {
+    const double xe = geo.xeH[cv.goff + i];
+    const_cast<double *>(geo.xm)[cv.goff + i] = 1.0 - xe;
+    const_cast<double *>(geo.xp)[cv.goff + i] = 1.0 + xe;
+    const_cast<double *>(geo.z)[cv.goff + i] = 2.0 * (double(i) / (cv.nx - 1)) - 1.0;
+  }
+  for (int j = threadIdx.x; j < cv.ny; j += 256) {
+    const double r = geo.ax[1][cv.goff + j] * cv.dcot;
+    const_cast<double *>(geo.ath1)[cv.goff + j] = r;
+    const_cast<double *>(geo.ath2)[cv.goff + j] =
+        r * (2.0 * cv.H * (double(j) / (cv.ny - 1)) * geo.xix[cv.goff + j]);
+  }
+  for (int b = threadIdx.x; b < cv.nblk_adj; b += 256) adj_cav[cv.adj0 + b] = blockIdx.x;
+  for (int b = threadIdx.x; b < cv.nblk_adj - cv.nblk_core; b += 256)
+    ring_cav[cv.ring0 + b] = blockIdx.x;
+}
+
 // Threads per block NT and registers as in staged64.cu: up to 255 registers on
 // small batches (8 blocks of a warp on an SM; 10, 12 and 14 blocks with fewer
 // registers ran at 0.96-1.04 of its speed), 168 with 128 threads.
@@ -589,6 +611,11 @@ __global__ void __launch_bounds__(256) k_adj_reduce(AdjArgs a) {
 }
 
 static const dim3 kT(TILE_X, TILE_Y);
+
+void launch_adjoint_setup(const CavDev *cav, const Geo &geo, int *adj_cav, int *ring_cav, int ncav,
+                          cudaStream_t s) {
+  k_adj_setup<<<ncav, 256, 0, s>>>(cav, geo, adj_cav, ring_cav);
+}
 
 void launch_adjoint_seed(const AdjArgs &a, cudaStream_t s) {
   k_adj_seed_energy<<<a.ntiles, kT, 0, s>>>(a);

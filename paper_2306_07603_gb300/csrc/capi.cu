@@ -1488,47 +1488,20 @@ int adjoint_ready(ifdlbm_ctx *h) {
         nullptr;
   ok &= (h->adj_tab = (double *)dalloc(h, 5 * GL * sizeof(double))) != nullptr;
   if (!ok) return fail(h, IFDLBM_ERR_OOM, "adjoint: device allocation failed");
-  // column and row tables of the gathers and of the theta partial (Geo), and
-  // the block tables
-  std::vector<double> tab(5 * GL);
-  std::vector<int> blocks;
-  for (int k = 0; k < h->ncav; ++k) blocks.insert(blocks.end(), h->cav[k].nblk_adj, k);
-  for (int k = 0; k < h->ncav; ++k)
-    blocks.insert(blocks.end(), h->cav[k].nblk_adj - h->cav[k].nblk_core, k);
-  for (int k = 0; k < h->ncav; ++k) {
-    const CavDev &cv = h->cav[k];
-    const ifdlbm_geometry &gm = h->spec[k].geom;
-    const double ct = cot_deg(gm.theta_deg);
-    for (int i = 0; i < cv.nx; ++i) {
-      const double z = 2.0 * (double(i) / (cv.nx - 1)) - 1.0;
-      const double xe = gm.H * ct * z / gm.H;
-      tab[cv.goff + i] = 1.0 - xe;
-      tab[GL + cv.goff + i] = 1.0 + xe;
-      tab[2 * GL + cv.goff + i] = z;
-    }
-    for (int j = 0; j < cv.ny; ++j) {
-      const double eta = double(j) / (cv.ny - 1), xix = 1.0 / (gm.L + 2.0 * gm.H * ct * eta);
-      const double r = cv.sxi[1] * xix * cv.dcot;
-      tab[3 * GL + cv.goff + j] = r;
-      tab[4 * GL + cv.goff + j] = r * 2.0 * gm.H * eta * xix;
-    }
-  }
-  cudaError_t e = cudaMemcpyAsync(h->adj_tab, tab.data(), tab.size() * sizeof(double),
-                                  cudaMemcpyHostToDevice, h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(h->adj_blocks, blocks.data(), blocks.size() * sizeof(int),
-                        cudaMemcpyHostToDevice, h->stream);
-  for (double *p : {g1, h->adj_fbarb})
-    if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, 9 * P, h->stream);
-  for (double *p : {h->adj_l1, h->adj_lamb2})
-    if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, P, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);  // the host tables go out of scope
-  if (e != cudaSuccess) return cuda_fail(h, e, "adjoint set-up");
   h->b.geo.xm = h->adj_tab;
   h->b.geo.xp = h->adj_tab + GL;
   h->b.geo.z = h->adj_tab + 2 * GL;
   h->b.geo.ath1 = h->adj_tab + 3 * GL;
   h->b.geo.ath2 = h->adj_tab + 4 * GL;
+  ifd::launch_adjoint_setup(h->b.cav, h->b.geo, h->adj_blocks, h->adj_blocks + h->nblk_adj,
+                            h->ncav, h->stream);
+  g_launches += 1;
+  cudaError_t e = cudaGetLastError();
+  for (double *p : {g1, h->adj_fbarb})
+    if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, 9 * P, h->stream);
+  for (double *p : {h->adj_l1, h->adj_lamb2})
+    if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, P, h->stream);
+  if (e != cudaSuccess) return cuda_fail(h, e, "adjoint set-up");
   h->adj_g1 = g1;
   return IFDLBM_OK;
 }

@@ -533,7 +533,7 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
         S.fb[sb][q][l] = gq + bb * now.d[q];
         sfme[s * SLOT + q * 32] = gq + bp * now.d[q];  // f-hat^+ in place of g
       }
-      if (ar == 0 || ar == ny - 1) {
+      if (RES && (ar == 0 || ar == ny - 1)) {
         const int e = ar == 0 ? 0 : 1;
         S.edge[e][0][l] = now.ux;
         S.edge[e][1][l] = now.uy;
@@ -603,7 +603,8 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
         if (hi) {                                                     // (ny-1, c): the lid
 #pragma unroll
           for (int q = 0; q < 9; ++q) W[q] = fh[q];
-          nee(W, Uw, Uwy, c_, cs2, ics2);
+          const volatile CavDev &cvl = cv;
+          nee(W, T((GEN ? cvl.lid_ux : cvl.U) / cvl.c), GEN ? T(cvl.lid_uy / cvl.c) : T(0), c_, cs2, ics2);
 #pragma unroll
           for (int q = 0; q < 9; ++q) S.lid[q][l] = W[q];
         }
@@ -699,7 +700,9 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
 #pragma unroll
           for (int q = 0; q < 9; ++q) F[q] = gnv[q];
         }
-        nee(F, (top && inner_c) ? Uw : T(0), (top && inner_c) ? Uwy : T(0), c_, cs2, ics2);
+        const volatile CavDev &cvl = cv;
+        nee(F, (top && inner_c) ? T((GEN ? cvl.lid_ux : cvl.U) / cvl.c) : T(0),
+            (GEN && top && inner_c) ? T(cvl.lid_uy / cvl.c) : T(0), c_, cs2, ics2);
         const int r = bottom ? 0 : ny - 1;
         const int64_t nd = int64_t(r) * pitch + c;
 #pragma unroll

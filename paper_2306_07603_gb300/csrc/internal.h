@@ -220,6 +220,9 @@ struct AdjArgs {
   int ntiles, ncav, nblk, nblk_adj, nblk_ring, nt;
   int most;                  // largest number of blocks of a cavity (launch_residual_reduce)
 };
+// Fills the tables xm, xp, z, ath1 and ath2 of geo and the block tables.
+void launch_adjoint_setup(const CavDev *cav, const Geo &geo, int *adj_cav, int *ring_cav, int ncav,
+                          cudaStream_t s);
 void launch_adjoint_seed(const AdjArgs &a, cudaStream_t s);
 void launch_adjoint_seed_psi(const AdjArgs &a, cudaStream_t s);
 void launch_adjoint_step(const AdjArgs &a, cudaStream_t s);
