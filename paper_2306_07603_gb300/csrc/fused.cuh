@@ -57,7 +57,7 @@ namespace ifd {
 namespace {
 
 constexpr int PF = 5;     // per-thread row slots: prefetched state, then f-hat^+
-constexpr int LEAF = 16;  // rows per leaf sum of the residual terms
+constexpr int LEAF = 16;  // iterations per leaf sum of the residual terms
 constexpr int RING = 6;   // rows of the f-bar^+ and f(t+dt/2) rings
 
 template <class T, int NT>
@@ -265,30 +265,28 @@ struct AdvectAllGen {
   }
 };
 
-// Residual terms of one node, summed over up to LEAF rows in T before they
-// are added to the FP64 partials (a leaf sum; every sum beyond it is FP64).
+// Residual terms of one thread, summed over LEAF iterations of the march (a row
+// each, and a wall row at most) in T; the warp then adds them, in FP64, to its sums
+// in shared memory (leaf_flush). Every sum beyond a leaf is FP64.
 template <class T>
 struct Leaf {
   T du2 = 0, u2 = 0, dP2 = 0, P2 = 0, ek = 0;
   T du2max = 0, u2max = 0;  // maxima are exact in any precision
-  int n = 0;
 };
 
+// Adds the warp's leaves to its five sums `acc`; every lane calls it.
 template <class T>
-__device__ __forceinline__ void leaf_flush(Leaf<T> &l, Partial &p) {
-  p.du2 += double(l.du2);
-  p.u2 += double(l.u2);
-  p.dP2 += double(l.dP2);
-  p.P2 += double(l.P2);
-  p.ek += double(l.ek);
+__device__ __forceinline__ void leaf_flush(Leaf<T> &l, double *acc, int lane) {
+  const double v[8] = {double(l.du2), double(l.u2), double(l.dP2), double(l.P2), double(l.ek)};
+  const double s = warp_sums8(v);
+  if ((lane & 3) == 0 && lane < 20) acc[lane >> 2] += s;
   l.du2 = l.u2 = l.dP2 = l.P2 = l.ek = T(0);
-  l.n = 0;
 }
 
 // In units of c. P1, P0 are pressures of the stored deviations; Pr their
 // reference (the pressure of Eq. 2.11 is Pr + P), which cancels in the difference.
 template <class T>
-__device__ __forceinline__ void leaf_add(Leaf<T> &l, Partial &p, T u1, T v1, T P1, T u0, T v0,
+__device__ __forceinline__ void leaf_add(Leaf<T> &l, T u1, T v1, T P1, T u0, T v0,
                                          T P0, T Pr, T wJ, unsigned *status) {
   if (!(isfinite(u1) && isfinite(v1))) atomicOr(status, 1u);
   const T du = u1 - u0, dv = v1 - v0, dP = P1 - P0;
@@ -301,7 +299,6 @@ __device__ __forceinline__ void leaf_add(Leaf<T> &l, Partial &p, T u1, T v1, T P
   l.ek += T(0.5) * wJ * u2;
   l.du2max = max(l.du2max, du2);
   l.u2max = max(l.u2max, u2);
-  if (++l.n == LEAF) leaf_flush(l, p);
 }
 
 }  // namespace
@@ -380,8 +377,12 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
   // live values spill there)
   constexpr bool FASTQ = !GEN;
 
-  Partial p = {0, 0, 0, 0, 0, 0, 0};
+  // The sums of the residual are kept per warp in shared memory (five FP64 values a
+  // thread would take 10 registers through the march: 64 cavities 504 us a step with
+  // the residual formed in every one, 500 so).
+  __shared__ double racc[RES ? NT / 32 : 1][7];
   Leaf<T> leaf;
+  if (RES && a.want_residual && (threadIdx.x & 31) < 7) racc[threadIdx.x >> 5][threadIdx.x & 31] = 0.0;
 
   const int kb = j0 - 4;
   const int rlo = max(kb, 0), rhi = min(j1 + 3, ny - 1);   // rows of stage A
@@ -685,7 +686,7 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
         else
           Jo = J2o;
         const T wJ = wx * wy_in * Jo;
-        leaf_add(leaf, p, ux, uy, P, u0, v0, P0, Pr, wJ, a.status);
+        leaf_add(leaf, ux, uy, P, u0, v0, P0, Pr, wJ, a.status);
       }
       // wall rows produced with their neighbour rows
       const bool bottom = o == 1 && j0 == 0;
@@ -717,11 +718,12 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
           else
             Jr = row_jac(r);
           const T wJ = wx * wy_edge * Jr;
-          leaf_add(leaf, p, wx2, wy2, wP2, S.edge[e][0][l], S.edge[e][1][l], S.edge[e][2][l], Pr,
+          leaf_add(leaf, wx2, wy2, wP2, S.edge[e][0][l], S.edge[e][1][l], S.edge[e][2][l], Pr,
                    wJ, a.status);
         }
       }
     }
+    if (RES && a.want_residual && it % LEAF == LEAF - 1) leaf_flush(leaf, racc[wid], lane);
     // this iteration's reads and writes of the warp's boxes are ordered before
     // the TMA copies that refill them after the next barrier
     fence_proxy_async_smem();
@@ -732,17 +734,21 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
   if (gave_up && issue)
     for (int s = 0; s < PF; ++s) mbar_wait(&S.bar[s][wid], ((phase >> s) & 1u) ^ 1u);
   if (RES && a.want_residual) {
-    leaf_flush(leaf, p);
-    // from units of c
-    const double c2 = cvc * cvc, c4 = c2 * c2;
-    p.du2 *= c2;
-    p.u2 *= c2;
-    p.ek *= c2;
-    p.dP2 *= c4;
-    p.P2 *= c4;
-    p.du2max = c2 * double(leaf.du2max);
-    p.u2max = c2 * double(leaf.u2max);
-    block_partial<NT / 32>(p, a.part, ti);
+    leaf_flush(leaf, racc[wid], lane);
+    const long long m0 = warp_max_key(max_key(double(leaf.du2max)));
+    const long long m1 = warp_max_key(max_key(double(leaf.u2max)));
+    if (lane == 0) {
+      racc[wid][5] = __longlong_as_double(m0);
+      racc[wid][6] = __longlong_as_double(m1);
+    }
+    __syncthreads();
+    if (threadIdx.x < 7) {   // over the warps, and from units of c
+      const int k = threadIdx.x;
+      double v = racc[0][k];
+      for (int w = 1; w < NT / 32; ++w) v = k < 5 ? v + racc[w][k] : fmax(v, racc[w][k]);
+      const double c2 = cvc * cvc;
+      a.part[int64_t(ti) * NPART + k] = v * (k == 2 || k == 3 ? c2 * c2 : c2);
+    }
     // The last task of the cavity to finish reduces the cavity's partials
     // (a counter, no waiting: every other CTA just moves on).
     __shared__ int last;
@@ -775,10 +781,10 @@ struct Occ {
 // taking positions from an atomic counter, with its reset before each launch,
 // ran 64 uneven cavities in 502 us a step where the first form took 485; in the
 // order of the tasks instead of largest first it takes 6 % more.)
-// RES: whether the residual can be asked for. The partials it accumulates take 22
-// registers through the whole march, which the steps before the last of a call
-// then have for their loads: 64 cavities 502 -> 422 us a step (with the task order
-// above), 2049^2 252 -> 220, ten 257^2 62 -> 56, ten quadrilaterals 76 -> 70.
+// RES: whether the residual can be asked for. Its moments, its sums and the
+// registers they take are then out of the steps before the last of a call: 64
+// cavities 502 -> 422 us a step (with the task order above), 2049^2 252 -> 220, ten
+// 257^2 62 -> 56, ten quadrilaterals 76 -> 70.
 template <class T, int NT, bool IMPL, bool GEN, bool P32, bool PERSIST, bool RES>
 __global__ void __launch_bounds__(NT, Occ<T, NT>::blocks) k_fused(FusedArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
