@@ -6,7 +6,7 @@
 // h = 0 takes the even rows of the march, half h = 1 the odd ones. Iteration
 // k (k = j0 - 4, j0 - 2, ...) runs, in half h,
 //
-//   stage A  row k + h     moments, f^eq, lagged power-law lambda (FP64 power),
+//   stage A  row k + h     moments, f^eq, lagged power-law lambda (pow_pair),
 //                          f-hat^+ (Eq. 2.15), f-bar^+ (Eq. 2.16)
 //   stage 1  row k - 2 + h half step f-bar(t+dt/2) (Eq. 3.7), its moments,
 //                          f(t+dt/2) (Eq. 2.17); wall values by extrapolation
@@ -37,10 +37,9 @@
 // (write_ghosts), written by the node that reads them, instead of per-plane
 // selects on the wall flags.
 //
-// FP64 work per node is kept to the power of Eq. (1.4) and the residual
-// accumulation: GB300 issues FP64 at 1/64 of the FP32 rate. With the pow32
-// opt-in of the FP32 form the power is FP32 too (pow_f32), and the FP64 work
-// is the conversion of lambda, whose plane is FP64, and the residual.
+// In FP32 the power of Eq. (1.4) is evaluated in pairs of floats (pow_pair), so that
+// only the residual's sums are left on the FP64 pipe: GB300 issues FP64 at 1/64 of
+// the FP32 rate. With the pow32 opt-in the power is plain FP32 (pow_f32).
 #pragma once
 #include <cstdint>
 
