@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(NT, ADJ_BLOCKS<NT>) k_adj_half(AdjArgs a) {
 
 // Per cavity, by a cluster of CS blocks (k_residual_reduce): dparams[cav][0..2]
 // += the sums of n3 triples of p3 and, for theta, of n1 values of p1, in a
-// fixed order.
+// fixed order. The kernel has called cluster_arrive().
 template <int CS>
 __device__ __forceinline__ void reduce_params(const double *p3, int n3, const double *p1, int n1,
                                               double *dparams) {
@@ -583,6 +583,7 @@ __device__ __forceinline__ void reduce_params(const double *p3, int n3, const do
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   const double s = warp_sums8(v);
   if ((l & 3) == 0 && l < 12) sh[w][l >> 2] = s;
+  cluster_running<CS>();
   __syncthreads();
   if (threadIdx.x < 3) {
     double acc = 0.0;
@@ -604,6 +605,7 @@ __global__ void __launch_bounds__(256) k_adj_reduce_seed(AdjArgs a) {
 template <int CS>
 __global__ void __launch_bounds__(256) k_adj_reduce(AdjArgs a) {
   const CavDev &cv = a.cav[blockIdx.x / CS];
+  cluster_arrive<CS>();
   previous_done();
   dependents_may_start();
   reduce_params<CS>(a.phalf + 3 * int64_t(cv.blk0), cv.nblk, a.pfull + cv.adj0, cv.nblk_adj,

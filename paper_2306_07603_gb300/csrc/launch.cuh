@@ -23,9 +23,23 @@ __device__ __forceinline__ void dependents_may_start() {
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
-// Address of p, in this block's shared memory, in that of the first block of the
-// cluster of CS blocks; and the barrier after which the first block reads what
-// the others wrote there.
+// Shared memory of the first block of a cluster of CS blocks. A block's shared
+// memory may be accessed from another one only once that block is known to run
+// (being launched together does not say so), and until it ends. So every thread
+// calls cluster_arrive() at the start of the kernel and cluster_running(), which
+// returns when all of the cluster's threads have done so, before the first use of
+// cluster_at(): the address of p, in this block's shared memory, in that of the
+// first block. The arrival orders no memory; what lies between the two hides it.
+// cluster_done() is the barrier after which the first block reads what the others
+// wrote there. Every thread of the block calls each of them, or none does.
+template <int CS>
+__device__ __forceinline__ void cluster_arrive() {
+  if constexpr (CS > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::);
+}
+template <int CS>
+__device__ __forceinline__ void cluster_running() {
+  if constexpr (CS > 1) asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");
+}
 template <int CS>
 __device__ __forceinline__ double *cluster_at(double *p) {
   if constexpr (CS == 1)

@@ -359,9 +359,11 @@ __global__ void __launch_bounds__(256) k_residual_reduce(ReduceArgs a) {
   const int k = blockIdx.x / CS, r = blockIdx.x % CS;
   const CavDev &cv = a.cav[k];
   const int s0 = int(int64_t(cv.nparts) * r / CS), s1 = int(int64_t(cv.nparts) * (r + 1) / CS);
+  cluster_arrive<CS>();
   previous_done();
   dependents_may_start();
   const Partial p = sum_slots(a.part + int64_t(cv.part0 + s0) * NPART, threadIdx.x, 256, s1 - s0);
+  cluster_running<CS>();
   block_reduce<8>(p, cluster_at<CS>(&all[r][0]));
   cluster_done<CS>();
   if (r == 0 && threadIdx.x == 0) {
@@ -443,6 +445,7 @@ __global__ void __launch_bounds__(32 * MSEG) k_macros(MacrosArgs a) {
   const double *gm = GEN ? a.geo.gmet + 7 * cv.off : nullptr;
   __shared__ double part[MSEG][33];  // (a line's sums are read along it too)
   __shared__ double below[CS][32];   // (first block's: the blocks' totals)
+  if (a.psi) cluster_arrive<CS>();   // (psi: uniform over the launch)
   previous_done();
   dependents_may_start();
   const double p0 = a.pref[a.cavity];
@@ -485,6 +488,7 @@ __global__ void __launch_bounds__(32 * MSEG) k_macros(MacrosArgs a) {
   __syncthreads();
   if (w > 0) acc = part[w - 1][threadIdx.x];
   if constexpr (CS > 1) {
+    cluster_running<CS>();
     if (w == MSEG - 1) cluster_at<CS>(&below[r][0])[threadIdx.x] = part[w][threadIdx.x];
     cluster_done<CS>();
     const double *all = cluster_at<CS>(&below[0][0]);
