@@ -331,7 +331,9 @@ int ifdlbm_probe_dev(ifdlbm_handle h, int n, const int *probes, double *out);
 
 /* Copies of the whole batch state between the handle and caller-owned
  * DEVICE memory of ifdlbm_state_bytes(h) bytes (opaque layout, valid only
- * for the same handle). Used for checkpoints. Do not synchronise. */
+ * for the same handle). Used for checkpoints. The memory may be another
+ * device's: the copy engine then copies it, otherwise a kernel does while the
+ * state is small. Do not synchronise. */
 int64_t ifdlbm_state_bytes(ifdlbm_handle h);
 int ifdlbm_save_state_dev(ifdlbm_handle h, void *dst);
 int ifdlbm_load_state_dev(ifdlbm_handle h, const void *src);

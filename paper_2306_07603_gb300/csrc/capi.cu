@@ -1400,7 +1400,7 @@ int ifdlbm_save_state_dev(ifdlbm_handle h, void *dst) {
   const cudaError_t e = ifd::launch_copy(
       {{h->b.g[h->cur], h->b.lam[h->cur], h->b.pref},
        {dst, (char *)dst + gb, (char *)dst + gb + lb},
-       {int64_t(gb), int64_t(lb), int64_t(h->ncav * sizeof(double))}}, h->stream);
+       {int64_t(gb), int64_t(lb), int64_t(h->ncav * sizeof(double))}}, dst, h->device, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "save_state_dev");
   return IFDLBM_OK;
 }
@@ -1414,7 +1414,7 @@ int ifdlbm_load_state_dev(ifdlbm_handle h, const void *src) {
   const cudaError_t e = ifd::launch_copy(
       {{src, (const char *)src + gb, (const char *)src + gb + lb},
        {h->b.g[h->cur], h->b.lam[h->cur], h->b.pref},
-       {int64_t(gb), int64_t(lb), int64_t(h->ncav * sizeof(double))}}, h->stream);
+       {int64_t(gb), int64_t(lb), int64_t(h->ncav * sizeof(double))}}, src, h->device, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "load_state_dev");
   return IFDLBM_OK;
 }
@@ -1630,7 +1630,7 @@ int ifdlbm_save_intermediates_dev(ifdlbm_handle h, void *dst) {
   const int64_t P9 = 9 * h->total_plane * int64_t(sizeof(double));
   const cudaError_t e = ifd::launch_copy({{h->b.fb, h->b.fp, h->b.fh},
                                           {dst, (char *)dst + P9, (char *)dst + 2 * P9},
-                                          {P9, P9, P9}}, h->stream);
+                                          {P9, P9, P9}}, dst, h->device, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "save_intermediates_dev");
   return IFDLBM_OK;
 }

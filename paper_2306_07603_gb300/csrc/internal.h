@@ -5,6 +5,8 @@
 #include <string>
 #include <cuda_runtime.h>
 
+#include "copy_route.h"
+
 namespace ifd {
 
 // Mixed difference of Eqs. (2.5)-(2.7) along one axis, times 2 d and signed so
@@ -188,16 +190,8 @@ constexpr int REDUCE_ONE = 512, REDUCE_CS = 8;
 void launch_residual_reduce(const CavDev *cav, const double *part, double *resid, int ncav,
                             int most, cudaStream_t s);
 
-// Device-to-device copies of up to three segments: one kernel while they are
-// small (COPY_MOST bytes in all), where the launches of three copies cost more
-// than the bytes.
-struct CopyArgs {
-  const void *src[3];
-  void *dst[3];
-  int64_t bytes[3];
-};
-constexpr int64_t COPY_MOST = int64_t(64) << 20;
-cudaError_t launch_copy(const CopyArgs &a, cudaStream_t s);
+// The copies of `a` on stream s; `mine` is the caller's buffer (copy_by_kernel).
+cudaError_t launch_copy(const CopyArgs &a, const void *mine, int device, cudaStream_t s);
 
 // Discrete adjoint of one staged FP64 step (adjoint.cu). Buffers use the
 // state layout: 9 planes then 1 plane per cavity at the usual offsets.

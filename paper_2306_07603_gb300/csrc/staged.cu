@@ -779,17 +779,13 @@ void launch_residual_reduce(const CavDev *cav, const double *part, double *resid
   else
     launch_after(k_residual_reduce<1>, ncav, 256, 0, s, a);
 }
-cudaError_t launch_copy(const CopyArgs &a, cudaStream_t s) {
-  // segments that are not on 16-byte boundaries, or not whole doubles, are left
-  // to the copy engine; so are large ones, where three launches do not count
-  int64_t total = 0;
-  bool plain = true;
-  for (int k = 0; k < 3; ++k) {
-    total += a.bytes[k];
-    plain &= ((uintptr_t(a.src[k]) | uintptr_t(a.dst[k])) & 15) == 0 && a.bytes[k] % 8 == 0;
-  }
-  if (plain && total <= COPY_MOST) {
-    const int64_t blocks = (total / 16 + 255) / 256;
+cudaError_t launch_copy(const CopyArgs &a, const void *mine, int device, cudaStream_t s) {
+  cudaPointerAttributes at = {};
+  const bool here = cudaPointerGetAttributes(&at, mine) == cudaSuccess &&
+                    at.type == cudaMemoryTypeDevice && at.device == device;
+  (void)cudaGetLastError();  // an address CUDA does not know: the copies below say so
+  if (copy_by_kernel(a, here)) {
+    const int64_t blocks = ((a.bytes[0] + a.bytes[1] + a.bytes[2]) / 16 + 255) / 256;
     launch_after(k_copy, int(std::max<int64_t>(1, std::min<int64_t>(blocks, 152 * 8))), 256, 0, s,
                  a);
     count_launches(1);
