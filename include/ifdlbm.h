@@ -57,10 +57,11 @@ extern "C" {
                             pressure every 1024 steps (a uniform pressure
                             offset is a neutral, drifting mode). The metrics
                             and all reductions are FP64; the power law of Eq.
-                            (1.4), on the FP32 strain rate, is FP64 or, in the
-                            fused kernel, pairs of floats (2^-40 before its one
-                            rounding; see power_fp32 for a plain FP32 power);
-                            the relaxation-time plane is stored in FP32. Every
+                            (1.4), on the FP32 strain rate, is FP64, rounded
+                            once to the FP32 relaxation-time plane (the fused
+                            kernel finds the same float in pairs of floats and
+                            evaluates FP64 only where those leave it in doubt;
+                            see power_fp32 for a plain FP32 power). Every
                             output includes P_ref. */
 
 /* Step kernel organisation. */
@@ -498,10 +499,10 @@ int ifdlbm_inject_tma_timeout(ifdlbm_handle h, int enable);
 int ifdlbm_selftest_pow_tab(ifdlbm_handle h, int cavity, int n, const double *x, double *out);
 
 /* Self-test of the same power as the fused kernel evaluates it, in pairs of
- * floats, rounded once to the FP32 relaxation-time plane: for n DEVICE doubles
- * x[k] whose float roundings are normal and > 0, writes out[k] = that value and
- * out[n + k] = the FP64 one of ifdlbm_selftest_pow_tab rounded to FP32, both
- * widened to double. `out` is a DEVICE array of 2n doubles; on the handle's
+ * floats where these settle its rounding to the FP32 relaxation-time plane: for n
+ * DEVICE doubles x[k] whose float roundings are normal and > 0, writes out[k] =
+ * that value and out[n + k] = the FP64 one of ifdlbm_selftest_pow_tab rounded to
+ * FP32, both widened to double: the two are equal. `out` is a DEVICE array of 2n doubles; on the handle's
  * stream (no sync). Errors: INVALID_ARG for a bad handle, cavity or pointers, or
  * an FP64 handle. */
 int ifdlbm_selftest_pow_pair(ifdlbm_handle h, int cavity, int n, const double *x, double *out);

@@ -426,7 +426,7 @@ def ifdlbm_selftest_pow_tab(h, cavity, x, out):
 
 def ifdlbm_selftest_pow_pair(h, cavity, x, out):
     """out[:n] = the fused kernel's FP32 C xf^m for cavity `cavity`, out[n:] = pow_tab's rounded
-    to FP32 (x: float64 CUDA tensor of n arguments, out: float64 CUDA tensor of 2n)."""
+    to FP32, equal to it (x: float64 CUDA tensor of n arguments, out: float64 CUDA tensor of 2n)."""
     n = int(x.numel())
     _device_f64("x", x, n)
     _device_f64("out", out, 2 * n)

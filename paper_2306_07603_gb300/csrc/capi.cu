@@ -526,7 +526,8 @@ void ifd::fill_cavity_pow_table(double *tab, double m, double C) {
 }
 // Table of pow_pair from pow_tab's: each double split into a pair of floats, and
 // the range of exponents whose factor lies in [2^-60, 2^60] (a contiguous one:
-// the factor is monotonic in the exponent; 0 and 255 are no normal floats).
+// the factor is monotonic in the exponent; 0 and 255 are no normal floats), empty
+// for an exponent m beyond the one its error is bounded for.
 void ifd::fill_cavity_pair_table(float *tab, const double *powt, CavDev &cv) {
   auto split = [](double v, float *hi) {
     hi[0] = float(v);
@@ -540,7 +541,7 @@ void ifd::fill_cavity_pair_table(float *tab, const double *powt, CavDev &cv) {
   for (int e = 0; e < 256; ++e) {
     const double A = powt[512 + e];
     split(A, tab + 1024 + 2 * e);
-    if (e >= 1 && e <= 254 && A >= 0x1p-60 && A <= 0x1p60) {
+    if (std::fabs(cv.half_nm1) <= 1.0 && e >= 1 && e <= 254 && A >= 0x1p-60 && A <= 0x1p60) {
       lo = std::min(lo, e);
       hi = e;
     }

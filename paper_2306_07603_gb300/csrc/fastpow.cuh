@@ -116,14 +116,19 @@ __device__ __forceinline__ double pow_tab(float x, const double *__restrict__ ta
 //   w = b1 + t (b2 + t (b3 + t b4)),
 //
 // table entries, 1/c_j and b1 as pairs, t, P, w and t w as pairs, the
-// polynomial's tail (below 2^-9 of w) in one float: every term is held to 2^-40
-// of the result or better (the first one dropped is t^5 b5 < 2^-45), then rounded
-// once. The float it gives differs from pow_tab's rounded one where the exact
-// value lies within 2^-40 of a rounding boundary (about one argument in 2^16)
-// and nowhere else; its error is 0.5 ulp as pow_tab's.
+// polynomial's tail (below 2^-9 of w) in one float. For |m| <= 1 (n <= 3) the pair
+// is within 2^-40 of the value: 2^-41 from the tail's roundings (7 half ulps of
+// t b2, |b2| <= 3/8, times t <= 2^-9), the rest from terms of 2^-44 and less. It is
+// used only where every value within 2^-38 of it rounds to the same float (A. Ziv,
+// "Fast evaluation of elementary mathematical functions with correctly rounded
+// last bit", ACM TOMS 17, 1991): that float is the one pow_tab's FP64 value rounds
+// to, and where it is in doubt (one argument in 2^13) pow_tab decides. So the
+// plane holds the rounded FP64 power law, bit for bit, at the cost of 5
+// instructions for the test.
 // Table (POWP_SIZE floats): [4j ..] = c_j^m hi, lo, 1/c_j hi, lo; [1024 + 2e ..] =
 // C 2^(m (e - 127)) hi, lo. Entries e outside [pe_lo, pe_lo + pe_n) are not in
-// [2^-60, 2^60] (their low parts or products could underflow): pow_tab.
+// [2^-60, 2^60] (their low parts or products could underflow), and for |m| > 1 none
+// is inside: pow_tab.
 constexpr int POWP_SIZE = 1536;
 
 struct PowPair {
@@ -151,10 +156,11 @@ __device__ __forceinline__ void pow_pair_parts(float x, const PowPair &c, float 
   hi = Ph + yh;
   lo = (yh - (hi - Ph)) + yl;
 }
-__device__ __forceinline__ float pow_pair(float x, const PowPair &c) {
+__device__ __forceinline__ bool pow_pair(float x, const PowPair &c, float &r) {
   float hi, lo;
   pow_pair_parts(x, c, hi, lo);
-  return hi + lo;
+  r = hi + fmaf(hi, -0x1p-38f, lo);
+  return r == hi + fmaf(hi, 0x1p-38f, lo);
 }
 
 // x^m in FP32 for the FP32-deviation form: 2^(m log2 x) with CUDA's log2f

@@ -37,9 +37,9 @@
 // (write_ghosts), written by the node that reads them, instead of per-plane
 // selects on the wall flags.
 //
-// In FP32 the power of Eq. (1.4) is evaluated in pairs of floats (pow_pair), so that
-// only the residual's sums are left on the FP64 pipe: GB300 issues FP64 at 1/64 of
-// the FP32 rate. With the pow32 opt-in the power is plain FP32 (pow_f32).
+// In FP32 the rounded FP64 power of Eq. (1.4) is found in pairs of floats (pow_pair),
+// so that little but the residual's sums is left on the FP64 pipe: GB300 issues FP64
+// at 1/64 of the FP32 rate. With the pow32 opt-in the power is plain FP32 (pow_f32).
 #pragma once
 #include <cstdint>
 
@@ -469,17 +469,15 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
         o.lam = solve(G2, lam_prev);
       return o;
     }
-    // Eqs. (2.12)-(2.14), (1.4): strain rate in T, power in FP64, by pairs of
-    // floats rounded once to the FP32 plane, or in FP32 with the pow32 opt-in
+    // Eqs. (2.12)-(2.14), (1.4): strain rate in T, power in FP64 (for the FP32
+    // plane the float it rounds to, by pow_pair), or in FP32 with the pow32 opt-in
     const T k = quot<FASTQ>(T(-2), (T(2) * lam_prev + dt) * cs2);
     const T Sxx = k * pxx, Sxy = k * pxy, Syy = k * pyy;
     if constexpr (sizeof(T) == 4) {
       const float qf = fmaxf(T(0.5) * (Sxx * Sxx + T(2) * Sxy * Sxy + Syy * Syy), gmin2_f);
       if constexpr (P32)
         o.lam = Kics2_f * pow_f32(qf, half_nm1_f);
-      else if (pow_pair_covers(qf, pw))
-        o.lam = pow_pair(qf, pw);
-      else
+      else if (!(pow_pair_covers(qf, pw) && pow_pair(qf, pw, o.lam)))
         o.lam = float(pow_tab(qf, powt, half_nm1, cv.pb2, cv.pb3, cv.pb4, cv.pb5));
     } else {
       o.lam = power_law64(T(0.5) * (Sxx * Sxx + T(2) * Sxy * Sxy + Syy * Syy), cv, a.powtab, powt);

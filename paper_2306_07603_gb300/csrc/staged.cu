@@ -681,8 +681,9 @@ void launch_pow_tab_selftest(int n, const double *x, double m, double C, const d
 }
 
 // The FP32 form's power of Eq. (1.4) as the fused kernel evaluates it (pow_pair
-// where its table covers the argument, else pow_tab): out[k] of the FP32
-// rounding of x[k], and out[n + k] = pow_tab's value rounded to FP32.
+// where its table covers the argument and the float is not in doubt, else
+// pow_tab): out[k] of the FP32 rounding of x[k], and out[n + k] = pow_tab's value
+// rounded to FP32.
 __global__ void k_pow_pair_selftest(int n, const double *x, const CavDev *cavs, int cavity,
                                     const double *powt, const float *powp, double *out) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -691,7 +692,8 @@ __global__ void k_pow_pair_selftest(int n, const double *x, const CavDev *cavs, 
   const PowPair pw = {powp, cv.pb1h, cv.pb1l, cv.pb2f, cv.pb3, cv.pb4, cv.pe_lo, cv.pe_n};
   const float xf = float(x[k]);
   const float t = float(pow_tab(xf, powt, cv.half_nm1, cv.pb2, cv.pb3, cv.pb4, cv.pb5));
-  out[k] = double(pow_pair_covers(xf, pw) ? pow_pair(xf, pw) : t);
+  float r;
+  out[k] = double(pow_pair_covers(xf, pw) && pow_pair(xf, pw, r) ? r : t);
   out[n + k] = double(t);
 }
 void launch_pow_pair_selftest(int n, const double *x, const CavDev *cav, int cavity,
