@@ -507,6 +507,16 @@ int ifdlbm_selftest_pow_tab(ifdlbm_handle h, int cavity, int n, const double *x,
  * an FP64 handle. */
 int ifdlbm_selftest_pow_pair(ifdlbm_handle h, int cavity, int n, const double *x, double *out);
 
+/* Self-test of the implicit relaxation time (IFDLBM_LAMBDA_IMPLICIT) as the fused
+ * kernel forms it: for n DEVICE doubles x[k] = (Pxx^2 + 2 Pxy^2 + Pyy^2) / 2 of
+ * the second moments of f-hat - f^eq in units of c (rounded to float, > 0) and
+ * x[n + k] = the lagged relaxation time (rounded to float, > 0), writes out[k] =
+ * that root and out[n + k] = the FP64 solve's rounded to FP32, both widened to
+ * double. `x` and `out` are DEVICE arrays of 2n doubles; on the handle's stream (no
+ * sync). Errors: INVALID_ARG for a bad handle, cavity or pointers, or an FP64
+ * handle. */
+int ifdlbm_selftest_implicit(ifdlbm_handle h, int cavity, int n, const double *x, double *out);
+
 /* Self-test of the FP32 power the FP32-power opt-in uses for Eq. (1.4):
  * for n DEVICE doubles x[k] (finite, > 0 after rounding to float) writes
  * out[k] = float(x[k])^float(m) as the library evaluates it, widened to

@@ -131,6 +131,7 @@ _SIGS = {
     "ifdlbm_selftest_pow_f32": (C.c_int, [_H, C.c_int, _P, C.c_double, _P]),
     "ifdlbm_selftest_pow_tab": (C.c_int, [_H, C.c_int, C.c_int, _P, _P]),
     "ifdlbm_selftest_pow_pair": (C.c_int, [_H, C.c_int, C.c_int, _P, _P]),
+    "ifdlbm_selftest_implicit": (C.c_int, [_H, C.c_int, C.c_int, _P, _P]),
     "ifdlbm_inject_tma_timeout": (C.c_int, [_H, C.c_int]),
     "ifdlbm_adjoint_seed_energy": (C.c_int, [_H, _P, _P, _P]),
     "ifdlbm_autotune": (C.c_int, [_H, C.c_int, C.c_void_p]),
@@ -431,6 +432,15 @@ def ifdlbm_selftest_pow_pair(h, cavity, x, out):
     _device_f64("x", x, n)
     _device_f64("out", out, 2 * n)
     return _check(load_library().ifdlbm_selftest_pow_pair(h, int(cavity), n, _ptr(x), _ptr(out)), h)
+
+
+def ifdlbm_selftest_implicit(h, cavity, x, out):
+    """out[:n] = the fused kernel's implicit root for cavity `cavity` at G2 = x[:n] from the
+    lagged value x[n:], out[n:] = the FP64 solve's (x, out: float64 CUDA tensors of 2n)."""
+    n = int(x.numel()) // 2
+    _device_f64("x", x, 2 * n)
+    _device_f64("out", out, 2 * n)
+    return _check(load_library().ifdlbm_selftest_implicit(h, int(cavity), n, _ptr(x), _ptr(out)), h)
 
 
 def ifdlbm_inject_tma_timeout(h, enable=True):

@@ -1772,6 +1772,20 @@ int ifdlbm_selftest_pow_pair(ifdlbm_handle h, int cavity, int n, const double *x
   return IFDLBM_OK;
 }
 
+int ifdlbm_selftest_implicit(ifdlbm_handle h, int cavity, int n, const double *x, double *out) {
+  if (!cavity_ok(h, cavity) || n < 0 || (n > 0 && (!x || !out)) || !h->b.powp)
+    return fail(h, IFDLBM_ERR_INVALID_ARG, "selftest_implicit: bad arguments or not an FP32 handle");
+  if (n == 0) return IFDLBM_OK;
+  cudaSetDevice(h->device);
+  ifd::launch_implicit_selftest(n, x, h->b.cav, cavity, h->b.powtab,
+                                h->b.powt + size_t(cavity) * ifd::POWT_SIZE,
+                                h->b.powp + size_t(cavity) * ifd::POWP_SIZE, out, h->stream);
+  g_launches += 1;
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(h, e, "selftest_implicit");
+  return IFDLBM_OK;
+}
+
 int ifdlbm_selftest_pow_f32(ifdlbm_handle h, int n, const double *x, double m, double *out) {
   if (!h || n < 0 || (n > 0 && (!x || !out)))
     return fail(h, IFDLBM_ERR_INVALID_ARG, "selftest_pow_f32: bad arguments");

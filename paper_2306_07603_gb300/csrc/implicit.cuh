@@ -98,10 +98,16 @@ __device__ __forceinline__ ImplPair impl_pair(const CavDev &cv) {
 }
 
 // The FP64 root rounded to float: lambda_approx, then one Newton step with
-// x = 2 lam + dt, 1 / x, q = 36 G2 / x^2 and P = C q^m as pairs of floats (pow_pair:
-// 2^-40), so that F = lam - P, whose leading difference is exact, has an error of
-// 2^-40 lam, and the step leaves the square of the approximation's. Rounded once.
-// Where the table does not cover q or the step is large, the FP64 solve.
+// x = 2 lam + dt, 1 / x, q = 36 G2 / x^2 and P = C q^m as pairs of floats, whose errors
+// are 2^-43, 2^-42 and (pow_pair) 2^-39.8: F = lam - P, whose leading difference is
+// exact, is known to 2^-38 lam. With D = F' = 1 + 2 m P / x, d = F / D the step and
+// F'' = -4 m (m + 1) P / x^2, |F''| <= |m (m + 1)| / lam to 2e-4, the error of lam - d is
+//   E = (2^-38 lam + |m (m + 1)| d^2 / (2 lam) + 2^-19 max(1, |m|) |d|) / D,
+// the last term for the roundings of D, of the quotients and of d. The float is taken
+// only where lam - d - E and lam - d + E round to it (pow_pair's rounding test; E is a
+// few 1e-12 lam, so that one root in 10^4 is in doubt); else, and where the table does
+// not cover q, the step is large, D is near zero (n < 0.02) or a low part could
+// underflow, the FP64 solve decides.
 __device__ __forceinline__ float lambda_implicit_pair(float G2, float lam_start, const ImplPair &s,
                                                       const PowPair &pw, const CavDev &cv,
                                                       const double *powtab, const double *powt) {
@@ -114,12 +120,16 @@ __device__ __forceinline__ float lambda_implicit_pair(float G2, float lam_start,
     const float sh = rh * rh, sl = fmaf(rh, rh, -sh) + 2.0f * rh * rl;
     const float Ah = 36.0f * G2, Al = fmaf(36.0f, G2, -Ah);
     const float qh = Ah * sh, ql = fmaf(Ah, sh, -qh) + (Ah * sl + Al * sh);
-    if (pow_pair_covers(qh, pw)) {
+    if (pow_pair_covers(qh, pw) && fminf(fminf(Ah, sh), qh) >= 0x1p-80f) {
       float Ph, Pl;
       pow_pair_parts(qh, pw, Ph, Pl);
       Pl = fmaf(Ph, s.hm * __fdividef(ql, qh), Pl);    // (q_h + q_l)^m
-      const float d = __fdividef((lam - Ph) - Pl, fmaf(2.0f * s.m * Ph, rh, 1.0f));
-      if (fabsf(d) <= 1e-4f * lam) return lam - d;
+      const float D = fmaf(2.0f * s.m * Ph, rh, 1.0f), d = __fdividef((lam - Ph) - Pl, D);
+      const float ad = fabsf(d), k = 0.55f * fabsf(s.m * (s.m + 1.0f));
+      const float E = __fdividef(
+          fmaf(lam, 0x1p-38f, ad * fmaf(k, __fdividef(ad, lam), 0x1p-19f * fmaxf(1.0f, fabsf(s.m)))), D);
+      const float r = lam - (d + E);
+      if (ad <= 1e-4f * lam && D >= 0x1p-6f && r == lam - (d - E)) return r;
     }
   }
   return float(lambda_implicit(6.0 * sqrt(double(G2)), double(lam_start), cv, powtab, powt));

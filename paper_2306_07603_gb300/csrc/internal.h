@@ -229,6 +229,9 @@ void launch_pow_tab_selftest(int n, const double *x, double m, double C, const d
                              double b2, float b3, float b4, float b5, double *out, cudaStream_t s);
 void launch_pow_pair_selftest(int n, const double *x, const CavDev *cav, int cavity,
                               const double *powt, const float *powp, double *out, cudaStream_t s);
+void launch_implicit_selftest(int n, const double *x, const CavDev *cav, int cavity,
+                              const double *powtab, const double *powt, const float *powp,
+                              double *out, cudaStream_t s);
 void launch_pow_f32_selftest(int n, const double *x, double m, double *out, cudaStream_t s);
 
 // Metrics of the bilinear map of a general quadrilateral at (xi, eta),

@@ -701,6 +701,27 @@ void launch_pow_pair_selftest(int n, const double *x, const CavDev *cav, int cav
   k_pow_pair_selftest<<<(n + 255) / 256, 256, 0, s>>>(n, x, cav, cavity, powt, powp, out);
 }
 
+// The implicit form's root as the fused kernel forms it (lambda_implicit_pair):
+// out[k] at G2 = x[k] (a float, in units of c) from the lagged value x[n + k], and
+// out[n + k] = the FP64 solve rounded to FP32.
+__global__ void k_implicit_selftest(int n, const double *x, const CavDev *cavs, int cavity,
+                                    const double *powtab, const double *powt, const float *powp,
+                                    double *out) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= n) return;
+  const CavDev &cv = cavs[cavity];
+  const PowPair pw = {powp, cv.pb1h, cv.pb1l, cv.pb2f, cv.pb3, cv.pb4, cv.pe_lo, cv.pe_n};
+  const float G2 = float(x[k]), start = float(x[n + k]);
+  out[k] = double(lambda_implicit_pair(G2, start, impl_pair(cv), pw, cv, powtab, powt));
+  out[n + k] =
+      double(float(lambda_implicit(6.0 * sqrt(double(G2)), double(start), cv, powtab, powt)));
+}
+void launch_implicit_selftest(int n, const double *x, const CavDev *cav, int cavity,
+                              const double *powtab, const double *powt, const float *powp,
+                              double *out, cudaStream_t s) {
+  k_implicit_selftest<<<(n + 255) / 256, 256, 0, s>>>(n, x, cav, cavity, powtab, powt, powp, out);
+}
+
 __global__ void k_pow_f32_selftest(int n, const double *x, double m, double *out) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
