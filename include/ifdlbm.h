@@ -517,6 +517,12 @@ int ifdlbm_selftest_pow_pair(ifdlbm_handle h, int cavity, int n, const double *x
  * handle. */
 int ifdlbm_selftest_implicit(ifdlbm_handle h, int cavity, int n, const double *x, double *out);
 
+/* Self-test of the power law of the FP64 staged kernels: for n DEVICE doubles
+ * x[k] > 0 writes the DEVICE doubles out[k] = K/c_s^2 x[k]^((n-1)/2) of cavity
+ * `cavity`; on the handle's stream (no sync). Errors: INVALID_ARG for a bad handle,
+ * cavity or pointers. */
+int ifdlbm_selftest_power64(ifdlbm_handle h, int cavity, int n, const double *x, double *out);
+
 /* Self-test of the FP32 power the FP32-power opt-in uses for Eq. (1.4):
  * for n DEVICE doubles x[k] (finite, > 0 after rounding to float) writes
  * out[k] = float(x[k])^float(m) as the library evaluates it, widened to

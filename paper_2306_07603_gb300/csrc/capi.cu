@@ -818,6 +818,7 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
     cv.inv_Re = 1.0 / s.Re;
     cv.half_nm1 = 0.5 * cv.nm1;
     cv.Kics2 = cv.K / cv.cs2;
+    cv.p64_n = std::fabs(cv.half_nm1) <= 1.0 ? 254u << 20 : 0u;
     {  // pow_tab: binomial coefficients of (1 + t)^m, m = (n - 1)/2, and the FP32 clamp
       const double m = cv.half_nm1;
       cv.pb2 = m * (m - 1.0) / 2.0;
@@ -1769,6 +1770,19 @@ int ifdlbm_selftest_pow_pair(ifdlbm_handle h, int cavity, int n, const double *x
   g_launches += 1;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e, "selftest_pow_pair");
+  return IFDLBM_OK;
+}
+
+int ifdlbm_selftest_power64(ifdlbm_handle h, int cavity, int n, const double *x, double *out) {
+  if (!cavity_ok(h, cavity) || n < 0 || (n > 0 && (!x || !out)))
+    return fail(h, IFDLBM_ERR_INVALID_ARG, "selftest_power64: bad arguments");
+  if (n == 0) return IFDLBM_OK;
+  cudaSetDevice(h->device);
+  ifd::launch_power64_selftest(n, x, h->b.cav, cavity, h->b.powtab,
+                               h->b.powt + size_t(cavity) * ifd::POWT_SIZE, out, h->stream);
+  g_launches += 1;
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(h, e, "selftest_power64");
   return IFDLBM_OK;
 }
 

@@ -55,6 +55,7 @@ struct CavDev {
   float g2c_f;              // ... the largest float G2 whose root is the clamp value (ImplPair)
   float pb1h, pb1l, pb2f;   // pow_pair: b1 = m as a pair of floats, b2 rounded
   unsigned pe_lo, pe_n;     // ... and the exponents its table covers
+  unsigned p64_n;           // power64: range of the table's high words, 0 where it is not used
   // FP64 staged kernels (staged64.cu): thread blocks of this cavity and, for the
   // half step [0] and the full step [1] (scale dt/2 and dt), the coefficients
   // of the mixed difference (xi, unscaled; eta of the trapezoid, times -scale
@@ -232,6 +233,8 @@ void launch_pow_pair_selftest(int n, const double *x, const CavDev *cav, int cav
 void launch_implicit_selftest(int n, const double *x, const CavDev *cav, int cavity,
                               const double *powtab, const double *powt, const float *powp,
                               double *out, cudaStream_t s);
+void launch_power64_selftest(int n, const double *x, const CavDev *cav, int cavity,
+                             const double *powtab, const double *powt, double *out, cudaStream_t s);
 void launch_pow_f32_selftest(int n, const double *x, double m, double *out, cudaStream_t s);
 
 // Metrics of the bilinear map of a general quadrilateral at (xi, eta),

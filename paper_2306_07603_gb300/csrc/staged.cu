@@ -722,6 +722,17 @@ void launch_implicit_selftest(int n, const double *x, const CavDev *cav, int cav
   k_implicit_selftest<<<(n + 255) / 256, 256, 0, s>>>(n, x, cav, cavity, powtab, powt, powp, out);
 }
 
+__global__ void k_power64_selftest(int n, const double *x, const CavDev *cavs, int cavity,
+                                   const double *powtab, const double *powt, double *out) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < n) out[k] = power64(x[k], cavs[cavity], powtab, powt);
+}
+void launch_power64_selftest(int n, const double *x, const CavDev *cav, int cavity,
+                             const double *powtab, const double *powt, double *out,
+                             cudaStream_t s) {
+  k_power64_selftest<<<(n + 255) / 256, 256, 0, s>>>(n, x, cav, cavity, powtab, powt, out);
+}
+
 __global__ void k_pow_f32_selftest(int n, const double *x, double m, double *out) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;

@@ -95,14 +95,17 @@ __device__ __forceinline__ bool nonnegative(double x) { return !negative(x) || z
 // K/c_s^2 q^m, m = (n-1)/2, for an FP64 argument q > 0: the table-driven binomial
 // form of pow_tab (fastpow.cuh) on the full FP64 fraction f of q = 2^e f. As
 // there, t = f (1/c_j) - 1 carries the rounding of 1/c_j (<= 1.2e-16 absolute) and
-// one of its own below 2^-62, the tail's coefficient is FP32, and the result is
-// within 6e-16: closer than pow_fast's 5e-16 + 2.2e-16 |m log2 q|, with 6 FP64
-// instructions instead of ~22. The table covers the exponents of a normal
-// float; an argument beyond them (or a NaN) takes pow_fast.
+// one of its own below 2^-62, and the tail's coefficient c3 is FP32: with the four
+// roundings of the tables and products the result is within 4.5e-16 + |m| 1.2e-16 +
+// |b3| 6.7e-16 + |C(m,6)| 5.6e-17, b3 = m (m-1) (m-2) / 6: 7.2e-16 for |m| <= 1
+// (n <= 3), against pow_fast's 5e-16 + 2.2e-16 |m log2 q|, with 6 FP64 instructions
+// instead of ~22. Beyond, b3 grows as m^3 (5e-14 at n = 20): pow_fast, as for an
+// argument whose exponent is not a normal float's, which the table does not cover,
+// and for a NaN.
 __device__ __forceinline__ double power64(double q, const CavDev &cv, const double *powtab,
                                           const double *__restrict__ powt) {
   const int hi = __double2hiint(q), lo = __double2loint(q);
-  if (unsigned(hi - (897 << 20)) >= unsigned(254 << 20))
+  if (unsigned(hi - (897 << 20)) >= cv.p64_n)
     return cv.Kics2 * pow_fast(q, cv.half_nm1, powtab);
   const unsigned e = (unsigned(hi) >> 20) - 896u, j = (unsigned(hi) >> 12) & 255u;
   const int fh = (hi & 0x000FFFFF) | 0x3FF00000;
