@@ -292,8 +292,8 @@ __device__ __forceinline__ double theta_partial(const CavDev &cv, const Geo &geo
   // k: dc/dtheta of the pair's first member; pos0, pos1: c >= 0 of either (both at c = 0)
   auto term = [&](int q0, bool pos0, bool pos1, double k, double r) {
     const double *F0 = F + q0 * plane, *F1 = F0 + 2 * plane;
-    const double a = mix64(F0, pos0 ? 1 : -1, pos0 ? clo : chi, mix, F0[0], 0.0, true);
-    const double b = mix64(F1, pos1 ? 1 : -1, pos1 ? clo : chi, mix, F1[0], 0.0, true);
+    const double a = mix64(F0, pos0 ? 1 : -1, pos0 ? clo : chi, mix, F0[0]);
+    const double b = mix64(F1, pos1 ? 1 : -1, pos1 ? clo : chi, mix, F1[0]);
     const double g0 = Gb[q0 * plane], g1 = Gb[(q0 + 2) * plane];
     return fma(fma(pos0 ? g0 : -g0, a, (pos1 ? -g1 : g1) * b), k, r);
   };

@@ -799,7 +799,8 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
         const double scale = st == 0 ? 0.5 * cv.dt : cv.dt;
         cv.sxi[st] = scale * opt.c * cv.inv2dxi;
         cv.seta[st] = scale * opt.c * cv.inv2deta;
-        const double E = -cv.seta[st] / H;
+        cv.seta_H[st] = cv.seta[st] / H;
+        const double E = -cv.seta_H[st];
         cv.mixe[st] = ifd::Mix64{E * cv.mix.ka, E * cv.mix.kb, E * cv.mix.k0,
                                  E * cv.mix.kf, E * cv.mix.wb, E * cv.mix.w0};
       }

@@ -58,12 +58,13 @@ struct CavDev {
   unsigned p64_n;           // power64: range of the table's high words, 0 where it is not used
   // FP64 staged kernels (staged64.cu): thread blocks of this cavity and, for the
   // half step [0] and the full step [1] (scale dt/2 and dt), the coefficients
-  // of the mixed difference (xi, unscaled; eta of the trapezoid, times -scale
-  // c / (2 deta H)) and scale c / (2 dxi), scale c / (2 deta)
+  // of the mixed difference (mix; mixe, the adjoint's along eta on the trapezoid:
+  // times -scale c / (2 deta H)) and scale c / (2 dxi), scale c / (2 deta) and the
+  // latter over H
   int blk0, nblk_in, nblk;
   int adj0, nblk_core, nblk_adj, ring0;  // adjoint: blocks over the interior, over its ring
   Mix64 mix, mixe[2];
-  double sxi[2], seta[2];
+  double sxi[2], seta[2], seta_H[2];
   double strain2;           // 2 c^4 / c_s^4: |gamma-dot|^2 = strain2 pp / (2 lam_prev + dt)^2
 };
 

@@ -191,7 +191,7 @@ __host__ __device__ constexpr bool second_of(int q) { return q == 3 || q == 4 ||
 // Contravariant velocities of a node, per pair of opposite directions: the
 // magnitude times scale / (2 d) (scale = dt/2 or dt), and whether the pair's
 // first member is advected from below (c >= 0). On the trapezoid the eta
-// velocity is uniform and its factor is in the coefficients Mix64.
+// velocity is uniform.
 template <bool GEN>
 struct Speeds64 {
   double xi[4], eta[GEN ? 4 : 1];
@@ -220,20 +220,20 @@ __device__ __forceinline__ Speeds64<GEN> speeds64(const CavDev &cv, const Geo &g
     const double m = 1.0 - xe, p = 1.0 + xe;
     s.xi[0] = A, s.xi[1] = A * fabs(xe), s.xi[2] = A * fabs(m), s.xi[3] = A * fabs(p);
     s.xpos[0] = true, s.xpos[1] = negative(xe), s.xpos[2] = !negative(m), s.xpos[3] = negative(p);
-    s.eta[0] = 0.0;
+    s.eta[0] = cv.seta_H[stage];
     s.epos[0] = s.epos[1] = s.epos[2] = s.epos[3] = true;  // e_y of the first members >= 0
   }
   return s;
 }
 
-// sum of the mixed difference's terms (Mix64) at F with stride d (signed: the
-// upwind neighbour is F[-d]), added to acc.
-__device__ __forceinline__ double mix64(const double *F, int d, bool edge, const Mix64 &m, double f0,
-                                        double acc, bool first) {
+// The mixed difference's terms (Mix64) at F with stride d (signed: the upwind
+// neighbour is F[-d]), summed before any speed multiplies them: with the default
+// blend, whose coefficients are short, a constant F gives exactly 0.
+__device__ __forceinline__ double mix64(const double *F, int d, bool edge, const Mix64 &m,
+                                        double f0) {
   const double a = F[d], b = F[-d], f = F[edge ? -d : -2 * d];
   const double kb = edge ? m.wb : m.kb, k0 = edge ? m.w0 : m.k0, kf = edge ? 0.0 : m.kf;
-  acc = first ? m.ka * a : fma(m.ka, a, acc);
-  return fma(kf, f, fma(k0, f0, fma(kb, b, acc)));
+  return fma(kf, f, fma(k0, f0, fma(kb, b, m.ka * a)));
 }
 
 // What the stencils of a node take besides the planes: its speeds, the
@@ -242,7 +242,7 @@ __device__ __forceinline__ double mix64(const double *F, int d, bool edge, const
 template <bool GEN>
 struct Stencil64 {
   Speeds64<GEN> s;
-  Mix64 mix, mixe;
+  Mix64 mix;
   int pitch;
   bool clo, chi, lo, hi;
 };
@@ -253,7 +253,6 @@ __device__ __forceinline__ Stencil64<GEN> stencil64(const CavDev &cv, const Geo 
   st.pitch = cv.pitch;
   st.s = speeds64<GEN>(cv, geo, stage, i, j, int64_t(j) * st.pitch + i);
   st.mix = cv.mix;
-  if constexpr (!GEN) st.mixe = cv.mixe[stage];
   st.clo = i == 1;
   st.chi = i == cv.nx - 2;
   st.lo = j == 1;
@@ -262,21 +261,26 @@ __device__ __forceinline__ Stencil64<GEN> stencil64(const CavDev &cv, const Geo 
 }
 
 // base - scale (c_xi D_xi + c_eta D_eta) F_q at interior node F (Eqs. 3.6-3.7):
-// 9 FP64 instructions a plane (5 where e_y = 0 on the trapezoid).
+// 10 FP64 instructions a plane (5 where e_y = 0 on the trapezoid). The eta speed of
+// the trapezoid could be in the coefficients, for 9; but four roundings at the size
+// of F then take the place of one, and a constant F leaves them behind (error of g
+// against extended precision, 1025^2, 2 steps: 1.42e-16 of its rms against 1.24e-16
+// so and 1.28e-16 with the differences formed first, for 14 instructions).
 template <int Q, bool GEN>
 __device__ __forceinline__ double advect64(double base, const double *F, double f0,
                                            const Stencil64<GEN> &st) {
   constexpr int p = pair_of(Q);
   const bool xpos = st.s.xpos[p] != second_of(Q);
   double out = fma(-st.s.xi[p],
-                   mix64(F, xpos ? 1 : -1, xpos ? st.clo : st.chi, st.mix, f0, 0.0, true), base);
+                   mix64(F, xpos ? 1 : -1, xpos ? st.clo : st.chi, st.mix, f0), base);
   if constexpr (GEN) {
     const bool epos = st.s.epos[p] != second_of(Q);
-    out = fma(-st.s.eta[p], mix64(F, epos ? st.pitch : -st.pitch, epos ? st.lo : st.hi, st.mix, f0,
-                                  0.0, true), out);
+    out = fma(-st.s.eta[p],
+              mix64(F, epos ? st.pitch : -st.pitch, epos ? st.lo : st.hi, st.mix, f0), out);
   } else if constexpr (Q != 1 && Q != 3) {
     constexpr bool epos = Q == 2 || Q == 5 || Q == 6;
-    out = mix64(F, epos ? st.pitch : -st.pitch, epos ? st.lo : st.hi, st.mixe, f0, out, false);
+    out = fma(-st.s.eta[0],
+              mix64(F, epos ? st.pitch : -st.pitch, epos ? st.lo : st.hi, st.mix, f0), out);
   }
   return out;
 }
