@@ -517,6 +517,11 @@ int ifdlbm_selftest_pow_pair(ifdlbm_handle h, int cavity, int n, const double *x
  * handle. */
 int ifdlbm_selftest_implicit(ifdlbm_handle h, int cavity, int n, const double *x, double *out);
 
+/* Self-test of the reciprocal of the FP64 kernels: for n DEVICE doubles x[k] writes
+ * the DEVICE doubles out[k] = 1 / x[k]; on the handle's stream (no sync). Errors:
+ * INVALID_ARG for a bad handle or pointers. */
+int ifdlbm_selftest_recip(ifdlbm_handle h, int n, const double *x, double *out);
+
 /* Self-test of the power law of the FP64 staged kernels: for n DEVICE doubles
  * x[k] > 0 writes the DEVICE doubles out[k] = K/c_s^2 x[k]^((n-1)/2) of cavity
  * `cavity`; on the handle's stream (no sync). Errors: INVALID_ARG for a bad handle,

@@ -132,6 +132,7 @@ _SIGS = {
     "ifdlbm_selftest_pow_tab": (C.c_int, [_H, C.c_int, C.c_int, _P, _P]),
     "ifdlbm_selftest_pow_pair": (C.c_int, [_H, C.c_int, C.c_int, _P, _P]),
     "ifdlbm_selftest_implicit": (C.c_int, [_H, C.c_int, C.c_int, _P, _P]),
+    "ifdlbm_selftest_recip": (C.c_int, [_H, C.c_int, _P, _P]),
     "ifdlbm_selftest_power64": (C.c_int, [_H, C.c_int, C.c_int, _P, _P]),
     "ifdlbm_inject_tma_timeout": (C.c_int, [_H, C.c_int]),
     "ifdlbm_adjoint_seed_energy": (C.c_int, [_H, _P, _P, _P]),
@@ -433,6 +434,14 @@ def ifdlbm_selftest_pow_pair(h, cavity, x, out):
     _device_f64("x", x, n)
     _device_f64("out", out, 2 * n)
     return _check(load_library().ifdlbm_selftest_pow_pair(h, int(cavity), n, _ptr(x), _ptr(out)), h)
+
+
+def ifdlbm_selftest_recip(h, x, out):
+    """out = the FP64 kernels' 1 / x (float64 CUDA tensors of n)."""
+    n = int(x.numel())
+    _device_f64("x", x, n)
+    _device_f64("out", out, n)
+    return _check(load_library().ifdlbm_selftest_recip(h, n, _ptr(x), _ptr(out)), h)
 
 
 def ifdlbm_selftest_power64(h, cavity, x, out):

@@ -1774,6 +1774,18 @@ int ifdlbm_selftest_pow_pair(ifdlbm_handle h, int cavity, int n, const double *x
   return IFDLBM_OK;
 }
 
+int ifdlbm_selftest_recip(ifdlbm_handle h, int n, const double *x, double *out) {
+  if (!h || n < 0 || (n > 0 && (!x || !out)))
+    return fail(h, IFDLBM_ERR_INVALID_ARG, "selftest_recip: bad arguments");
+  if (n == 0) return IFDLBM_OK;
+  cudaSetDevice(h->device);
+  ifd::launch_recip_selftest(n, x, out, h->stream);
+  g_launches += 1;
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(h, e, "selftest_recip");
+  return IFDLBM_OK;
+}
+
 int ifdlbm_selftest_power64(ifdlbm_handle h, int cavity, int n, const double *x, double *out) {
   if (!cavity_ok(h, cavity) || n < 0 || (n > 0 && (!x || !out)))
     return fail(h, IFDLBM_ERR_INVALID_ARG, "selftest_power64: bad arguments");

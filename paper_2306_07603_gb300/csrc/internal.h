@@ -236,6 +236,7 @@ void launch_implicit_selftest(int n, const double *x, const CavDev *cav, int cav
                               double *out, cudaStream_t s);
 void launch_power64_selftest(int n, const double *x, const CavDev *cav, int cavity,
                              const double *powtab, const double *powt, double *out, cudaStream_t s);
+void launch_recip_selftest(int n, const double *x, double *out, cudaStream_t s);
 void launch_pow_f32_selftest(int n, const double *x, double m, double *out, cudaStream_t s);
 
 // Metrics of the bilinear map of a general quadrilateral at (xi, eta),

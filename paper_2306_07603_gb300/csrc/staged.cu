@@ -722,6 +722,14 @@ void launch_implicit_selftest(int n, const double *x, const CavDev *cav, int cav
   k_implicit_selftest<<<(n + 255) / 256, 256, 0, s>>>(n, x, cav, cavity, powtab, powt, powp, out);
 }
 
+__global__ void k_recip_selftest(int n, const double *x, double *out) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < n) out[k] = recip(x[k]);
+}
+void launch_recip_selftest(int n, const double *x, double *out, cudaStream_t s) {
+  k_recip_selftest<<<(n + 255) / 256, 256, 0, s>>>(n, x, out);
+}
+
 __global__ void k_power64_selftest(int n, const double *x, const CavDev *cavs, int cavity,
                                    const double *powtab, const double *powt, double *out) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
