@@ -407,11 +407,12 @@ int ifdlbm_residual_fields_static(int nx, int ny, const double *u1, const double
                                   const double *p0, double *out, void *stream);
 
 /* Autotuner of the batched fused step (pattern "batching"): times
- * `trial_steps` >= 1 steps of every combination of fused_threads {64, 128,
- * 256}, rows per task {16, 32, 64, 128, 256} and schedule {GRID,
- * STATIC, DYNAMIC} on the handle's own cavities, starting each trial from
- * the same saved state, and keeps the fastest. The state is restored
- * afterwards, so the call does not advance the simulation. Needs a handle
+ * `trial_steps` >= 1 steps with fused_threads {64, 128, 256}, each with the
+ * schedule GRID and rows per task {the automatic ones, 4, 8, 16, 24, 32, 48, 64,
+ * 128, 256} and with the schedule STATIC and rows {16, 32, 64, 128, 256}, and with
+ * the handle's layout if it is another, on the handle's own cavities, starting
+ * each trial from the same saved state, and keeps the fastest. The state is
+ * restored afterwards, so the call does not advance the simulation. Needs a handle
  * using IFDLBM_KERNEL_FUSED. Synchronises; *best receives the choice. */
 int ifdlbm_autotune(ifdlbm_handle h, int trial_steps, ifdlbm_tuning *best);
 

@@ -119,6 +119,20 @@ void *dalloc(ifdlbm_ctx *h, size_t bytes) {
   return p;
 }
 
+// Returns memory of dalloc before the handle ends; nothing on the stream may use it.
+void dfree(ifdlbm_ctx *h, void *p) {
+  for (size_t k = 0; k < h->allocs.size(); ++k)
+    if (h->allocs[k].p == p) {
+      if (h->free_fn)
+        h->free_fn(p, h->allocs[k].bytes, (void *)h->stream, h->alloc_ctx);
+      else
+        cudaFree(p);
+      h->bytes -= int64_t(h->allocs[k].bytes);
+      h->allocs.erase(h->allocs.begin() + std::ptrdiff_t(k));
+      return;
+    }
+}
+
 void release_all(ifdlbm_ctx *h) {
   for (auto e : h->ev_pool) cudaEventDestroy(e);
   h->ev_pool.clear();
@@ -429,6 +443,26 @@ int automatic_rows(const ifdlbm_ctx *h, int nt) {
   return best;
 }
 
+// Room for n tasks: their table, the order and a partial slot each. The old arrays,
+// whose contents the caller replaces, go once the stream has no more use of them.
+int reserve_tasks(ifdlbm_ctx *h, int n) {
+  if (n <= h->task_cap) return IFDLBM_OK;
+  void *t = dalloc(h, size_t(n) * sizeof(ifd::Task)), *o = dalloc(h, size_t(n) * sizeof(int)),
+       *p = dalloc(h, size_t(n) * ifd::NPART * sizeof(double));
+  if (!t || !o || !p) {
+    for (void *q : {t, o, p})
+      if (q) dfree(h, q);
+    return fail(h, IFDLBM_ERR_OOM, "fused layout: device allocation failed");
+  }
+  const cudaError_t e = cudaStreamSynchronize(h->stream);
+  for (void *q : {(void *)h->tasks, (void *)h->order, (void *)h->b.part}) dfree(h, q);
+  h->tasks = (ifd::Task *)t;
+  h->order = (int *)o;
+  h->b.part = (double *)p;
+  h->task_cap = n;
+  return e == cudaSuccess ? IFDLBM_OK : cuda_fail(h, e, "fused layout");
+}
+
 // (Re)builds the fused kernel's tasks: per cavity, balanced strips of at most
 // nt/2 - 8 columns times balanced segments of about `rows` rows (0: automatic),
 // partial slots per cavity contiguous, and the scheduling order (largest
@@ -458,8 +492,7 @@ int build_fused_tasks(ifdlbm_ctx *h, int nt, int rows, int sched) {
       }
     cv.nparts = int(tasks.size()) - cv.part0;
   }
-  if (int(tasks.size()) > h->task_cap)
-    return fail(h, IFDLBM_ERR_INVALID_ARG, "fused layout needs more tasks than allocated");
+  if (int rc = reserve_tasks(h, int(tasks.size()))) return rc;
   std::vector<int> order(tasks.size());
   for (size_t i = 0; i < order.size(); ++i) order[i] = int(i);
   auto cost = [&](int i) {
@@ -911,7 +944,7 @@ int create_impl(int ncav, const ifdlbm_cavity *cavs, const ifdlbm_quad_cavity *q
     }
     h->nblk64 = int(blk_cav.size());
   }
-  if (fused) {  // task capacity: the finest layout the autotuner tries (64 threads, 16 rows)
+  if (fused) {  // task capacity: 64 threads and 16 rows; finer layouts grow it (reserve_tasks)
     int cap = 0;
     const int rmin = opt.fused_rows ? std::min(opt.fused_rows, 16) : 16;
     const int wmin = ifd::fused_strip_width(64);  // the narrowest strips
@@ -1677,33 +1710,45 @@ int ifdlbm_autotune(ifdlbm_handle h, int trial_steps, ifdlbm_tuning *best) {
   cudaEventCreate(&e1);
   ifdlbm_tuning b{};
   b.ms_per_step = 1e300;
-  const int nts[3] = {64, 128, 256};
-  const int rows[5] = {16, 32, 64, 128, 256};
-  for (int nt : nts) {
-    for (int r : rows)
-      for (int sc = IFDLBM_SCHED_GRID; sc <= IFDLBM_SCHED_DYNAMIC; ++sc) {
-        if ((rc = build_fused_tasks(h, nt, r, sc))) goto done;
-        if ((rc = ifdlbm_load_state_dev(h, saved))) goto done;
-        for (int w = 0; w < 2; ++w) enqueue_step_any(h, h->cur ^ (w & 1), false);
-        cudaEventRecord(e0, h->stream);
-        for (int st = 0; st < trial_steps; ++st) enqueue_step_any(h, h->cur ^ (st & 1), false);
-        cudaEventRecord(e1, h->stream);
-        cudaError_t e = cudaEventSynchronize(e1);
-        if (e != cudaSuccess) {
-          rc = cuda_fail(h, e, "autotune trial");
-          goto done;
-        }
-        float ms = 0;
-        cudaEventElapsedTime(&ms, e0, e1);
-        g_launches += int64_t(trial_steps + 2) * launches_per_step(h, false);
-        ++b.candidates;
-        if (ms / trial_steps < b.ms_per_step) {
-          b.ms_per_step = ms / trial_steps;
-          b.fused_threads = nt;
-          b.fused_rows = r;
-          b.schedule = sc;
-        }
-      }
+  // GRID with the rows that the handle's own rule gives (automatic_rows), rows finer than
+  // 16, which it gives small batches, and coarse ones; STATIC, whose CTAs take several
+  // tasks each, with coarse ones; and the present layout, if it is none of these (DYNAMIC
+  // is GRID), so that what is kept is no slower than it
+  struct Trial {
+    int nt, rows, sched;
+    bool operator==(const Trial &o) const { return nt == o.nt && rows == o.rows && sched == o.sched; }
+  };
+  std::vector<Trial> trials;
+  for (int nt : {64, 128, 256}) {
+    for (int r : {automatic_rows(h, nt), 4, 8, 16, 24, 32, 48, 64, 128, 256})
+      trials.push_back({nt, r, IFDLBM_SCHED_GRID});
+    for (int r : {16, 32, 64, 128, 256}) trials.push_back({nt, r, IFDLBM_SCHED_STATIC});
+  }
+  const Trial now = {h->fused_nt, h->fused_rows ? h->fused_rows : automatic_rows(h, h->fused_nt),
+                     h->schedule == IFDLBM_SCHED_STATIC ? IFDLBM_SCHED_STATIC : IFDLBM_SCHED_GRID};
+  if (std::find(trials.begin(), trials.end(), now) == trials.end()) trials.insert(trials.begin(), now);
+  for (const Trial &t : trials) {
+    if ((rc = build_fused_tasks(h, t.nt, t.rows, t.sched))) goto done;
+    if ((rc = ifdlbm_load_state_dev(h, saved))) goto done;
+    for (int w = 0; w < 2; ++w) enqueue_step_any(h, h->cur ^ (w & 1), false);
+    cudaEventRecord(e0, h->stream);
+    for (int st = 0; st < trial_steps; ++st) enqueue_step_any(h, h->cur ^ (st & 1), false);
+    cudaEventRecord(e1, h->stream);
+    cudaError_t e = cudaEventSynchronize(e1);
+    if (e != cudaSuccess) {
+      rc = cuda_fail(h, e, "autotune trial");
+      goto done;
+    }
+    float ms = 0;
+    cudaEventElapsedTime(&ms, e0, e1);
+    g_launches += int64_t(trial_steps + 2) * launches_per_step(h, false);
+    ++b.candidates;
+    if (ms / trial_steps < b.ms_per_step) {
+      b.ms_per_step = ms / trial_steps;
+      b.fused_threads = t.nt;
+      b.fused_rows = t.rows;
+      b.schedule = t.sched;
+    }
   }
   rc = build_fused_tasks(h, b.fused_threads, b.fused_rows, b.schedule);
   if (!rc) rc = ifdlbm_load_state_dev(h, saved);
