@@ -197,6 +197,7 @@ KERNEL_SOURCES = {
     "half": ["staged64.cu", "step64.cuh", "launch.cuh", "internal.h"],
     "full": ["staged64.cu", "step64.cuh", "reduce.cuh", "launch.cuh", "internal.h"],
 }
+TRAFFIC = os.path.join(ROOT, "profiles", "traffic.json")
 
 
 def _code_only(text):
@@ -217,44 +218,32 @@ def kernel_source_digest(kernel="fused"):
     return h.hexdigest()[:16]
 
 
-def _record(d, kernel, precision, workload):
-    """The workload's own record, else (trapezoid workloads only) the kernel's."""
-    e = d.get(f"{kernel}:{precision}:{workload}")
-    if e is None and not is_general(workload):
-        e = d[f"{kernel}:{precision}"]
-    return e
-
-
 def is_general(workload):
     """Workloads of general quadrilaterals (per-node metrics)."""
     return workload is not None and workload.startswith("quad")
 
 
-def profile_record(kernel, precision, workload=None):
-    """The ncu record of this kernel (and workload) if its sources are unchanged."""
-    path = os.path.join(ROOT, "profiles", "traffic.json")
-    try:
-        with open(path) as f:
-            d = json.load(f)
-        e = _record(d, kernel, precision, workload)
-        return e if e.get("src_digest") == kernel_source_digest(kernel) else None
-    except Exception:
-        return None
+def fused_layout(info):
+    """The layout a fused handle's launches run with, as the ncu records state it."""
+    return {"fused_threads": info.fused_threads, "fused_rows": info.fused_rows,
+            "schedule": "static" if info.schedule == 1 else "grid"}    # (dynamic is grid)
 
 
-def traffic_per_launch(kernel, precision, lu_per_launch, workload=None):
-    """DRAM bytes per launch from the ncu record of this kernel (and workload,
-    where one was captured: an L2-resident workload moves fewer bytes)."""
-    path = os.path.join(ROOT, "profiles", "traffic.json")
+def profile_record(kernel, precision, workload, layout=None, path=TRAFFIC):
+    """The ncu record of this kernel on this workload, if it describes the timed launches:
+    captured from the present sources, on a step that formed the residual (every timed one
+    does; steps that do not run other kernels or less of them) and, for the fused kernel, with
+    the same layout. Else None: no bound is reported from another launch's counters."""
     try:
         with open(path) as f:
-            d = json.load(f)
-        e = _record(d, kernel, precision, workload)
-        if e.get("src_digest") != kernel_source_digest(kernel):
-            return None
-        return float(e["bytes_per_lu"]) * lu_per_launch
-    except Exception:
+            e = json.load(f)[f"{kernel}:{precision}:{workload}"]
+    except (OSError, KeyError, ValueError):
         return None
+    if e.get("src_digest") != kernel_source_digest(kernel) or e.get("residual") is not True:
+        return None
+    if kernel == "fused" and e.get("layout") != layout:
+        return None
+    return e
 
 
 # ---------------------------------------------------------------------------
@@ -522,6 +511,9 @@ def run_ours(args):
     # roofline of the dominant kernel, from its live event times
     peak, peak_src = load_peaks()
     dom = max(kern, key=lambda k: kern[k][0]) if kern else None
+    # the ncu record of that kernel, of the lagged relaxation time with the FP64 power
+    rec = (profile_record(dom, args.precision, args.workload, fused_layout(capi.ifdlbm_info(s.h, 0)))
+           if dom is not None and args.lambda_mode == "lagged" and not args.power_fp32 else None)
     roofline = None
     if dom is not None and (dom, args.precision) in ALGO_BYTES:
         ms, n = kern[dom]
@@ -531,8 +523,7 @@ def run_ours(args):
         achieved = algo / per_launch_s / 1e9
         roofline = {"bound": "hbm", "kernel": DEVICE_KERNEL[dom], "achieved": round(achieved, 1),
                     "peak": peak, "unit": "GB/s", "frac": round(achieved / peak, 4),
-                    "traffic": traffic_per_launch(dom, args.precision, lu_step, args.workload)
-                    if args.lambda_mode == "lagged" and not args.power_fp32 else None,
+                    "traffic": rec["bytes_per_lu"] * lu_step if rec is not None else None,
                     "algorithmic_bytes": algo, "peak_source": f"{peak_src} (MEASURED_PEAKS.json hbm_gbs)"
                     if peak_src == "measured" else "fallback",
                     "time_share": round(ms / sum(v[0] for v in kern.values()), 4)}
@@ -540,9 +531,6 @@ def run_ours(args):
     # what bounds the step before HBM does, from the ncu record of the same
     # kernel sources: the FP64 pipe (1/64 of the FP32 rate on GB300; the FP64
     # form) and the schedulers' instruction issue (the FP32-deviation form)
-    # (the ncu records are of the lagged kernels)
-    rec = (profile_record(dom, args.precision, args.workload)
-           if dom is not None and args.lambda_mode == "lagged" and not args.power_fp32 else None)
     fp64 = issue = None
     if rec is not None and "fp64_pipe_pct_elapsed" in rec:
         fp64 = {"bound": "alu", "unit": "fraction of the FP64 pipe's peak issue rate",
