@@ -246,6 +246,16 @@ def profile_record(kernel, precision, workload, layout=None, path=TRAFFIC):
     return e
 
 
+def power_law(args):
+    """How Eq. (1.4) is evaluated, for the bench line."""
+    if args.power_fp32:
+        return "fp32 (opt-in)"
+    if args.precision == "fp64":
+        return "fp64"
+    return ("fp64, rounded to the fp32 relaxation-time plane; the fused kernel finds that float in "
+            "float pairs and evaluates fp64 where they leave it in doubt")
+
+
 # ---------------------------------------------------------------------------
 # Oracle CPU baseline (the only use of oracle/ in this file)
 # ---------------------------------------------------------------------------
@@ -583,7 +593,7 @@ def run_ours(args):
                        "grids": sorted({f"{sp.nx}x{sp.ny}" for sp in specs}),
                        "lattice_updates_per_step": lu_step, "precision": args.precision,
                        "kernel": args.kernel, "lambda_mode": args.lambda_mode,
-                       "power_law": "fp32 (opt-in)" if args.power_fp32 else "fp64",
+                       "power_law": power_law(args),
                        "parallelism": f"replicas x{world}" if world > 1 else "1 GPU",
                        "l2": "256 MiB buffer written between timed steps (outside the events)",
                        "metric_definition": HEADLINE_METRIC},

@@ -29,3 +29,11 @@ def test_a_record_describes_the_timed_launch_or_is_not_used(tmp_path, change, fo
     assert (got is not None) == found
     # nor does one workload's record describe another's launches
     assert bench.profile_record("fused", "fp32dev", "sweep257", LAYOUT, path=str(path)) is None
+
+
+def test_the_bench_line_states_how_the_power_law_is_evaluated():
+    """The FP32 form does not evaluate every power in FP64, and the line says what it does."""
+    said = {p: bench.power_law(bench.parse_args(a)) for p, a in
+            {"default": [], "fp64": ["--precision", "fp64"], "opt-in": ["--power-fp32"]}.items()}
+    assert said["fp64"] == "fp64" and said["opt-in"].startswith("fp32")
+    assert "float pairs" in said["default"] and "rounded" in said["default"]
