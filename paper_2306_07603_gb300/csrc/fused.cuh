@@ -44,6 +44,7 @@
 #include <cstdint>
 
 #include "d2q9.cuh"
+#include "device_once.h"
 #include "implicit.cuh"
 #include "internal.h"
 #include "launch.cuh"
@@ -809,19 +810,21 @@ __global__ void __launch_bounds__(NT, Occ<T, NT>::blocks) k_fused(FusedArgs a) {
 }
 
 template <class T, int NT, bool IMPL, bool GEN, bool P32, bool PERSIST, bool RES>
-static void configure_nt() {
-  static bool configured = false;  // the attribute is per function
-  if (!configured) {
-    cudaFuncSetAttribute(k_fused<T, NT, IMPL, GEN, P32, PERSIST, RES>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, fused_smem_size<T, NT>());
-    configured = true;
-  }
+static bool configure_nt() {
+  static DeviceOnce once;  // the attribute is the function's on one device
+  int device = 0;
+  if (cudaGetDevice(&device) != cudaSuccess) return false;
+  return once(device, [] {
+    return cudaFuncSetAttribute(k_fused<T, NT, IMPL, GEN, P32, PERSIST, RES>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                fused_smem_size<T, NT>()) == cudaSuccess;
+  });
 }
 
 template <class T, int NT, bool IMPL, bool GEN, bool P32, bool PERSIST, bool RES>
 static void launch_kernel(const FusedArgs &a, int grid, cudaStream_t s) {
   constexpr int smem = fused_smem_size<T, NT>();
-  configure_nt<T, NT, IMPL, GEN, P32, PERSIST, RES>();
+  if (!configure_nt<T, NT, IMPL, GEN, P32, PERSIST, RES>()) return;  // (the caller sees CUDA's error)
   if (!PERSIST && a.early)
     launch_after(k_fused<T, NT, IMPL, GEN, P32, PERSIST, RES>, grid, NT, smem, s, a);
   else
@@ -866,8 +869,8 @@ static void launch_fused_nt(const FusedArgs &a, int grid, cudaStream_t s) {
 
 template <class T, int NT>
 static int blocks_per_sm_nt() {
-  configure_nt<T, NT, false, false, false, true, true>();
   int n = 0;
+  if (!configure_nt<T, NT, false, false, false, true, true>()) return 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused<T, NT, false, false, false, true, true>, NT,
                                                 fused_smem_size<T, NT>());
   return n;
