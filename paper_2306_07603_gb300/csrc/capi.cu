@@ -64,6 +64,7 @@ struct ifdlbm_ctx {
   // adjoint scratch (allocated on the first adjoint call)
   double *adj_g1 = nullptr, *adj_l1 = nullptr, *adj_fbarb = nullptr, *adj_lamb2 = nullptr,
          *adj_ppart = nullptr, *adj_pfull = nullptr, *adj_phalf = nullptr, *adj_tab = nullptr;
+  bool adj_set = false;      // its tables and zeros have been enqueued (adjoint_ready)
   int *adj_nodes = nullptr;  // [ncav][2] nodes of the psi objective
   int *adj_blocks = nullptr;  // block -> cavity of the kernels over the interior and its ring
   int nblk_adj = 0, nblk_ring = 0;
@@ -1508,37 +1509,44 @@ int adjoint_ready(ifdlbm_ctx *h) {
     return fail(h, IFDLBM_ERR_INVALID_ARG, "adjoint: differentiates the trapezoid map of Eq. (3.8.1)");
   if (h->opt.wall_pressure != IFDLBM_WALLP_ZEROTH)
     return fail(h, IFDLBM_ERR_INVALID_ARG, "adjoint: differentiates the zeroth-order wall pressure");
-  if (h->adj_g1) return IFDLBM_OK;
+  if (h->adj_set) return IFDLBM_OK;
   const size_t P = size_t(h->total_plane) * sizeof(double), GL = size_t(h->geo_len);
-  bool ok = true;
-  double *g1 = nullptr;
-  ok &= (g1 = (double *)dalloc(h, 9 * P)) != nullptr;
-  ok &= (h->adj_l1 = (double *)dalloc(h, P)) != nullptr;
-  ok &= (h->adj_fbarb = (double *)dalloc(h, 9 * P)) != nullptr;
-  ok &= (h->adj_lamb2 = (double *)dalloc(h, P)) != nullptr;
-  ok &= (h->adj_ppart = (double *)dalloc(h, size_t(h->ntiles) * 3 * sizeof(double))) != nullptr;
-  ok &= (h->adj_pfull = (double *)dalloc(h, size_t(h->nblk_adj) * sizeof(double))) != nullptr;
-  ok &= (h->adj_phalf = (double *)dalloc(h, size_t(h->nblk64) * 3 * sizeof(double))) != nullptr;
-  ok &= (h->adj_nodes = (int *)dalloc(h, size_t(h->ncav) * 2 * sizeof(int))) != nullptr;
-  ok &= (h->adj_blocks = (int *)dalloc(h, size_t(h->nblk_adj + h->nblk_ring) * sizeof(int))) !=
-        nullptr;
-  ok &= (h->adj_tab = (double *)dalloc(h, 5 * GL * sizeof(double))) != nullptr;
-  if (!ok) return fail(h, IFDLBM_ERR_OOM, "adjoint: device allocation failed");
-  h->b.geo.xm = h->adj_tab;
-  h->b.geo.xp = h->adj_tab + GL;
-  h->b.geo.z = h->adj_tab + 2 * GL;
-  h->b.geo.ath1 = h->adj_tab + 3 * GL;
-  h->b.geo.ath2 = h->adj_tab + 4 * GL;
+  if (!h->adj_g1) {
+    bool ok = true;
+    double *g1 = nullptr;
+    ok &= (g1 = (double *)dalloc(h, 9 * P)) != nullptr;
+    ok &= (h->adj_l1 = (double *)dalloc(h, P)) != nullptr;
+    ok &= (h->adj_fbarb = (double *)dalloc(h, 9 * P)) != nullptr;
+    ok &= (h->adj_lamb2 = (double *)dalloc(h, P)) != nullptr;
+    ok &= (h->adj_ppart = (double *)dalloc(h, size_t(h->ntiles) * 3 * sizeof(double))) != nullptr;
+    ok &= (h->adj_pfull = (double *)dalloc(h, size_t(h->nblk_adj) * sizeof(double))) != nullptr;
+    ok &= (h->adj_phalf = (double *)dalloc(h, size_t(h->nblk64) * 3 * sizeof(double))) != nullptr;
+    ok &= (h->adj_nodes = (int *)dalloc(h, size_t(h->ncav) * 2 * sizeof(int))) != nullptr;
+    ok &= (h->adj_blocks = (int *)dalloc(h, size_t(h->nblk_adj + h->nblk_ring) * sizeof(int))) !=
+          nullptr;
+    ok &= (h->adj_tab = (double *)dalloc(h, 5 * GL * sizeof(double))) != nullptr;
+    if (!ok) return fail(h, IFDLBM_ERR_OOM, "adjoint: device allocation failed");
+    h->b.geo.xm = h->adj_tab;
+    h->b.geo.xp = h->adj_tab + GL;
+    h->b.geo.z = h->adj_tab + 2 * GL;
+    h->b.geo.ath1 = h->adj_tab + 3 * GL;
+    h->b.geo.ath2 = h->adj_tab + 4 * GL;
+    h->adj_g1 = g1;
+  }
+  // A call that is being captured only records this: it is there for the graph's
+  // replays, and the next call enqueues it again.
   ifd::launch_adjoint_setup(h->b.cav, h->b.geo, h->adj_blocks, h->adj_blocks + h->nblk_adj,
                             h->ncav, h->stream);
   g_launches += 1;
   cudaError_t e = cudaGetLastError();
-  for (double *p : {g1, h->adj_fbarb})
+  for (double *p : {h->adj_g1, h->adj_fbarb})
     if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, 9 * P, h->stream);
   for (double *p : {h->adj_l1, h->adj_lamb2})
     if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, P, h->stream);
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (e == cudaSuccess) e = cudaStreamIsCapturing(h->stream, &capturing);
   if (e != cudaSuccess) return cuda_fail(h, e, "adjoint set-up");
-  h->adj_g1 = g1;
+  h->adj_set = capturing == cudaStreamCaptureStatusNone;
   return IFDLBM_OK;
 }
 
