@@ -1512,26 +1512,34 @@ int adjoint_ready(ifdlbm_ctx *h) {
   if (h->adj_set) return IFDLBM_OK;
   const size_t P = size_t(h->total_plane) * sizeof(double), GL = size_t(h->geo_len);
   if (!h->adj_g1) {
+    const size_t D = sizeof(double), I = sizeof(int);
+    const struct {
+      void **at;
+      size_t bytes;
+    } want[] = {{(void **)&h->adj_g1, 9 * P},
+                {(void **)&h->adj_l1, P},
+                {(void **)&h->adj_fbarb, 9 * P},
+                {(void **)&h->adj_lamb2, P},
+                {(void **)&h->adj_ppart, size_t(h->ntiles) * 3 * D},
+                {(void **)&h->adj_pfull, size_t(h->nblk_adj) * D},
+                {(void **)&h->adj_phalf, size_t(h->nblk64) * 3 * D},
+                {(void **)&h->adj_nodes, size_t(h->ncav) * 2 * I},
+                {(void **)&h->adj_blocks, size_t(h->nblk_adj + h->nblk_ring) * I},
+                {(void **)&h->adj_tab, 5 * GL * D}};
     bool ok = true;
-    double *g1 = nullptr;
-    ok &= (g1 = (double *)dalloc(h, 9 * P)) != nullptr;
-    ok &= (h->adj_l1 = (double *)dalloc(h, P)) != nullptr;
-    ok &= (h->adj_fbarb = (double *)dalloc(h, 9 * P)) != nullptr;
-    ok &= (h->adj_lamb2 = (double *)dalloc(h, P)) != nullptr;
-    ok &= (h->adj_ppart = (double *)dalloc(h, size_t(h->ntiles) * 3 * sizeof(double))) != nullptr;
-    ok &= (h->adj_pfull = (double *)dalloc(h, size_t(h->nblk_adj) * sizeof(double))) != nullptr;
-    ok &= (h->adj_phalf = (double *)dalloc(h, size_t(h->nblk64) * 3 * sizeof(double))) != nullptr;
-    ok &= (h->adj_nodes = (int *)dalloc(h, size_t(h->ncav) * 2 * sizeof(int))) != nullptr;
-    ok &= (h->adj_blocks = (int *)dalloc(h, size_t(h->nblk_adj + h->nblk_ring) * sizeof(int))) !=
-          nullptr;
-    ok &= (h->adj_tab = (double *)dalloc(h, 5 * GL * sizeof(double))) != nullptr;
-    if (!ok) return fail(h, IFDLBM_ERR_OOM, "adjoint: device allocation failed");
+    for (const auto &w : want) ok = ok && (*w.at = dalloc(h, w.bytes)) != nullptr;
+    if (!ok) {  // all or none: another call starts over
+      for (const auto &w : want) {
+        if (*w.at) dfree(h, *w.at);
+        *w.at = nullptr;
+      }
+      return fail(h, IFDLBM_ERR_OOM, "adjoint: device allocation failed");
+    }
     h->b.geo.xm = h->adj_tab;
     h->b.geo.xp = h->adj_tab + GL;
     h->b.geo.z = h->adj_tab + 2 * GL;
     h->b.geo.ath1 = h->adj_tab + 3 * GL;
     h->b.geo.ath2 = h->adj_tab + 4 * GL;
-    h->adj_g1 = g1;
   }
   // A call that is being captured only records this: it is there for the graph's
   // replays, and the next call enqueues it again.
