@@ -65,3 +65,28 @@ def test_saved_state_comes_back(nx, ny, kernels):
     got = s.get_state(0)[0]
     s.close()
     assert torch.equal(first, again) and (got == want).all()
+
+
+@pytest.mark.gpu
+def test_copies_can_be_captured():
+    """Looking the buffer's device up is no stream operation: a capture records the copies."""
+    import torch
+
+    from paper_2306_07603_gb300 import capi
+    from paper_2306_07603_gb300.solver import Solver, cavity
+    s = Solver([cavity(65, 47, 400.0, 0.75)])
+    a, b = (torch.zeros(capi.ifdlbm_state_bytes(s.h) // 8, dtype=torch.float64, device="cuda")
+            for _ in range(2))
+    s.step(2)
+    capi.ifdlbm_save_state_dev(s.h, a)
+    s.sync()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s.stream):
+        capi.ifdlbm_load_state_dev(s.h, a)
+        capi.ifdlbm_save_state_dev(s.h, b)
+    assert not torch.equal(a, b)
+    with torch.cuda.stream(s.stream):
+        graph.replay()
+    s.sync()
+    s.close()
+    assert torch.equal(a, b)
