@@ -376,9 +376,9 @@ int ifdlbm_profile_read(ifdlbm_handle h, int kernel, double *total_ms, int64_t *
  * (a multi-tenant service, a real-time loop), where an allocation would
  * synchronise the device, fragment the pool or fail at the worst moment.
  * This entry point allocates nothing, directly or through any library
- * (PyTorch's allocator included). Its scratch, one partial sum per 256
- * nodes, is a fixed 512 KiB array in device memory that every GPU which
- * loads libifdlbm.so holds until the process exits.
+ * (PyTorch's allocator included). Its scratch, one partial sum per
+ * block of the kernel, is a fixed 38 KiB array in device memory that every GPU
+ * which loads libifdlbm.so holds until the process exits.
  *
  *  nx, ny   field size; nx * ny <= IFDLBM_STATIC_MAX_NODES, larger fields
  *           are rejected with IFDLBM_ERR_INVALID_ARG and a message
@@ -393,7 +393,7 @@ int ifdlbm_profile_read(ifdlbm_handle h, int kernel, double *total_ms, int64_t *
  * device is its set-up: it looks up the scratch array's device address
  * (cudaGetSymbolAddress) and loads the entry point's two kernels. Under lazy
  * module loading (the CUDA default) that is when the driver sets up this
- * module on the device, the 512 KiB array included, so the first call may
+ * module on the device, the 38 KiB array included, so the first call may
  * take device memory and can fail when none is left. Make that first call at
  * set-up time, before any stream capture and before the memory budget is
  * spent; later calls take nothing. Every

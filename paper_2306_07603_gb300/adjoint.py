@@ -58,7 +58,6 @@ def _forward(params, nx, ny, T, every, U_lid, L, H, eta_b):
     final = _state_buffer(s.h, s.stream)
     capi.ifdlbm_save_state_dev(s.h, final)
     return s, ckpt, final, inter
-    return s, ckpt, final
 
 
 def _backward(ctx, seed, gJ):

@@ -317,8 +317,6 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
   const int nx = cv.nx, ny = cv.ny, pitch = cv.pitch;
   const int64_t plane = cv.plane, goff = cv.goff;
   const double cvc = cv.c, cvH = cv.H;
-  const T Uw = GEN ? T(cv.lid_ux / cvc) : T(cv.U / cvc);  // lid velocity / c
-  const T Uwy = GEN ? T(cv.lid_uy / cvc) : T(0);
   [[maybe_unused]] const int part0 = cv.part0, nparts = cv.nparts;
   // c xi_x of row j and the Jacobian x_xi H: FP64 metrics for FP64
   // arithmetic, their rounded float copies for FP32 arithmetic.
@@ -378,8 +376,8 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
   constexpr bool FASTQ = !GEN;
 
   // The sums of the residual are kept per warp in shared memory (five FP64 values a
-  // thread would take 10 registers through the march: 64 cavities 504 us a step with
-  // the residual formed in every one, 500 so).
+  // thread would take 10 registers through the march: 64 cavities 511 us a step with
+  // the residual formed in every one, 504 so).
   __shared__ double racc[RES ? NT / 32 : 1][7];
   Leaf<T> leaf;
   if (RES && a.want_residual && (threadIdx.x & 31) < 7) racc[threadIdx.x >> 5][threadIdx.x & 31] = 0.0;

@@ -134,8 +134,8 @@ struct StepArgs {
   int want_residual;
 };
 
-// One CTA task of the fused kernel: owned columns [i0, i1) (at most NT - 8)
-// and rows [j0, j1) of cavity `cav`.
+// One CTA task of the fused kernel: owned columns [i0, i1) (at most NT / 2 - 8) and
+// rows [j0, j1) of cavity `cav`.
 struct Task {
   int cav, i0, i1, j0, j1, pad0, pad1, pad2;
 };

@@ -17,17 +17,16 @@
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kMaxBlocks = IFDLBM_STATIC_MAX_NODES / kThreads;  // 8192 partial slots
 constexpr int kMaxDevices = 64;
 // Blocks of k_field_partials: 4 on each of the 152 SMs, each thread taking every
 // 608 x 256th node. A block's reduction then costs the FP64 pipe once per some
 // nodes instead of once per node, and the second kernel has 608 slots at most
 // (1025^2: 89 + 24 -> 40 + 10 us, from a cold cache).
 constexpr int kBlocks = 608;
-static_assert(kBlocks <= kMaxBlocks, "partial slots");
 
-// 8192 slots x 8 doubles = 512 KiB per device.
-static __device__ __align__(256) double g_static_partials[kMaxBlocks * ifd::NPART];
+// 608 slots x 8 doubles = 38 KiB per device. (The limit on the nodes is from a
+// form with a slot per 256 of them; it stays what callers can rely on.)
+static __device__ __align__(256) double g_static_partials[kBlocks * ifd::NPART];
 
 std::mutex g_mu;
 double *g_addr[kMaxDevices] = {nullptr};
