@@ -142,9 +142,12 @@ typedef struct {
 #define IFDLBM_SCHED_GRID 0    /* one CTA per task: the hardware hands the next one
                                   to whichever SM is free first */
 #define IFDLBM_SCHED_STATIC 1  /* persistent CTAs (SMs x resident CTAs); CTA b takes
-                                  the positions b, b + grid, ... */
+                                  the positions b, b + grid, ... Its kernel can
+                                  always form the residual, where GRID's steps
+                                  before the last of a call run a smaller one */
 #define IFDLBM_SCHED_DYNAMIC 2 /* the same as GRID, whose CTAs the hardware
-                                  schedules dynamically */
+                                  schedules dynamically (the autotuner never
+                                  picks this name) */
 
 /* Result of ifdlbm_autotune. */
 typedef struct {

@@ -123,8 +123,9 @@ __device__ __forceinline__ double pow_tab(float x, const double *__restrict__ ta
 // "Fast evaluation of elementary mathematical functions with correctly rounded
 // last bit", ACM TOMS 17, 1991): that float is the one pow_tab's FP64 value rounds
 // to, and where it is in doubt (one argument in 2^13) pow_tab decides. So the
-// plane holds the rounded FP64 power law, bit for bit, at the cost of 5
-// instructions for the test.
+// plane holds the rounded FP64 power law, bit for bit. The test takes 5
+// instructions: 64 cavities 422.0 -> 426.5 us a step, 2049^2 221.0 -> 223.8, one 65^2
+// 9.06 -> 9.20; pow_tab in the place of the pair took 4 to 6 % (before the other steps).
 // Table (POWP_SIZE floats): [4j ..] = c_j^m hi, lo, 1/c_j hi, lo; [1024 + 2e ..] =
 // C 2^(m (e - 127)) hi, lo. Entries e outside [pe_lo, pe_lo + pe_n) are not in
 // [2^-60, 2^60] (their low parts or products could underflow), and for |m| > 1 none

@@ -370,9 +370,9 @@ __device__ __forceinline__ void fused_task(const FusedArgs &a, FusedSmem<T, NT> 
   // The FP32 trapezoid stencils take their near-wall form from ghost values
   // (write_ghosts) instead of per-plane selects on the wall flags.
   constexpr bool GHOST = sizeof(T) == 4;
-  // approximate FP32 quotients (quot); the general-quadrilateral variant, whose
-  // registers are at the cap, keeps the division (the approximation's extra
-  // live values spill there)
+  // approximate FP32 quotients (quot); the general-quadrilateral variant keeps the
+  // division: with the residual's registers it is at the cap, and the
+  // approximation's extra live values spilled there (without them not measured)
   constexpr bool FASTQ = !GEN;
 
   // The sums of the residual are kept per warp in shared memory (five FP64 values a
@@ -780,7 +780,8 @@ struct Occ {
 // RES: whether the residual can be asked for. Its moments, its sums and the
 // registers they take are then out of the steps before the last of a call: 64
 // cavities 502 -> 422 us a step (with the task order above), 2049^2 252 -> 220, ten
-// 257^2 62 -> 56, ten quadrilaterals 76 -> 70.
+// 257^2 62 -> 56, ten quadrilaterals 76 -> 70 (426, 224, 53 and 68 now). The persistent
+// form exists with RES only, so that it does not gain from this.
 template <class T, int NT, bool IMPL, bool GEN, bool P32, bool PERSIST, bool RES>
 __global__ void __launch_bounds__(NT, Occ<T, NT>::blocks) k_fused(FusedArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -107,7 +107,8 @@ __device__ __forceinline__ ImplPair impl_pair(const CavDev &cv) {
 // only where lam - d - E and lam - d + E round to it (pow_pair's rounding test; E is a
 // few 1e-12 lam, so that one root in 10^4 is in doubt); else, and where the table does
 // not cover q, the step is large, D is near zero (n < 0.02) or a low part could
-// underflow, the FP64 solve decides.
+// underflow, the FP64 solve decides. (Six 300x260 cavities, without this test 56.4 us
+// a step, with it 58.9.)
 __device__ __forceinline__ float lambda_implicit_pair(float G2, float lam_start, const ImplPair &s,
                                                       const PowPair &pw, const CavDev &cv,
                                                       const double *powtab, const double *powt) {

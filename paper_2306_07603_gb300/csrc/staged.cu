@@ -424,9 +424,10 @@ struct MacrosArgs {
 // the rows in MSEG segments. Pass 1: rho, u, v and I at every node (I parked in
 // psi), and the segment's sum of I. The sums of the segments below, in the block
 // and in the cluster's blocks before it, give each segment its offset, and pass
-// 2 writes psi. Bound by the FP64 pipe (8 instructions a node) and the bytes
-// about alike; one block per 32 lines left 119 of the 152 SMs
-// idle (1025^2: 157 us, now 71, both from a cold cache).
+// 2 writes psi. One block per 32 lines left 119 of the 152 SMs idle (1025^2: 157
+// us, now 71, both from a cold cache). Bound now by latency: the FP64 pipe (11
+// instructions a node) has 19 us of work in it and the bytes take 13, but 264
+// blocks at one per SM are 1.7 rounds, each thread taking its rows one by one.
 constexpr int MSEG = 32;
 constexpr int MACROS_CS = 8;
 

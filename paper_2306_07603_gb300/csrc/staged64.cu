@@ -7,13 +7,15 @@
 //   k_full64     Step (5): f-hat(t+dt) (Eq. 3.6); wall nodes (Step 6); residual
 //                partials of Eq. (2.19) and Eq. (5.1)
 //
-// Bound: the FP64 pipe (step64.cuh), 85-89 % busy. A node's step takes 102 + 133
-// + 70 FP64 instructions in the three kernels, which is why the intermediate
-// planes are kept (they stay in L2 for a cavity sweep) rather than recomputed.
-// Ten 257^2 cavities, us per step: 394 = 134 + 166 + 92. The form before, tiles
-// of 32 x 8 nodes with both upwind sides evaluated, the power by log2 and exp2
-// and the wall rule in every edge warp, took 218 + 356 + 259 instructions and
-// 1211 us. One 65^2 cavity: 21.6 us a step against 94; there the three launches
+// Bound: the FP64 pipe (step64.cuh), busy 81-85 % of the kernels' time. A node's
+// step takes 102 + 139 + 76 FP64 instructions in the three kernels (105 + 139 + 128
+// where the residual is formed), which is why the intermediate planes are kept
+// (they stay in L2 for a cavity sweep) rather than recomputed. Ten 257^2 cavities:
+// 391 us a step, 333 at the pipe's rate (133 + 173 + 95 from a cold cache, one
+// launch after another). The form before, tiles of 32 x 8 nodes with both upwind
+// sides evaluated, the power by log2 and exp2 and the wall rule in every edge
+// warp, took 218 + 356 + 259 instructions and
+// 1211 us. One 65^2 cavity: 20.3 us a step against 94; there the three launches
 // and the latency of a warp count, so each kernel starts while the one before
 // it ends (launch.cuh) and forms what the step does not change before waiting
 // for it, and blocks are one warp (34.1 us before these three).
