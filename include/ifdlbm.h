@@ -132,8 +132,10 @@ typedef struct {
  * / c_s^2 at every node, gamma-dot(lambda) = a / (2 lambda + dt) with a from
  * sum_i c_i c_i (f-hat_i - f^eq_i) (Eq. 2.18 at the same lambda), by a
  * bracketed Newton iteration in FP64 (the root is unique: the residual
- * increases strictly with lambda; in FP32 with the power_fp32 opt-in). Both
- * forms share steady states. The adjoint needs the lagged form. */
+ * increases strictly with lambda; in FP32 with the power_fp32 opt-in). FP32DEV
+ * rounds it to its FP32 plane (the fused kernel finds the same float from an
+ * FP32 root where one Newton step in pairs of floats settles it). Both forms
+ * share steady states. The adjoint needs the lagged form. */
 #define IFDLBM_LAMBDA_LAGGED 0   /* default */
 #define IFDLBM_LAMBDA_IMPLICIT 1
 

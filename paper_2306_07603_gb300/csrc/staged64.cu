@@ -14,11 +14,11 @@
 // 391 us a step, 333 at the pipe's rate (133 + 173 + 95 from a cold cache, one
 // launch after another). The form before, tiles of 32 x 8 nodes with both upwind
 // sides evaluated, the power by log2 and exp2 and the wall rule in every edge
-// warp, took 218 + 356 + 259 instructions and
-// 1211 us. One 65^2 cavity: 20.3 us a step against 94; there the three launches
-// and the latency of a warp count, so each kernel starts while the one before
-// it ends (launch.cuh) and forms what the step does not change before waiting
-// for it, and blocks are one warp (34.1 us before these three).
+// warp, took 218 + 356 + 259 instructions and 1211 us. One 65^2 cavity: 20.3 us a
+// step against 94; there the three launches and the latency of a warp count, so
+// each kernel starts while the one before it ends (launch.cuh) and forms what the
+// step does not change before waiting for it, and blocks are one warp (34.1 us
+// before these three).
 //
 // Wall nodes follow the rule of the FP32 staged kernels (staged.cu): a wall
 // node (i, j) takes the node (clamp(i, 1, nx-2), clamp(j, 1, ny-2)), which its
