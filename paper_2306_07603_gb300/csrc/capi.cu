@@ -1718,7 +1718,10 @@ int ifdlbm_autotune(ifdlbm_handle h, int trial_steps, ifdlbm_tuning *best) {
   void *saved = dalloc(h, size_t(nbytes));
   if (!saved) return fail(h, IFDLBM_ERR_OOM, "autotune: device allocation failed");
   int rc = ifdlbm_save_state_dev(h, saved);
-  if (rc) return rc;
+  if (rc) {
+    dfree(h, saved);
+    return rc;
+  }
   const bool profiling = h->profiling;
   h->profiling = false;
   cudaEvent_t e0, e1;
@@ -1740,6 +1743,7 @@ int ifdlbm_autotune(ifdlbm_handle h, int trial_steps, ifdlbm_tuning *best) {
       trials.push_back({nt, r, IFDLBM_SCHED_GRID});
     for (int r : {16, 32, 64, 128, 256}) trials.push_back({nt, r, IFDLBM_SCHED_STATIC});
   }
+  const int given = h->fused_rows, sched = h->schedule;
   const Trial now = {h->fused_nt, h->fused_rows ? h->fused_rows : automatic_rows(h, h->fused_nt),
                      h->schedule == IFDLBM_SCHED_STATIC ? IFDLBM_SCHED_STATIC : IFDLBM_SCHED_GRID};
   if (std::find(trials.begin(), trials.end(), now) == trials.end()) trials.insert(trials.begin(), now);
@@ -1772,6 +1776,13 @@ int ifdlbm_autotune(ifdlbm_handle h, int trial_steps, ifdlbm_tuning *best) {
   b.ntasks = h->ntasks;
   *best = b;
 done:
+  if (rc) {  // (the error's text is the trial's): the layout and the state it began with
+    const std::string text = h->err;
+    if (build_fused_tasks(h, now.nt, given, sched) == IFDLBM_OK) ifdlbm_load_state_dev(h, saved);
+    h->err = text;
+  }
+  cudaStreamSynchronize(h->stream);
+  dfree(h, saved);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   h->profiling = profiling;
