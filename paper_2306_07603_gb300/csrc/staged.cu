@@ -826,7 +826,9 @@ cudaError_t launch_copy(const CopyArgs &a, const void *mine, int device, cudaStr
   cudaPointerAttributes at = {};
   const bool here = cudaPointerGetAttributes(&at, mine) == cudaSuccess &&
                     at.type == cudaMemoryTypeDevice && at.device == device;
-  (void)cudaGetLastError();  // an address CUDA does not know: the copies below say so
+  // (an address CUDA does not know: the copies below say so; and an error left by
+  // earlier, unrelated work is not this call's)
+  (void)cudaGetLastError();
   if (copy_by_kernel(a, here)) {
     const int64_t blocks = ((a.bytes[0] + a.bytes[1] + a.bytes[2]) / 16 + 255) / 256;
     launch_after(k_copy, int(std::max<int64_t>(1, std::min<int64_t>(blocks, 152 * 8))), 256, 0, s,

@@ -2,10 +2,10 @@
 
 The pairs of floats it is found in are within 2^-40 of the value; where the exact
 value lies that close to the middle between two floats they may point to the wrong
-one. Arguments: 2^20 random ones, of which those nearest to a middle (about one in
-2^13 within 2^-36 of the value; NumPy's extended precision) are where a plain
-rounding of the pair fails, and both ends of the exponents. n from 0.1 to 3, and
-beyond, where FP64 has to take over. No tolerance: the two floats are equal.
+one. Arguments: of 2^24 random ones those within 2^-36 of a middle (by a power good to
+2^-52; about one in 2^12), where a plain rounding of the pair fails now and then,
+2^18 of the others, and both ends of the exponents. n from 0.1 to 3, and beyond, where
+FP64 has to take over. No tolerance: the two floats are equal.
 """
 import numpy as np
 import pytest
